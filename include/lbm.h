@@ -209,14 +209,18 @@ int lbm_set_solid(lbm_handle* h, const unsigned char* mask, double mu_w);
  * handle parameters, initial state and n give the same bits on every run:
  * where several thread blocks contribute to one node's next density, their
  * partial sums are combined in an order-independent way (two floating-point
- * additions onto zero, or exact 64-bit fixed-point additions). */
+ * additions onto zero, or exact 64-bit fixed-point additions).  Calls of n >= 2
+ * steps with tau = 1 may carry only the moments from step to step and form the
+ * populations of the last one (FP32DEV explicit schemes): n single steps then
+ * agree with them within FP32 rounding. */
 int lbm_step(lbm_handle* h, long long n);
 
 /* As lbm_step (n <= 100000), timing every step on the handle's stream with
  * CUDA events recorded between the launches; synchronises once at the end.
  * ms[3] receives the summed
  * milliseconds of the mu pass (0 when the step is a single fused kernel), of
- * the collision/streaming pass (the whole step when fused), and of both. */
+ * the collision/streaming pass (the whole step when fused; whatever else the
+ * call runs included), and of both. */
 int lbm_step_timed(lbm_handle* h, long long n, double* ms);
 
 /* Observables of the current state (synchronises the stream).  Returns

@@ -22,6 +22,7 @@ struct Launch {
   void* mu;     // N floats: mu field of the split D3Q19 FP32DEV path (else unused)
   Mrt mrt;      // D2Q9 collision operator (on = 0: single relaxation)
   cudaEvent_t ev_mid;  // if set: recorded between the mu pass and the collision pass
+  cudaEvent_t* ev_mu;  // mom3d_steps, if set: recorded before and after each step's mu pass (2 n events)
   const void* tmap;    // D3Q19 FP32DEV: tensor map (CUtensorMap) of the populations fin, or null
   int rpt2d;           // D2Q9 FP32DEV split tiles: rows per thread (1, 2, 4; 0 = default 2)
   // D3Q19 FP32DEV collision pass: corner accumulators (coll3d_corner_count
@@ -49,6 +50,13 @@ int fast_zchunk_heuristic(const KParams& kp, int R);
 // launch one fused step (mode MODE_STEP), an observation pass (MODE_OBS) or a
 // field dump (MODE_FIELDS); returns the number of CTAs through *nblocks
 using StepFn = cudaError_t (*)(const Launch&, int mode, int* nblocks);
+
+// n >= 2 steps of the D3Q19 FP32DEV explicit line schemes at tau = 1 on the
+// moments rho, j (mom3d.cuh): from the populations and density fin, rin back
+// into the same buffers; fout is scratch.  mom3d_ok: whether the case and the
+// scratch (19 N floats) allow it.
+bool mom3d_ok(const KParams& kp, int scheme, int prec);
+cudaError_t mom3d_steps(const Launch& c, int scheme, int prec, long long n);
 
 // precision index: 0 = FP64, 1 = FP32DEV with FP32 mu, 2 = FP32DEV with FP64 mu
 StepFn step2d_fn(int scheme, int prec);

@@ -902,8 +902,21 @@ extern "C" int lbm_autotune(lbm_handle* h, int* zc_out) {
   return best_zc > 0 ? LBM_OK : LBM_ECUDA;
 }
 
+// calls of two or more steps that run on the moments: the state between the
+// steps of one call is never seen, and at tau = 1 the populations are not
+// needed to advance it.  A call costs gather + expand once (0.63 ms at 256^3)
+// and 0.31 ms a step against 0.608 on the populations: break-even at two.
+static bool on_moments(const lbm_handle* h, long long n) {
+  return n >= 2 && h->D == 3 && h->mu && !h->compact && !h->layer && mom3d_ok(h->kp, h->p.scheme, h->prec);
+}
+
 extern "C" int lbm_step(lbm_handle* h, long long n) {
   if (!h || n < 0) return LBM_EINVAL;
+  if (on_moments(h, n)) {
+    if (mom3d_steps(make_launch(h, 1 - h->cur), h->p.scheme, h->prec, n) != cudaSuccess) return LBM_ECUDA;
+    h->t += n;
+    return LBM_OK;
+  }
   for (long long s = 0; s < n; ++s) {
     Launch c = make_launch(h, 1 - h->cur);
     if (run_pass(h, c, MODE_STEP, nullptr) != cudaSuccess) return LBM_ECUDA;
@@ -930,6 +943,35 @@ extern "C" int lbm_step_timed(lbm_handle* h, long long n, double* ms) {
   int rc = LBM_OK;
   for (; made < ne; ++made)
     if (cudaEventCreate(&e[made]) != cudaSuccess) { rc = LBM_ECUDA; break; }
+  if (rc == LBM_OK && on_moments(h, n)) {
+    // two events around every mu pass, one before and one after the call's work
+    cudaEvent_t ends[2] = {};
+    if (cudaEventCreate(&ends[0]) != cudaSuccess || cudaEventCreate(&ends[1]) != cudaSuccess) rc = LBM_ECUDA;
+    if (rc == LBM_OK) {
+      Launch c = make_launch(h, 1 - h->cur);
+      c.ev_mu = e;
+      cudaEventRecord(ends[0], h->stream);
+      if (mom3d_steps(c, h->p.scheme, h->prec, n) != cudaSuccess) rc = LBM_ECUDA;
+      cudaEventRecord(ends[1], h->stream);
+      h->t += n;
+    }
+    if (rc == LBM_OK && cudaEventSynchronize(ends[1]) != cudaSuccess) rc = LBM_ECUDA;
+    float a = 0.f;
+    for (long long s = 0; s < n && rc == LBM_OK; ++s) {
+      cudaEventElapsedTime(&a, e[2 * s], e[2 * s + 1]);
+      ms[0] += a;
+    }
+    if (rc == LBM_OK) {
+      cudaEventElapsedTime(&a, ends[0], ends[1]);
+      ms[2] = a;
+      ms[1] = ms[2] - ms[0];
+    }
+    for (cudaEvent_t x : ends)
+      if (x) cudaEventDestroy(x);
+    for (size_t k = 0; k < made; ++k) cudaEventDestroy(e[k]);
+    delete[] e;
+    return rc;
+  }
   for (long long s = 0; s < n && rc == LBM_OK; ++s) {
     Launch c = make_launch(h, 1 - h->cur);
     c.ev_mid = split ? e[3 * s + 1] : nullptr;

@@ -1,0 +1,124 @@
+// Launchers of the moment steps (mom3d.cuh): D3Q19, FP32 deviations, tau = 1,
+// explicit line schemes.
+#include <algorithm>
+
+#include "launch.cuh"
+#include "mom3d.cuh"
+
+namespace lbmd {
+
+namespace {
+
+#ifndef MOM_W
+#define MOM_W 16
+#endif
+constexpr int MW3 = MOM_W;  // warps of a k_mom3d CTA
+
+// columns per tile: the fewest tiles of at most 64 columns, evenly cut, none
+// narrower than four columns (a row's two edge nodes then lie in two lanes)
+MomGeo mom_geo(const KParams& kp) {
+  MomGeo g{};
+  g.LX = (kp.nx + 3) / 4 * 4 + 8;
+  g.PL = g.LX * kp.ny;
+  g.P = (g.PL * kp.nz + 63) / 64 * 64;
+  const int nt = (kp.nx + 63) / 64;
+  g.TW = ((kp.nx + nt - 1) / nt + 3) / 4 * 4;
+  while (kp.nx % g.TW != 0 && kp.nx % g.TW < 4) g.TW -= 4;
+  g.nt = (kp.nx + g.TW - 1) / g.TW;
+  return g;
+}
+
+// rows per band and planes per chunk (zc > 0: that many) together: the waves
+// of CTAs (one per SM) times a CTA's planes (two collided beyond the chunk,
+// the prologue worth two more) times the time of a plane, which grows with
+// the rows held (the band, one beyond either side, the edge warp, and about
+// four rows' worth of barrier and latency)
+void mom_cut(const KParams& kp, MomGeo* g, int* zc) {
+  const long long slots = device_sms();
+  const int fixed = *zc;
+  double best = 1e300;
+  for (int nb = (kp.ny + MW3 - 4) / (MW3 - 3); nb <= kp.ny; ++nb) {
+    const int rb = (kp.ny + nb - 1) / nb, bands = (kp.ny + rb - 1) / rb;
+    if (2 * rb < MW3 - 3 && best < 1e300) break;
+    for (int n = 1; n <= kp.nz; ++n) {
+      const int c = fixed > 0 ? fixed : (kp.nz + n - 1) / n;
+      if (c < 4 && n > 1) break;
+      const long long ctas = (long long)g->nt * bands * ((kp.nz + c - 1) / c);
+      const double cost = double((ctas + slots - 1) / slots) * (c + 4) * (rb + 7);
+      if (cost < best - 1e-9) { best = cost; *zc = c; g->RB = rb; g->nb = bands; }
+      if (fixed > 0 || ctas > 8 * slots) break;
+    }
+  }
+}
+
+template <int S>
+MomConst mom_const() {
+  auto two = [](double v) { return float2{float(v), float(v)}; };
+  MomConst k{};
+  for (int m = 1; m <= Sch<S>::R; ++m) {
+    k.g[m - 1] = two(Sch<S>::g(m));
+    k.h[m - 1] = two(Sch<S>::g(m) / 3.0);
+  }
+  k.m1 = two(-1.0); k.c45 = two(4.5); k.m15 = two(-1.5); k.m12 = two(-12.0);
+  k.w0 = two(1.0 / 3); k.w1 = two(1.0 / 18); k.w2 = two(1.0 / 36);
+  k.t1 = two(3.0 / 18); k.t2 = two(3.0 / 36); k.n1 = two(-3.0 / 18); k.n2 = two(-3.0 / 36);
+  return k;
+}
+
+template <int S, bool M64>
+cudaError_t steps(const Launch& c, long long n) {
+  const KParams& kp = c.kp;
+  MomGeo g = mom_geo(kp);
+  int zc = c.zc;
+  mom_cut(kp, &g, &zc);
+  using Sh = MomShape<S, MW3>;
+  static_assert(Sh::bytes <= size_t(227) * 1024, "shared memory of one CTA");
+  if (cudaError_t e = ensure_smem(k_mom3d<S, MW3>, Sh::bytes); e != cudaSuccess) return e;
+  float* s = static_cast<float*>(c.fout);  // scratch: rho x 2, j x 2, mu
+  float* r[2] = {s, s + g.P};
+  float* j[2] = {s + 2 * g.P, s + 5 * g.P};
+  float* mu = s + 8 * g.P;
+  const int elems = g.PL * kp.nz;
+  k_mom_gather<<<(elems + 255) / 256, 256, 0, c.stream>>>(kp, g, static_cast<const float*>(c.fin),
+                                                          static_cast<const float*>(c.rin), r[0], j[0], r[1], mu, j[1],
+                                                          c.aux.bad_step, c.aux.t);
+  // mu pass: about eight CTAs per SM, at least eight planes each
+  const int gm = ((kp.nx + 3) / 4 * kp.ny + 255) / 256;
+  const int nz8 = std::max(1, std::min((8 * device_sms() + gm - 1) / gm, (kp.nz + 7) / 8));
+  const int zm = (kp.nz + nz8 - 1) / nz8;
+  const dim3 gridm(gm, (kp.nz + zm - 1) / zm);
+  const dim3 grid(g.nt, g.nb, (kp.nz + zc - 1) / zc);
+  for (long long k = 0; k < n; ++k) {
+    const int a = int(k & 1);
+    if (c.ev_mu) cudaEventRecord(c.ev_mu[2 * k], c.stream);
+    k_mom_mu<S, M64><<<gridm, 256, 0, c.stream>>>(kp, g, r[a], mu, zm);
+    if (c.ev_mu) cudaEventRecord(c.ev_mu[2 * k + 1], c.stream);
+    k_mom3d<S, MW3><<<grid, Sh::NT, Sh::bytes, c.stream>>>(kp, g, r[a], mu, j[a], r[a ^ 1], j[a ^ 1], c.aux.bad_step,
+                                                           c.aux.t + k, zc, mom_const<S>());
+  }
+  const int a = int((n - 1) & 1);
+  k_mom_expand<S><<<int((kp.n + 255) / 256), 256, 0, c.stream>>>(
+      kp, g, r[a], mu, j[a], r[a ^ 1], const_cast<float*>(static_cast<const float*>(c.fin)),
+      const_cast<float*>(static_cast<const float*>(c.rin)));
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+bool mom3d_ok(const KParams& kp, int scheme, int prec) {
+  if ((prec != 1 && prec != 2) || kp.omega != 1.0) return false;
+  if (scheme != S_EFDS2 && scheme != S_EFDS4 && scheme != S_EFDS6) return false;
+  const long long LX = (kp.nx + 3) / 4 * 4 + 8, P = (LX * kp.ny * kp.nz + 63) / 64 * 64;
+  return 9 * P <= 19 * kp.n && 19 * kp.n < (1LL << 31);
+}
+
+cudaError_t mom3d_steps(const Launch& c, int scheme, int prec, long long n) {
+  switch (scheme) {
+    case S_EFDS2: return prec == 2 ? steps<S_EFDS2, true>(c, n) : steps<S_EFDS2, false>(c, n);
+    case S_EFDS4: return prec == 2 ? steps<S_EFDS4, true>(c, n) : steps<S_EFDS4, false>(c, n);
+    case S_EFDS6: return prec == 2 ? steps<S_EFDS6, true>(c, n) : steps<S_EFDS6, false>(c, n);
+    default: return cudaErrorNotSupported;
+  }
+}
+
+}  // namespace lbmd

@@ -1,0 +1,77 @@
+"""Steps on the moments (tau = 1: the populations between the steps of one call
+are not needed) against the same number of single steps, which carry the
+populations, and against the oracle."""
+import numpy as np
+import pytest
+
+import oracle as O
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def L():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2205_09186_gb300 as pkg
+    pkg.build()
+    from paper_2205_09186_gb300 import lbm
+    return lbm
+
+
+def start(L, lattice, shape, **kw):
+    nx, ny, nz = shape
+    s = L.Sim(L.make_params(lattice=lattice, nx=nx, ny=ny, nz=nz, Tr=0.9, k=0.3, kappa=0.1, **kw))
+    rng = np.random.default_rng(nx * 1000 + ny * 10 + nz)
+    rho = 0.15 + 0.01 * rng.standard_normal((nz, ny, nx))
+    s.lbm_init_density(rho)
+    return s, rho
+
+
+def check(L, a, b, steps, tol):
+    # FP32: each path rounds a population of about 0.15 a few times per step
+    # (2^-24 each), on either side: a few 1e-8 of the density per step
+    a.lbm_step(steps)
+    for _ in range(steps):
+        b.lbm_step(1)
+    assert a.lbm_get_step() == b.lbm_get_step() == steps
+    fa, fb = a.lbm_get_f(), b.lbm_get_f()
+    assert np.max(np.abs(fa - fb)) / 0.15 < tol
+    ra, rb = a.lbm_get_density(), b.lbm_get_density()
+    assert np.max(np.abs(ra - rb)) / 0.15 < tol
+    assert np.max(np.abs(ra - fa.sum(0).reshape(ra.shape))) / 0.15 < 1e-6  # the density is that of the populations
+    oa, ob = a.lbm_observables(), b.lbm_observables()
+    assert oa["status"] == ob["status"] == 0
+    assert oa["mass"] == pytest.approx(ob["mass"], rel=1e-6)
+
+
+# tiles of up to 64 columns, two per lane: odd nx ends a row in half a pair, 65
+# and 130 cut into 36 + 29 and 44 + 44 + 42; bands of up to 13 rows: 13 fills
+# one, 14 and 27 cut unevenly; 8 wraps every halo; 2 and 3 steps end in either
+# buffer
+@pytest.mark.parametrize("shape", [(8, 8, 8), (64, 13, 8), (65, 14, 12), (130, 27, 9), (33, 40, 21), (12, 9, 30)])
+@pytest.mark.parametrize("scheme,mu64,steps", [("EFDS2", 0, 2), ("EFDS4", 0, 3), ("EFDS6", 0, 12), ("EFDS6", 1, 3)])
+def test_d3q19_steps_on_moments(L, shape, scheme, mu64, steps):
+    kw = dict(scheme=scheme, precision=L.LBM_FP32DEV, mu_fp64=mu64)
+    (a, rho), (b, _) = start(L, L.LBM_D3Q19, shape, **kw), start(L, L.LBM_D3Q19, shape, **kw)
+    check(L, a, b, steps, 1e-6)
+    o = O.Sim(lattice=O.D3Q19, nx=shape[0], ny=shape[1], nz=shape[2], Tr=0.9, k=0.3, kappa=0.1, scheme=scheme)
+    o.set_f(np.stack([w * rho for w in O.lattice(O.D3Q19)[1]]))
+    assert o.step(steps) == 0
+    assert np.max(np.abs(a.lbm_get_density() - o.density())) / 0.15 < 1e-5
+
+
+def test_moments_report_the_first_bad_step(L):
+    # a cold second-order droplet: the density goes non-positive within the call
+    kw = dict(lattice=L.LBM_D3Q19, nx=48, ny=40, nz=36, Tr=0.3, k=0.3, kappa=0.1, scheme="EFDS2",
+              precision=L.LBM_FP32DEV)
+    a, b = L.Sim(L.make_params(**kw)), L.Sim(L.make_params(**kw))
+    for s in (a, b):
+        s.lbm_init_droplet(9.0)
+    a.lbm_step(400)
+    for _ in range(400):
+        b.lbm_step(1)
+    oa, ob = a.lbm_observables(), b.lbm_observables()
+    assert oa["status"] == ob["status"] == L.LBM_EUNSTABLE
+    assert abs(oa["step"] - ob["step"]) <= 2
