@@ -530,7 +530,11 @@ cudaError_t step_prec(const CompactBufs& cb, Launch c, int D, int mode, int* nbl
   c.gi.grho = grho;
   c.gi.mu = mu;
   if (gf3) return coll3d_gf_step(c, nblocks);
-  if (mode == MODE_STEP) return launch_gf<P, MODE_STEP>(c, D, nblocks);
+  if constexpr (std::is_same<P, PrecF64>::value) {
+    if (mode == MODE_STEP) return step64(c, D, S_CFDS4, nullptr);
+  } else {
+    if (mode == MODE_STEP) return launch_gf<P, MODE_STEP>(c, D, nblocks);
+  }
   if (mode == MODE_OBS) return launch_gf<P, MODE_OBS>(c, D, nblocks);
   return launch_gf<P, MODE_FIELDS>(c, D, nblocks);
 }

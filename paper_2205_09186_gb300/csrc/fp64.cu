@@ -1,0 +1,51 @@
+// Launchers of the FP64 step (fp64.cuh).
+#include "fp64.cuh"
+#include "launch.cuh"
+
+namespace lbmd {
+
+namespace {
+
+// nodes per block: 128, fewer where that would leave SMs without a block
+int block64(const KParams& kp) {
+  const long long sms = device_sms();
+  return kp.n >= 4 * 128 * sms ? 128 : (kp.n >= 4 * 64 * sms ? 64 : 32);
+}
+
+template <int S, int LAT>
+cudaError_t step(const Launch& c, double* mu) {
+  const KParams& kp = c.kp;
+  const int bs = block64(kp), g = int((kp.n + bs - 1) / bs);
+  const double *fin = static_cast<const double*>(c.fin), *rin = static_cast<const double*>(c.rin);
+  double *fout = static_cast<double*>(c.fout), *rout = static_cast<double*>(c.rout);
+  if constexpr (!Sch<S>::GF) k64_mu<S, LAT><<<g, bs, 0, c.stream>>>(kp, rin, mu);
+  if (LAT == 0 && c.mrt.on) {
+    if constexpr (LAT == 0) k64_coll<S, LAT, 2><<<g, bs, 0, c.stream>>>(kp, fin, fout, rin, mu, c.gi, c.aux, c.mrt);
+  } else if (kp.omega == 1.0) {
+    k64_coll<S, LAT, 0><<<g, bs, 0, c.stream>>>(kp, fin, fout, rin, mu, c.gi, c.aux, c.mrt);
+  } else {
+    k64_coll<S, LAT, 1><<<g, bs, 0, c.stream>>>(kp, fin, fout, rin, mu, c.gi, c.aux, c.mrt);
+  }
+  k64_rho<Lattice<LAT>::Q><<<g, bs, 0, c.stream>>>(kp, fout, rout, c.aux.bad_step, c.aux.t + 1);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t step64(const Launch& c, int D, int scheme, double* mu) {
+  const bool two = D == 2;
+  switch (scheme) {
+    case S_EFDS2: return two ? step<S_EFDS2, 0>(c, mu) : step<S_EFDS2, 1>(c, mu);
+    case S_EFDS4: return two ? step<S_EFDS4, 0>(c, mu) : step<S_EFDS4, 1>(c, mu);
+    case S_EFDS6: return two ? step<S_EFDS6, 0>(c, mu) : step<S_EFDS6, 1>(c, mu);
+    case S_E4: return two ? step<S_E4, 0>(c, mu) : step<S_E4, 1>(c, mu);
+    case S_E8: return two ? step<S_E8, 0>(c, mu) : cudaErrorNotSupported;
+    case S_CFDS4:
+    case S_CFDS6:
+    case S_CFDS8:
+    case S_OCFDS4: return two ? step<S_CFDS4, 0>(c, mu) : step<S_CFDS4, 1>(c, mu);
+    default: return cudaErrorNotSupported;
+  }
+}
+
+}  // namespace lbmd

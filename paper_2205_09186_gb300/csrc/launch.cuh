@@ -58,6 +58,10 @@ using StepFn = cudaError_t (*)(const Launch&, int mode, int* nblocks);
 bool mom3d_ok(const KParams& kp, int scheme, int prec);
 cudaError_t mom3d_steps(const Launch& c, int scheme, int prec, long long n);
 
+// one FP64 step on node-parallel passes (fp64.cuh), explicit and isotropic
+// schemes with mu an N-double buffer, compact ones reading c.gi
+cudaError_t step64(const Launch& c, int D, int scheme, double* mu);
+
 // precision index: 0 = FP64, 1 = FP32DEV with FP32 mu, 2 = FP32DEV with FP64 mu
 StepFn step2d_fn(int scheme, int prec);
 StepFn step3d_fn(int scheme, int prec);

@@ -44,6 +44,7 @@ struct lbm_handle {
   bool compact = false;
   int zc = 0;  // z-chunk of the pipelined D3Q19 kernel (0 = heuristic)
   void* mu = nullptr;  // mu field of the split D3Q19 FP32DEV path
+  double* mu64 = nullptr;  // mu field of the FP64 step (explicit and isotropic schemes)
   signed char* layer = nullptr;  // wall layers (Appendix A): 0 fluid, 1..3, 4 deeper; null: no walls
   void* wmu = nullptr;           // mu field of the wall step (N values of the precision's mu type)
   double mu_w = 0.0;             // wall chemical potential
@@ -543,6 +544,7 @@ extern "C" void lbm_destroy(lbm_handle* h) {
   dfree(h, h->d_partials, size_t(h->n_partials) * 4 * 8);
   dfree(h, h->d_obs, 64 + sizeof(lbm_obs));
   dfree(h, h->mu, size_t(h->N) * 4);
+  dfree(h, h->mu64, size_t(h->N) * 8);
   dfree(h, h->qc, size_t(h->n_qc) * 8);
   dfree(h, h->layer, size_t(h->N));
   dfree(h, h->wmu, size_t(h->N) * 8);
@@ -620,6 +622,8 @@ extern "C" int lbm_create(const lbm_params* params, void* stream, const lbm_allo
     h->mu = dalloc(h, size_t(h->N) * 4);
     ok = h->mu != nullptr;
   }
+  // (without this buffer the step runs on the fused kernels)
+  if (ok && !h->compact && h->prec == 0) h->mu64 = static_cast<double*>(dalloc(h, size_t(h->N) * 8));
   // tensor maps of both population buffers for the D3Q19 FP32DEV collision
   // pass's copies (split explicit schemes and compact schemes)
   if (ok && h->D == 3 && (h->prec == 1 || h->prec == 2)) {
@@ -809,6 +813,7 @@ static cudaError_t run_pass(lbm_handle* h, const Launch& c, int mode, int* nb) {
     return wall_step(w, h->D == 2 ? 0 : 1, h->p.scheme, h->prec, mode, nb);
   }
   if (h->compact) return compact_step(h->cb, c, h->D, h->p.scheme, h->prec, mode, nb);
+  if (mode == MODE_STEP && h->mu64) return step64(c, h->D, h->p.scheme, h->mu64);
   return h->fn(c, mode, nb);
 }
 
