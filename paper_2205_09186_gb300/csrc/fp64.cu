@@ -18,6 +18,15 @@ cudaError_t step(const Launch& c, double* mu) {
   const int bs = block64(kp), g = int((kp.n + bs - 1) / bs);
   const double *fin = static_cast<const double*>(c.fin), *rin = static_cast<const double*>(c.rin);
   double *fout = static_cast<double*>(c.fout), *rout = static_cast<double*>(c.rout);
+  if constexpr (LAT == 0 && !Sch<S>::GF) {
+    const dim3 t((kp.nx + T64X - 1) / T64X, (kp.ny + T64Y - 1) / T64Y);
+    if ((long long)t.x * t.y <= device_sms()) {
+      if (c.mrt.on) k64_tile<S, 2><<<t, T64N, 0, c.stream>>>(kp, fin, fout, rin, rout, c.aux, c.mrt);
+      else if (kp.omega == 1.0) k64_tile<S, 0><<<t, T64N, 0, c.stream>>>(kp, fin, fout, rin, rout, c.aux, c.mrt);
+      else k64_tile<S, 1><<<t, T64N, 0, c.stream>>>(kp, fin, fout, rin, rout, c.aux, c.mrt);
+      return cudaGetLastError();
+    }
+  }
   if constexpr (!Sch<S>::GF) k64_mu<S, LAT><<<g, bs, 0, c.stream>>>(kp, rin, mu);
   if (LAT == 0 && c.mrt.on) {
     if constexpr (LAT == 0) k64_coll<S, LAT, 2><<<g, bs, 0, c.stream>>>(kp, fin, fout, rin, mu, c.gi, c.aux, c.mrt);

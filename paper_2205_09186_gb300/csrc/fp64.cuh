@@ -129,7 +129,72 @@ __device__ constexpr int opp64(int i) {
   return i;
 }
 
-// COLL: 0 single relaxation at tau = 1, 1 at any tau, 2 the D2Q9 MRT operator.
+// Post-collision populations of one node from its populations f, density r and
+// the gradients of mu and rho, handed to put(i, value).  COLL: 0 single
+// relaxation at tau = 1, 1 at any tau, 2 the D2Q9 MRT operator.
+template <int LAT, int COLL, class Put>
+__device__ __forceinline__ void post64(const KParams& p, const Mrt& mrt, const double* f, double r, const double* gm,
+                                       const double* gr, Put put) {
+  using L = Lattice<LAT>;
+  constexpr int Q = L::Q, D = L::D;
+  double jx = 0.0, jy = 0.0, jz = 0.0;
+#pragma unroll
+  for (int i = 1; i < Q; ++i) {
+    const int o = opp64<L>(i);
+    if (o < i) continue;
+    const double d = f[i] - f[o];
+    if (L::ex(i) != 0) jx = L::ex(i) > 0 ? jx + d : jx - d;
+    if (L::ey(i) != 0) jy = L::ey(i) > 0 ? jy + d : jy - d;
+    if (L::ez(i) != 0) jz = L::ez(i) > 0 ? jz + d : jz - d;
+  }
+  // v = u + F / rho, F = -rho grad mu + grad rho / 3 (Eq. 12)
+  const double ir = rcp64(r), ir3 = ir * (1.0 / 3.0);
+  const double vx = fma(gr[0], ir3, fma(jx, ir, -gm[0])), vy = fma(gr[1], ir3, fma(jy, ir, -gm[1])),
+               vz = D == 3 ? fma(gr[2], ir3, fma(jz, ir, -gm[2])) : 0.0;
+  const double ux = COLL ? jx * ir : 0.0, uy = COLL ? jy * ir : 0.0, uz = COLL && D == 3 ? jz * ir : 0.0;
+  if constexpr (COLL == 2) {
+    double post[Q];
+    mrt_post9<double>(f, r, r, ux, uy, vx, vy, mrt, post);
+#pragma unroll
+    for (int i = 0; i < Q; ++i) put(i, post[i]);
+  } else {
+    // w rho (1 - 1.5 v.v + 4.5 (e.v)^2 +- 3 e.v) at tau = 1; else the same with
+    // omega for 1 and the u terms times omega - 1 added, plus (1 - omega) f_i
+    const double o1 = p.omega - 1.0;
+    double vv = vx * vx + vy * vy;
+    if constexpr (D == 3) vv = fma(vz, vz, vv);
+    double ev = fma(-1.5, vv, 1.0), sx = vx, sy = vy, sz = vz;
+    if constexpr (COLL == 1) {
+      double uu = ux * ux + uy * uy;
+      if constexpr (D == 3) uu = fma(uz, uz, uu);
+      ev = fma(o1, fma(-1.5, uu, 1.0), ev);
+      sx = fma(o1, ux, sx);
+      sy = fma(o1, uy, sy);
+      sz = fma(o1, uz, sz);
+    }
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+      const int o = opp64<L>(i);
+      if (o < i) continue;
+      const double wr = L::w(i) * r;
+      if (i == 0) {
+        put(0, COLL == 1 ? fma(wr, ev, -o1 * f[0]) : wr * ev);
+        continue;
+      }
+      const double E = edot64<L>(i, vx, vy, vz), t = (3.0 * L::w(i)) * r;
+      double even = fma(4.5, E * E, ev), odd = E;
+      if constexpr (COLL == 1) {
+        const double U = edot64<L>(i, ux, uy, uz);
+        even = fma(4.5 * o1, U * U, even);
+        odd = edot64<L>(i, sx, sy, sz);
+      }
+      const double a = wr * even;
+      put(i, COLL == 1 ? fma(-o1, f[i], fma(t, odd, a)) : fma(t, odd, a));
+      put(o, COLL == 1 ? fma(-o1, f[o], fma(-t, odd, a)) : fma(-t, odd, a));
+    }
+  }
+}
+
 // A compact scheme (GF) reads grad mu and grad rho from gi, the others take
 // them from rho and mu.
 template <int S, int LAT, int COLL>
@@ -158,60 +223,77 @@ __global__ void k64_coll(const KParams p, const double* __restrict__ fin, double
     grad64<S, LAT>(rho, c, gr);
   }
   if (!(r > 0.0)) atomicMin(aux.bad_step, (unsigned long long)aux.t);
-  double jx = 0.0, jy = 0.0, jz = 0.0;
-#pragma unroll
-  for (int i = 1; i < Q; ++i) {
-    const int o = opp64<L>(i);
-    if (o < i) continue;
-    const double d = f[i] - f[o];
-    if (L::ex(i) != 0) jx = L::ex(i) > 0 ? jx + d : jx - d;
-    if (L::ey(i) != 0) jy = L::ey(i) > 0 ? jy + d : jy - d;
-    if (L::ez(i) != 0) jz = L::ez(i) > 0 ? jz + d : jz - d;
+  post64<LAT, COLL>(p, mrt, f, r, gm, gr,
+                    [&](int i, double v) { fout[i * N + c.at(L::ex(i), L::ey(i), L::ez(i))] = v; });
+}
+
+// The whole D2Q9 step of an 8 x 4 tile by one CTA of four warps (one per
+// scheduler, each with its own FP64 pipe): density of the tile and its halo in
+// shared memory, mu on the tile and R + 1 beyond, collision of the tile and a
+// ring, next density from the ring's and the tile's populations.  For lattices
+// whose tiles find an SM each: the redundant nodes run on pipes that would idle,
+// and one launch takes the place of three.  64^2 EFDS2 takes 8.2 us a step (16.4
+// on the three passes); with two tiles per SM the pipes are shared and the passes
+// (16.4 us at 96^2 EFDS6) are level with it.
+constexpr int T64X = 8, T64Y = 4, T64N = 128;
+
+template <int S, int COLL>
+__global__ void __launch_bounds__(T64N) k64_tile(const KParams p, const double* __restrict__ fin,
+                                                 double* __restrict__ fout, const double* __restrict__ rin,
+                                                 double* __restrict__ rout, const StepAux aux, const Mrt mrt) {
+  using L = Lattice<0>;
+  constexpr int Q = 9, R = Sch<S>::R, H = 2 * R + 1;
+  constexpr int RW = T64X + 2 * H, RH = T64Y + 2 * H, MW = T64X + 2 * R + 2, MH = T64Y + 2 * R + 2;
+  constexpr int CW = T64X + 2, CH = T64Y + 2;
+  __shared__ double s_r[RH * RW], s_m[MH * MW], s_f[Q][CH * CW];
+  const int nx = p.nx, ny = p.ny, N = int(p.n), x0 = blockIdx.x * T64X, y0 = blockIdx.y * T64Y;
+  const int tid = threadIdx.x;
+  for (int e = tid; e < RW * RH; e += T64N) {
+    const int ry = e / RW, rx = e - ry * RW;
+    int gx = x0 - H + rx, gy = y0 - H + ry;
+    gx = wrapn(gx, nx);
+    gy = wrapn(gy, ny);
+    s_r[e] = rin[gy * nx + gx];
   }
-  const double ir = 1.0 / r;
-  const double ux = jx * ir, uy = jy * ir, uz = D == 3 ? jz * ir : 0.0;
-  // v = u + F / rho, F = -rho grad mu + grad rho / 3 (Eq. 12)
-  const double ir3 = ir * (1.0 / 3.0);
-  const double vx = ux + (gr[0] * ir3 - gm[0]), vy = uy + (gr[1] * ir3 - gm[1]),
-               vz = D == 3 ? uz + (gr[2] * ir3 - gm[2]) : 0.0;
-  auto push = [&](int i, double v) { fout[i * N + c.at(L::ex(i), L::ey(i), L::ez(i))] = v; };
-  if constexpr (COLL == 2) {
-    double post[Q];
-    mrt_post9<double>(f, r, r, ux, uy, vx, vy, mrt, post);
+  // the populations of this thread's collided node travel meanwhile
+  double f[Q];
+  const int cy = tid / CW, cx = tid - cy * CW;
+  const bool col = tid < CW * CH;
+  const int gx = wrapn(x0 - 1 + cx, nx), gy = wrapn(y0 - 1 + cy, ny);
+  if (col) {
 #pragma unroll
-    for (int i = 0; i < Q; ++i) push(i, post[i]);
-  } else {
-    // w rho (1 - 1.5 v.v + 4.5 (e.v)^2 +- 3 e.v) at tau = 1; else the same with
-    // omega for 1 and the u terms times omega - 1 added, plus (1 - omega) f_i
-    const double om = p.omega, o1 = om - 1.0;
-    double ev = 1.0 - 1.5 * (vx * vx + vy * vy + (D == 3 ? vz * vz : 0.0));
-    double sx = vx, sy = vy, sz = vz;
-    if constexpr (COLL == 1) {
-      ev += o1 - (1.5 * o1) * (ux * ux + uy * uy + (D == 3 ? uz * uz : 0.0));
-      sx += o1 * ux;
-      sy += o1 * uy;
-      sz += o1 * uz;
-    }
+    for (int i = 0; i < Q; ++i) f[i] = fin[i * N + gy * nx + gx];
+  }
+  __syncthreads();
+  for (int e = tid; e < MW * MH; e += T64N) {
+    const int my = e / MW, mx = e - my * MW, sx = mx + R, sy = my + R;
+    const double r = s_r[sy * RW + sx];
+    s_m[e] = p.k2 * eos_mu<double>(r, p) - p.kappa * lap2d<S, double>(s_r, RW, sx, sy);
+  }
+  __syncthreads();
+  if (col) {
+    const int lx = cx - 1, ly = cy - 1;
+    const bool own = lx >= 0 && lx < T64X && ly >= 0 && ly < T64Y && x0 + lx < nx && y0 + ly < ny;
+    const double r = s_r[(ly + H) * RW + lx + H];
+    double gm[3], gr[3];
+    grad2d<S, double>(s_m, MW, lx + R + 1, ly + R + 1, gm[0], gm[1]);
+    grad2d<S, double>(s_r, RW, lx + H, ly + H, gr[0], gr[1]);
+    gm[2] = gr[2] = 0.0;
+    if (own && !(r > 0.0)) atomicMin(aux.bad_step, (unsigned long long)aux.t);
+    post64<0, COLL>(p, mrt, f, r, gm, gr, [&](int i, double v) {
+      s_f[i][tid] = v;
+      if (own) fout[i * N + wrapi(gy + L::ey(i), ny) * nx + wrapi(gx + L::ex(i), nx)] = v;
+    });
+  }
+  __syncthreads();
+  if (tid < T64X * T64Y) {
+    const int ly = tid / T64X, lx = tid - ly * T64X;
+    if (x0 + lx < nx && y0 + ly < ny) {
+      double a = 0.0;
 #pragma unroll
-    for (int i = 0; i < Q; ++i) {
-      const int o = opp64<L>(i);
-      if (o < i) continue;
-      const double w = L::w(i);
-      const double wr = w * r;
-      if (i == 0) {
-        push(0, COLL == 1 ? wr * ev - o1 * f[0] : wr * ev);
-        continue;
-      }
-      const double E = edot64<L>(i, vx, vy, vz);
-      double even = 4.5 * (E * E) + ev, odd = E;
-      if constexpr (COLL == 1) {
-        const double U = edot64<L>(i, ux, uy, uz);
-        even += (4.5 * o1) * (U * U);
-        odd = edot64<L>(i, sx, sy, sz);
-      }
-      const double a = wr * even, b = (3.0 * wr) * odd;
-      push(i, COLL == 1 ? (a + b) - o1 * f[i] : a + b);
-      push(o, COLL == 1 ? (a - b) - o1 * f[o] : a - b);
+      for (int i = 0; i < Q; ++i) a += s_f[i][(ly + 1 - L::ey(i)) * CW + lx + 1 - L::ex(i)];
+      rout[(y0 + ly) * nx + x0 + lx] = a;
+      if (!(a > 0.0)) atomicMin(aux.bad_step, (unsigned long long)(aux.t + 1));
     }
   }
 }

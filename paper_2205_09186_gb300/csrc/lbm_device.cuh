@@ -135,6 +135,11 @@ __device__ __forceinline__ T eos_mu(T rho, const KParams& p) {
   return cs_mu<T>(rho, T(p.RT), T(p.b4), T(p.two_a));
 }
 
+// FP64: eos64.cuh (included at the end of this file)
+__device__ __forceinline__ double eos_mu64(double rho, const KParams& p);
+template <>
+__device__ __forceinline__ double eos_mu<double>(double rho, const KParams& p) { return eos_mu64(rho, p); }
+
 // FP32 form with the hardware logarithm and division approximations, for the
 // FP32-deviation kernels; the constants converted once per thread
 struct EosF {
@@ -375,3 +380,5 @@ struct FSum {
 };
 
 }  // namespace lbmd
+
+#include "eos64.cuh"

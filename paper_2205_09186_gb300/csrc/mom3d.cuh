@@ -164,6 +164,7 @@ __global__ void __launch_bounds__(256) k_mom_mu(const KParams p, const MomGeo g,
   auto ld = [&](int zo, int o) { return __ldg(reinterpret_cast<const float4*>(rin + zo + o)); };
   const float k2 = float(p.k2), kap = float(p.kappa), rref = float(p.rho_ref);
   const EosF ef = eos_f(p);
+  const MuConst<M64> mc(p);
   float4 q[2 * R + 1];
 #pragma unroll
   for (int d = 1; d <= 2 * R; ++d) q[d] = ld(wrapi(z0 - R - 1 + d, nz) * g.PL, col);
@@ -191,7 +192,7 @@ __global__ void __launch_bounds__(256) k_mom_mu(const KParams p, const MomGeo g,
     const float lap[4] = {la.x, la.y, lb.x, lb.y};
     float res[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) res[k] = mu_value<M64>(p, ef, k2, kap, rref, row[4 + k], lap[k]);
+    for (int k = 0; k < 4; ++k) res[k] = mu_value<M64>(p, ef, mc, k2, kap, rref, row[4 + k], lap[k]);
     float* out = mu + zo + col;
     if (x + 4 <= nx) *reinterpret_cast<float4*>(out) = make_float4(res[0], res[1], res[2], res[3]);
     if (x < 4 || x + 8 > nx) {

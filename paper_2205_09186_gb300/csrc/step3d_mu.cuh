@@ -74,16 +74,31 @@ struct EdgeZero {
 // through the 8 planes with the z neighbours in a register queue.
 constexpr int MUX = 32, MUY = 8, MUZ = 8, MUT = MUX * MUY;
 
-// M64: the EOS chemical potential k^2 psi'(rho) evaluated in FP64 from
-// rho = rho_ref + deviation (FP64 division and logarithm), the Laplacian term
-// in FP32 as with M64 off, the sum rounded once to the float mu field.
+// M64: the EOS chemical potential k^2 psi'(rho) from rho = rho_ref + deviation
+// beyond FP32, the Laplacian (FP32 as with M64 off) subtracted, the sum rounded
+// once to the float mu field: Carnahan-Starling in double-float, which rounds
+// to the float FP64 gives but for about one node in a million, on the FP32 pipe
+// (256^3, k_mom_mu: 1.74 -> 0.129 ms); the other equations of state, and densities outside
+// the double-float's range, in FP64.
 template <bool M64>
-__device__ __forceinline__ float mu_value(const KParams& p, const EosF& ef, float k2, float kap, float rref, float dev,
-                                          float lap) {
-  if constexpr (M64)
+struct MuConst {
+  __device__ __forceinline__ explicit MuConst(const KParams&) {}
+};
+template <>
+struct MuConst<true> {
+  CsDf cs;
+  __device__ __forceinline__ explicit MuConst(const KParams& p) : cs(cs_df(p)) {}
+};
+template <bool M64>
+__device__ __forceinline__ float mu_value(const KParams& p, const EosF& ef, const MuConst<M64>& mc, float k2, float kap,
+                                          float rref, float dev, float lap) {
+  if constexpr (M64) {
+    float mu;
+    if (p.eos == 0 && cs_mu_df(dev, lap, mc.cs, &mu)) return mu;
     return float(p.k2 * eos_mu<double>(p.rho_ref + double(dev), p) - p.kappa * double(lap));
-  else
+  } else {
     return k2 * eos_mu_f(rref + dev, ef) - kap * lap;
+  }
 }
 
 // line schemes only (the isotropic 3D Laplacian needs diagonal neighbours)
@@ -123,6 +138,7 @@ __global__ void __launch_bounds__(MUT) k_mu3d(const KParams p, const float* __re
   if (x0 + tx >= nx || y0 + ty >= ny) return;
   const float k2 = float(p.k2), kap = float(p.kappa);
   const EosF ef = eos_f(p);
+  const MuConst<M64> mc(p);
   const float rref = float(p.rho_ref);
   const int cx = tx + R, cy = ty + R;
   float q[2 * R + 1];  // q[R + d]: density deviation at plane z + d of this column
@@ -144,7 +160,7 @@ __global__ void __launch_bounds__(MUT) k_mu3d(const KParams p, const float* __re
       for (int m = 1; m <= R; ++m)
         lap += float(Sch<S>::l(m)) * ((blk[pz][cy][cx + m] + blk[pz][cy][cx - m]) +
                                       (blk[pz][cy + m][cx] + blk[pz][cy - m][cx]) + (q[R + m] + q[R - m]));
-      out[dz * NXY] = mu_value<M64>(p, ef, k2, kap, rref, c, lap);
+      out[dz * NXY] = mu_value<M64>(p, ef, mc, k2, kap, rref, c, lap);
       if (enode) {
         ez.rz[(out - mu) + dz * NXY] = 0.f;
         if (!(rref + c > 0.f)) atomicMin(ez.bad, (unsigned long long)ez.t);
@@ -223,6 +239,7 @@ __global__ void __launch_bounds__(MZT) k_mu3d_zm(const KParams p, const float* _
   auto ld = [&](int z) { return __ldg(reinterpret_cast<const float4*>(rin + wrapi(z, nz) * NXY + col)); };
   const float k2 = float(p.k2), kap = float(p.kappa);
   const EosF ef = eos_f(p);
+  const MuConst<M64> mc(p);
   const float rref = float(p.rho_ref);
   issue(z0, 0);
   float4 q[2 * R + 1];  // q[R + d]: the four nodes' deviations at plane z + d
@@ -262,7 +279,7 @@ __global__ void __launch_bounds__(MZT) k_mu3d_zm(const KParams p, const float* _
       float lap = float(3.0 * Sch<S>::l(0)) * cv;
 #pragma unroll
       for (int m = 1; m <= R; ++m) lap += float(Sch<S>::l(m)) * ((row[4 + k + m] + row[4 + k - m]) + yz[k][m - 1]);
-      res[k] = mu_value<M64>(p, ef, k2, kap, rref, cv, lap);
+      res[k] = mu_value<M64>(p, ef, mc, k2, kap, rref, cv, lap);
     }
     *reinterpret_cast<float4*>(mu + z * NXY + col) = make_float4(res[0], res[1], res[2], res[3]);
     if (erow) {
