@@ -189,6 +189,260 @@ __global__ void k_adam(long long n, float* __restrict__ P, float* __restrict__ m
   P[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
 }
 
+// ------------------------------------------------------------------ training
+// All iterations of a training call in one launch by one cluster of eight
+// CTAs.  Each CTA owns an eighth of every layer's outputs: those rows of W and
+// b with their Adam moments stay in its shared memory for the whole call.
+// An iteration is a chain of 2 nl - 2 exchanges between the layers, a few
+// hundred kFLOP each at a few dozen samples, so its time is their latency; a
+// cluster barrier and a round trip through L2 take about a microsecond, where a
+// launch per pass (forward and backward by one CTA per 32 samples, reduction,
+// Adam) took 386 us an iteration for 31 samples of the 4-128-128-128-64
+// network, XX now.
+//  forward   z = W h + b for the CTA's outputs; lane = sample, warp = output
+//  backward  the CTA's share of W^T d, published; after the barrier the shares
+//            are added in the CTAs' order, dW and db are summed over the
+//            samples and Adam updates the rows in place
+// Activations are kept transposed, [feature][sample] with Bp = 32 ceil(B / 32)
+// samples, in global scratch read through L2 (another SM's L1 is not coherent);
+// h alternates between two buffers by iteration and the shares by layer, so
+// that one barrier separates every write from the next write of the buffer.
+constexpr int TC = 8;               // CTAs of the cluster
+constexpr int TRO = MAXW / TC;      // outputs per CTA at most
+constexpr int TNT = 32 * TRO;       // threads: one warp per output
+constexpr int TS = 36;              // row stride of the staged samples (16-byte rows, spread over banks)
+
+struct TrainScratch {
+  float* h;    // [2][nl][MAXW][Bp]
+  float* z;    // [nl][MAXW][Bp]
+  float* d;    // [2][MAXW][Bp]
+  float* part; // [2][TC][MAXW][Bp]
+  float* lossp;
+};
+
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+__host__ __device__ inline int train_ld(int in) { return (in + 3) / 4 * 4; }  // row stride of W in shared memory
+
+// where layer l starts in a copy of the CTA's rows (W, then b, of every layer,
+// each layer a multiple of 16 bytes); l = nl: the floats of the copy
+__host__ __device__ inline int train_off(const Net& net, int l) {
+  int n = 0;
+  for (int k = 0; k < l; ++k) n += (((net.sizes[k + 1] + TC - 1) / TC) * (train_ld(net.sizes[k]) + 1) + 3) / 4 * 4;
+  return n;
+}
+__host__ __device__ inline int train_rows(const Net& net) { return train_off(net, net.nl); }
+
+__global__ void __launch_bounds__(TNT, 1) k_mlp_train(const Net net, float* __restrict__ P, float* __restrict__ m,
+                                                      float* __restrict__ v, const float* __restrict__ x,
+                                                      const float* __restrict__ t, int B, int Bp, TrainScratch sc,
+                                                      int iters, float lr, double p1, double p2, float* loss) {
+  extern __shared__ __align__(16) float sm[];
+  const int nr = train_rows(net), tid = threadIdx.x, lane = tid & 31, w = tid >> 5, c = blockIdx.x;
+  float *sP = sm, *sM = sm + nr, *sV = sM + nr;
+  float* hT = sV + nr;           // [MAXW][TS]
+  float* dT = hT + MAXW * TS;    // [TRO][TS]
+  __shared__ float red[TNT / 32];
+  const int nl = net.nl, nout = net.sizes[nl];
+  const float scale = 2.f / (float(B) * float(nout)), b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
+  // the CTA's rows of layer l: where they start in sP, their first output, their count
+  auto rows = [&](int l, int& off, int& o0, int& no) {
+    off = train_off(net, l);
+    const int ro = (net.sizes[l + 1] + TC - 1) / TC;
+    o0 = c * ro;
+    no = max(0, min(ro, net.sizes[l + 1] - o0));
+  };
+  for (int k = tid; k < 3 * nr; k += TNT) sm[k] = 0.f;
+  __syncthreads();
+  for (int l = 0; l < nl; ++l) {
+    int off, o0, no;
+    rows(l, off, o0, no);
+    const int in = net.sizes[l], ld = train_ld(in), ro = (net.sizes[l + 1] + TC - 1) / TC;
+    for (int k = tid; k < no * in; k += TNT) {
+      const int o = k / in, i = k - o * in, to = off + o * ld + i;
+      const long long g = net.woff[l] + (long long)(o0 + o) * in + i;
+      sP[to] = P[g]; sM[to] = m[g]; sV[to] = v[g];
+    }
+    for (int o = tid; o < no; o += TNT) {
+      const int to = off + ro * ld + o;
+      const long long g = net.boff[l] + o0 + o;
+      sP[to] = P[g]; sM[to] = m[g]; sV[to] = v[g];
+    }
+  }
+  auto H = [&](int par, int l) { return sc.h + ((long long)par * nl + l) * MAXW * Bp; };
+  auto Z = [&](int l) { return sc.z + (long long)l * MAXW * Bp; };
+  auto D = [&](int l) { return sc.d + (long long)(l & 1) * MAXW * Bp; };
+  auto S = [&](int l, int cta) { return sc.part + ((long long)(l & 1) * TC + cta) * MAXW * Bp; };
+  // samples s0 .. s0 + 31 of layer l's input into hT (rows past the input are zero)
+  auto stage = [&](int par, int l, int s0) {
+    const int in = net.sizes[l], ld = train_ld(in);
+    for (int k = tid; k < ld * 32; k += TNT) {
+      const int i = k >> 5, s = k & 31;
+      float q = 0.f;
+      if (i < in && s0 + s < B)
+        q = l == 0 ? x[(long long)(s0 + s) * in + i] : __ldcg(H(par, l - 1) + (long long)i * Bp + s0 + s);
+      hT[i * TS + s] = q;
+    }
+  };
+  float lsum = 0.f;
+  for (int it = 0; it < iters; ++it) {
+    const int par = it & 1;
+    p1 *= double(b1);
+    p2 *= double(b2);
+    const float c1 = 1.f - float(p1), c2 = 1.f - float(p2);
+    lsum = 0.f;
+    // ---- forward
+    for (int l = 0; l < nl; ++l) {
+      int off, o0, no;
+      rows(l, off, o0, no);
+      const int ld = train_ld(net.sizes[l]), ro = (net.sizes[l + 1] + TC - 1) / TC;
+      for (int s0 = 0; s0 < Bp; s0 += 32) {
+        __syncthreads();
+        stage(par, l, s0);
+        __syncthreads();
+        if (w < no) {
+          const float* W = sP + off + w * ld;
+          float a0 = sP[off + ro * ld + w], a1 = 0.f, a2 = 0.f, a3 = 0.f;
+          for (int i = 0; i < ld; i += 4) {
+            const float4 q = *reinterpret_cast<const float4*>(W + i);
+            a0 += q.x * hT[i * TS + lane];
+            a1 += q.y * hT[(i + 1) * TS + lane];
+            a2 += q.z * hT[(i + 2) * TS + lane];
+            a3 += q.w * hT[(i + 3) * TS + lane];
+          }
+          const float a = (a0 + a1) + (a2 + a3);
+          const long long g = (long long)(o0 + w) * Bp + s0 + lane;
+          if (l < nl - 1) {
+            Z(l)[g] = a;
+            __stcg(H(par, l) + g, gelu(a));
+          } else {
+            float e = 0.f;
+            if (s0 + lane < B) e = a - t[(long long)(s0 + lane) * nout + o0 + w];
+            lsum += e * e;
+            D(l)[g] = e * scale;
+          }
+        }
+      }
+      if (l < nl - 1) cluster_sync();
+    }
+    // ---- backward
+    for (int l = nl - 1; l >= 0; --l) {
+      int off, o0, no;
+      rows(l, off, o0, no);
+      const int in = net.sizes[l], ld = train_ld(in), ro = (net.sizes[l + 1] + TC - 1) / TC;
+      __syncthreads();
+      if (l > 0) {
+        // this CTA's share of W^T d: eight inputs per warp
+        for (int s0 = 0; s0 < Bp; s0 += 32) {
+          float d[TRO];
+#pragma unroll
+          for (int o = 0; o < TRO; ++o) d[o] = o < no ? D(l)[(long long)(o0 + o) * Bp + s0 + lane] : 0.f;
+          const int i0 = w * 8;
+          if (i0 < in) {
+            float a[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int o = 0; o < TRO; ++o) {
+              if (o >= no) break;
+              const float* W = sP + off + o * ld + i0;
+              const float4 q = *reinterpret_cast<const float4*>(W);
+              a[0] += q.x * d[o]; a[1] += q.y * d[o]; a[2] += q.z * d[o]; a[3] += q.w * d[o];
+              if (i0 + 4 < ld) {
+                const float4 r = *reinterpret_cast<const float4*>(W + 4);
+                a[4] += r.x * d[o]; a[5] += r.y * d[o]; a[6] += r.z * d[o]; a[7] += r.w * d[o];
+              }
+            }
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+              if (i0 + k < in) __stcg(S(l, c) + (long long)(i0 + k) * Bp + s0 + lane, a[k]);
+          }
+        }
+        cluster_sync();
+        // d of the layer below at this CTA's outputs there
+        int offp, p0, np;
+        rows(l - 1, offp, p0, np);
+        for (int s0 = 0; s0 < Bp; s0 += 32)
+          if (w < np) {
+            const long long g = (long long)(p0 + w) * Bp + s0 + lane;
+            float q[TC];
+#pragma unroll
+            for (int k = 0; k < TC; ++k) q[k] = __ldcg(S(l, k) + g);
+            float a = 0.f;
+#pragma unroll
+            for (int k = 0; k < TC; ++k) a += q[k];
+            D(l - 1)[g] = s0 + lane < B ? a * gelu_d(Z(l - 1)[g]) : 0.f;
+          }
+      }
+      // dW, db over the samples, then Adam; thread: input i, outputs 4 og .. + 3
+      const int i = tid & (MAXW - 1), og = tid / MAXW;
+      float a[4] = {0.f, 0.f, 0.f, 0.f}, ab = 0.f;
+      for (int s0 = 0; s0 < Bp; s0 += 32) {
+        if (s0 > 0) __syncthreads();
+        stage(par, l, s0);
+        for (int k = tid; k < TRO * 32; k += TNT) {
+          const int o = k >> 5, s = k & 31;
+          dT[o * TS + s] = o < no ? D(l)[(long long)(o0 + o) * Bp + s0 + s] : 0.f;
+        }
+        __syncthreads();
+        if (i < in)
+#pragma unroll
+          for (int s = 0; s < 32; s += 4) {
+            const float4 q = *reinterpret_cast<const float4*>(hT + i * TS + s);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const float4 e = *reinterpret_cast<const float4*>(dT + (4 * og + k) * TS + s);
+              a[k] += (e.x * q.x + e.y * q.y) + (e.z * q.z + e.w * q.w);
+            }
+          }
+        if (tid < no)
+          for (int s = 0; s < 32; ++s) ab += dT[tid * TS + s];
+      }
+      auto adam = [&](int at, float g) {
+        const float mi = b1 * sM[at] + (1.f - b1) * g, vi = b2 * sV[at] + (1.f - b2) * g * g;
+        sM[at] = mi;
+        sV[at] = vi;
+        sP[at] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+      };
+      if (i < in)
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (4 * og + k < no) adam(off + (4 * og + k) * ld + i, a[k]);
+      if (tid < no) adam(off + ro * ld + tid, ab);
+    }
+  }
+  // the loss of the last evaluated parameters, then the rows back
+  for (int k = 16; k > 0; k >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, k);
+  if (lane == 0) red[w] = lsum;
+  __syncthreads();
+  if (tid == 0) {
+    float a = 0.f;
+    for (int k = 0; k < TNT / 32; ++k) a += red[k];
+    __stcg(sc.lossp + c, a);
+  }
+  for (int l = 0; l < nl; ++l) {
+    int off, o0, no;
+    rows(l, off, o0, no);
+    const int in = net.sizes[l], ld = train_ld(in), ro = (net.sizes[l + 1] + TC - 1) / TC;
+    for (int k = tid; k < no * in; k += TNT) {
+      const int o = k / in, i = k - o * in, to = off + o * ld + i;
+      const long long g = net.woff[l] + (long long)(o0 + o) * in + i;
+      P[g] = sP[to]; m[g] = sM[to]; v[g] = sV[to];
+    }
+    for (int o = tid; o < no; o += TNT) {
+      const int to = off + ro * ld + o;
+      const long long g = net.boff[l] + o0 + o;
+      P[g] = sP[to]; m[g] = sM[to]; v[g] = sV[to];
+    }
+  }
+  cluster_sync();
+  if (c == 0 && tid == 0 && iters > 0) {
+    float a = 0.f;
+    for (int k = 0; k < TC; ++k) a += __ldcg(sc.lossp + k);
+    *loss = a / (float(B) * float(nout));
+  }
+}
+
 }  // namespace
 
 struct lbm_mlp {
@@ -200,10 +454,15 @@ struct lbm_mlp {
   float *P = nullptr, *m = nullptr, *v = nullptr, *grad = nullptr, *gpart = nullptr, *lpart = nullptr;
   float *x = nullptr, *t = nullptr, *y = nullptr, *zs = nullptr, *hs = nullptr, *loss = nullptr;
   size_t act_floats = 0;
+  float* train = nullptr;  // scratch of k_mlp_train (null: training on the separate passes)
   int ndata = 0;
   int adam_t = 0;
   std::vector<std::pair<void*, size_t>> blocks;
 };
+
+// dynamic shared memory and scratch of k_mlp_train
+static size_t train_smem(const Net& net) { return size_t(3 * train_rows(net) + (MAXW + TRO) * TS) * 4; }
+static size_t train_floats(const Net& net, int Bp) { return size_t(3 * net.nl + 2 + 2 * TC) * MAXW * Bp + TC; }
 
 static void* malloc_cb(size_t b, void*) {
   void* p = nullptr;
@@ -268,6 +527,7 @@ extern "C" int lbm_mlp_create(const int* sizes, int nlayers, int max_batch, void
     lbm_mlp_destroy(m);
     return LBM_ENOMEM;
   }
+  if (train_smem(m->net) <= size_t(227) * 1024) m->train = mget(m, train_floats(m->net, (max_batch + 31) / 32 * 32));
   cudaMemsetAsync(m->m, 0, size_t(off) * 4, m->stream);
   cudaMemsetAsync(m->v, 0, size_t(off) * 4, m->stream);
   if (cudaStreamSynchronize(m->stream) != cudaSuccess) { lbm_mlp_destroy(m); return LBM_ECUDA; }
@@ -346,12 +606,55 @@ extern "C" int lbm_mlp_set_data(lbm_mlp* m, const float* host_x, const float* ho
   return e == cudaSuccess ? LBM_OK : LBM_ECUDA;
 }
 
+// n iterations by k_mlp_train; false (nothing launched) if it cannot be launched
+static bool launch_train(lbm_mlp* m, int n, float lr) {
+  const size_t smem = train_smem(m->net);
+  if (cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  const int B = m->ndata, Bp = (B + 31) / 32 * 32;
+  TrainScratch sc;
+  sc.h = m->train;
+  sc.z = sc.h + size_t(2) * m->net.nl * MAXW * Bp;
+  sc.d = sc.z + size_t(m->net.nl) * MAXW * Bp;
+  sc.part = sc.d + size_t(2) * MAXW * Bp;
+  sc.lossp = sc.part + size_t(2) * TC * MAXW * Bp;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = TC;
+  cfg.blockDim = TNT;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = m->stream;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = TC;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  const double p1 = std::pow(double(0.9f), double(m->adam_t)), p2 = std::pow(double(0.999f), double(m->adam_t));
+  if (cudaLaunchKernelEx(&cfg, k_mlp_train, m->net, m->P, m->m, m->v, static_cast<const float*>(m->x),
+                         static_cast<const float*>(m->t), B, Bp, sc, n, lr, p1, p2, m->loss) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  m->adam_t += n;
+  return true;
+}
+
 // iters full-batch Adam steps on the data set by lbm_mlp_set_data; the final
 // loss (of the parameters before the last update) is returned in *host_loss
 extern "C" int lbm_mlp_train(lbm_mlp* m, int iters, float lr, float* host_loss) {
   if (!m || iters < 0 || m->ndata < 1) return LBM_EINVAL;
   const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-  for (int it = 0; it < iters; ++it) {
+  // a launch per 2000 iterations (some tens of milliseconds): other work on
+  // the GPU's queue is not kept waiting by a long training call
+  int done = 0;
+  while (m->train && done < iters) {
+    const int n = iters - done < 2000 ? iters - done : 2000;
+    if (!launch_train(m, n, lr)) break;
+    done += n;
+  }
+  for (int it = done; it < iters; ++it) {
     cudaError_t e = run_grad(m, m->x, m->t, m->ndata);
     if (e != cudaSuccess) return LBM_ECUDA;
     m->adam_t += 1;

@@ -70,3 +70,32 @@ def test_adam_training_follows_oracle(L):
     l0 = O.mlp_loss_grad(sizes, p0, x, t)[0]
     lg, lo = O.mlp_loss_grad(sizes, pg.astype(np.float64), x, t)[0], O.mlp_loss_grad(sizes, po, x, t)[0]
     assert lo < 0.7 * l0 and lg == pytest.approx(lo, rel=2e-2)
+
+
+# training runs in one launch by a cluster whose CTAs own an eighth of every
+# layer's outputs: one layer and many, widths that do not divide by eight or by
+# four, fewer outputs than CTAs, one sample, a block of 32 samples and one
+# more, several blocks; a second call goes on from the first one's Adam state
+@pytest.mark.parametrize("sizes,batch", [([4, 128, 128, 128, 64], 31), ([3, 5], 1), ([7, 10, 3], 32), ([1, 33, 127, 6, 9], 33),
+                                         ([128, 128, 1], 70)])
+def test_cluster_training_follows_oracle(L, sizes, batch):
+    # twelve steps with gradients of order 1e-2: FP32 gradients are off by some
+    # 1e-7 of their scale, and Adam's steps of lr each by that over the
+    # gradient, so the bulk of the parameters moves together (test above)
+    p0 = init_params(sizes, 5).astype(np.float32).astype(np.float64)
+    rng = np.random.default_rng(batch)
+    x = rng.uniform(-1, 1, (batch, sizes[0])).astype(np.float32).astype(np.float64)
+    t = np.tanh(x @ rng.standard_normal((sizes[0], sizes[-1]))).astype(np.float32).astype(np.float64)
+    m = L.MLP(sizes, 80)
+    m.lbm_mlp_set_params(p0)
+    m.lbm_mlp_set_data(x, t)
+    m.lbm_mlp_train(5, lr=1e-3)
+    loss = m.lbm_mlp_train(7, lr=1e-3)
+    pg = m.lbm_mlp_get_params()
+    po, mo, vo = p0.copy(), np.zeros_like(p0), np.zeros_like(p0)
+    for it in range(1, 13):
+        lo, g = O.mlp_loss_grad(sizes, po, x, t)
+        O.adam_step(po, mo, vo, g, 1e-3, it)
+    assert loss == pytest.approx(lo, rel=1e-4)
+    d = np.abs(pg - po)
+    assert np.quantile(d, 0.99) < 1e-4 and np.median(d) < 1e-6
