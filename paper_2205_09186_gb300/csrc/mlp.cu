@@ -198,7 +198,7 @@ __global__ void k_adam(long long n, float* __restrict__ P, float* __restrict__ m
 // cluster barrier and a round trip through L2 take about a microsecond, where a
 // launch per pass (forward and backward by one CTA per 32 samples, reduction,
 // Adam) took 386 us an iteration for 31 samples of the 4-128-128-128-64
-// network, XX now.
+// network, 29 now (77 for 128 samples).
 //  forward   z = W h + b for the CTA's outputs; lane = sample, warp = output
 //  backward  the CTA's share of W^T d, published; after the barrier the shares
 //            are added in the CTAs' order, dW and db are summed over the
@@ -218,6 +218,19 @@ struct TrainScratch {
   float* d;    // [2][MAXW][Bp]
   float* part; // [2][TC][MAXW][Bp]
   float* lossp;
+};
+
+// Adam's constants of an iteration and its update of one parameter
+struct AdamK {
+  float b1, b2, eps, a, ic2;  // lr / (1 - b1^t), 1 / sqrt(1 - b2^t)
+  __device__ __forceinline__ AdamK(float lr, double p1, double p2)
+      : b1(0.9f), b2(0.999f), eps(1e-8f), a(lr / (1.f - float(p1))), ic2(1.f / sqrtf(1.f - float(p2))) {}
+  __device__ __forceinline__ void step(float* P, float* m, float* v, float g) const {
+    const float mi = b1 * *m + (1.f - b1) * g, vi = b2 * *v + (1.f - b2) * g * g;
+    *m = mi;
+    *v = vi;
+    *P -= __fdividef(a * mi, sqrtf(vi) * ic2 + eps);
+  }
 };
 
 __device__ __forceinline__ void cluster_sync() {
@@ -244,16 +257,23 @@ __global__ void __launch_bounds__(TNT, 1) k_mlp_train(const Net net, float* __re
   float *sP = sm, *sM = sm + nr, *sV = sM + nr;
   float* hT = sV + nr;           // [MAXW][TS]
   float* dT = hT + MAXW * TS;    // [TRO][TS]
+  float* zT = dT + TRO * TS;     // [4][TRO][32] partial sums of the forward pass
   __shared__ float red[TNT / 32];
+  __shared__ int s_off[MAXL], s_o0[MAXL], s_no[MAXL];
   const int nl = net.nl, nout = net.sizes[nl];
-  const float scale = 2.f / (float(B) * float(nout)), b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
+  const float scale = 2.f / (float(B) * float(nout));
   // the CTA's rows of layer l: where they start in sP, their first output, their count
   auto rows = [&](int l, int& off, int& o0, int& no) {
-    off = train_off(net, l);
-    const int ro = (net.sizes[l + 1] + TC - 1) / TC;
-    o0 = c * ro;
-    no = max(0, min(ro, net.sizes[l + 1] - o0));
+    off = s_off[l];
+    o0 = s_o0[l];
+    no = s_no[l];
   };
+  if (tid < nl) {
+    const int ro = (net.sizes[tid + 1] + TC - 1) / TC;
+    s_off[tid] = train_off(net, tid);
+    s_o0[tid] = c * ro;
+    s_no[tid] = max(0, min(ro, net.sizes[tid + 1] - c * ro));
+  }
   for (int k = tid; k < 3 * nr; k += TNT) sm[k] = 0.f;
   __syncthreads();
   for (int l = 0; l < nl; ++l) {
@@ -278,20 +298,26 @@ __global__ void __launch_bounds__(TNT, 1) k_mlp_train(const Net net, float* __re
   // samples s0 .. s0 + 31 of layer l's input into hT (rows past the input are zero)
   auto stage = [&](int par, int l, int s0) {
     const int in = net.sizes[l], ld = train_ld(in);
-    for (int k = tid; k < ld * 32; k += TNT) {
-      const int i = k >> 5, s = k & 31;
-      float q = 0.f;
-      if (i < in && s0 + s < B)
-        q = l == 0 ? x[(long long)(s0 + s) * in + i] : __ldcg(H(par, l - 1) + (long long)i * Bp + s0 + s);
-      hT[i * TS + s] = q;
+    float q[MAXW * 32 / TNT];
+#pragma unroll
+    for (int k = 0; k < MAXW * 32 / TNT; ++k) {
+      const int i = w + k * (TNT / 32);
+      q[k] = 0.f;
+      if (i < in && s0 + lane < B)
+        q[k] = l == 0 ? x[(long long)(s0 + lane) * in + i] : __ldcg(H(par, l - 1) + (long long)i * Bp + s0 + lane);
+    }
+#pragma unroll
+    for (int k = 0; k < MAXW * 32 / TNT; ++k) {
+      const int i = w + k * (TNT / 32);
+      if (i < ld) hT[i * TS + lane] = q[k];
     }
   };
   float lsum = 0.f;
   for (int it = 0; it < iters; ++it) {
     const int par = it & 1;
-    p1 *= double(b1);
-    p2 *= double(b2);
-    const float c1 = 1.f - float(p1), c2 = 1.f - float(p2);
+    p1 *= double(0.9f);
+    p2 *= double(0.999f);
+    const AdamK ad(lr, p1, p2);
     lsum = 0.f;
     // ---- forward
     for (int l = 0; l < nl; ++l) {
@@ -302,17 +328,35 @@ __global__ void __launch_bounds__(TNT, 1) k_mlp_train(const Net net, float* __re
         __syncthreads();
         stage(par, l, s0);
         __syncthreads();
-        if (w < no) {
-          const float* W = sP + off + w * ld;
-          float a0 = sP[off + ro * ld + w], a1 = 0.f, a2 = 0.f, a3 = 0.f;
-          for (int i = 0; i < ld; i += 4) {
-            const float4 q = *reinterpret_cast<const float4*>(W + i);
-            a0 += q.x * hT[i * TS + lane];
-            a1 += q.y * hT[(i + 1) * TS + lane];
-            a2 += q.z * hT[(i + 2) * TS + lane];
-            a3 += q.w * hT[(i + 3) * TS + lane];
+        // four outputs and a quarter of the inputs per warp: a staged value
+        // is read once for four multiply-adds; the quarters meet in zT
+        {
+          const int og = 4 * (w & 3), kq = w >> 2, n4 = ld >> 2;
+          const int ia = 4 * (kq * n4 / 4), ib = 4 * ((kq + 1) * n4 / 4);
+          if (og < no) {
+            const float* W = sP + off + og * ld;
+            const int w1 = og + 1 < no ? ld : 0, w2 = og + 2 < no ? 2 * ld : 0, w3 = og + 3 < no ? 3 * ld : 0;
+            float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+#pragma unroll 4
+            for (int i = ia; i < ib; i += 4) {
+              const float4 q0 = *reinterpret_cast<const float4*>(W + i), q1 = *reinterpret_cast<const float4*>(W + w1 + i),
+                           q2 = *reinterpret_cast<const float4*>(W + w2 + i), q3 = *reinterpret_cast<const float4*>(W + w3 + i);
+              const float h0 = hT[i * TS + lane], h1 = hT[(i + 1) * TS + lane], h2 = hT[(i + 2) * TS + lane],
+                          h3 = hT[(i + 3) * TS + lane];
+              a0 += q0.x * h0; a1 += q1.x * h0; a2 += q2.x * h0; a3 += q3.x * h0;
+              a0 += q0.y * h1; a1 += q1.y * h1; a2 += q2.y * h1; a3 += q3.y * h1;
+              a0 += q0.z * h2; a1 += q1.z * h2; a2 += q2.z * h2; a3 += q3.z * h2;
+              a0 += q0.w * h3; a1 += q1.w * h3; a2 += q2.w * h3; a3 += q3.w * h3;
+            }
+            float* zq = zT + (kq * TRO + og) * 32 + lane;
+            zq[0] = a0; zq[32] = a1; zq[64] = a2; zq[96] = a3;
           }
-          const float a = (a0 + a1) + (a2 + a3);
+        }
+        __syncthreads();
+        if (w < no) {
+          const float* zq = zT + w * 32 + lane;
+          const float a = sP[off + ro * ld + w] +
+                          ((zq[0] + zq[TRO * 32]) + (zq[2 * TRO * 32] + zq[3 * TRO * 32]));
           const long long g = (long long)(o0 + w) * Bp + s0 + lane;
           if (l < nl - 1) {
             Z(l)[g] = a;
@@ -398,17 +442,11 @@ __global__ void __launch_bounds__(TNT, 1) k_mlp_train(const Net net, float* __re
         if (tid < no)
           for (int s = 0; s < 32; ++s) ab += dT[tid * TS + s];
       }
-      auto adam = [&](int at, float g) {
-        const float mi = b1 * sM[at] + (1.f - b1) * g, vi = b2 * sV[at] + (1.f - b2) * g * g;
-        sM[at] = mi;
-        sV[at] = vi;
-        sP[at] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-      };
       if (i < in)
 #pragma unroll
         for (int k = 0; k < 4; ++k)
-          if (4 * og + k < no) adam(off + (4 * og + k) * ld + i, a[k]);
-      if (tid < no) adam(off + ro * ld + tid, ab);
+          if (4 * og + k < no) ad.step(sP + off + (4 * og + k) * ld + i, sM + off + (4 * og + k) * ld + i, sV + off + (4 * og + k) * ld + i, a[k]);
+      if (tid < no) ad.step(sP + off + ro * ld + tid, sM + off + ro * ld + tid, sV + off + ro * ld + tid, ab);
     }
   }
   // the loss of the last evaluated parameters, then the rows back
@@ -443,6 +481,225 @@ __global__ void __launch_bounds__(TNT, 1) k_mlp_train(const Net net, float* __re
   }
 }
 
+// The same for up to 32 samples (one per lane) and networks whose layers fit
+// beside each other in shared memory: every layer's input stays staged for the
+// backward pass, and what another CTA needs is stored straight into its shared
+// memory, so that a barrier is all that lies between two layers (31 samples of
+// the 4-128-128-128-64 network: 18 us an iteration against 29 through L2).
+//  hT     [nl + 1][MAXW][TS] inputs of the layers; the first hidden one twice,
+//         by iteration: it is stored before an iteration's first barrier, when
+//         another CTA may still be in the last backward pass (every other
+//         buffer's next store lies behind a barrier)
+//  part   [2][TC][TRO][32] shares of W^T d at this CTA's inputs, by layer parity
+__host__ __device__ inline int one_floats(const Net& net) {
+  return 3 * train_rows(net) + ((net.nl + 1) * MAXW + 2 * TRO) * TS + 2 * TC * TRO * 32 + net.nl * TRO * 32 + 4 * TRO * 32;
+}
+
+// address of this CTA's shared variable p in CTA `cta` of the cluster
+__device__ __forceinline__ unsigned remote(const float* p, int cta) {
+  unsigned a;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(unsigned(__cvta_generic_to_shared(p))), "r"(cta));
+  return a;
+}
+__device__ __forceinline__ void st_remote(unsigned a, float v) {
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
+
+__global__ void __launch_bounds__(TNT, 1) k_mlp_train_one(const Net net, float* __restrict__ P, float* __restrict__ m,
+                                                          float* __restrict__ v, const float* __restrict__ x,
+                                                          const float* __restrict__ t, int B, float* lossp, int iters,
+                                                          float lr, double p1, double p2, float* loss) {
+  extern __shared__ __align__(16) float sm[];
+  const int nr = train_rows(net), tid = threadIdx.x, lane = tid & 31, w = tid >> 5, c = blockIdx.x;
+  const int nl = net.nl, nout = net.sizes[nl];
+  float *sP = sm, *sM = sm + nr, *sV = sM + nr;
+  float* hT = sV + nr;                       // layer l's input: slot l, the first hidden one slot 1 or nl
+  float* dT = hT + (nl + 1) * MAXW * TS;     // [2][TRO][TS]
+  float* part = dT + 2 * TRO * TS;
+  float* zs = part + 2 * TC * TRO * 32;      // [nl][TRO][32]
+  float* zT = zs + nl * TRO * 32;            // [4][TRO][32]
+  __shared__ float red[TNT / 32];
+  __shared__ int s_off[MAXL], s_ro[MAXL];
+  const float scale = 2.f / (float(B) * float(nout));
+  for (int k = tid; k < one_floats(net); k += TNT) sm[k] = 0.f;
+  if (tid < nl) {
+    s_off[tid] = train_off(net, tid);
+    s_ro[tid] = (net.sizes[tid + 1] + TC - 1) / TC;
+  }
+  __syncthreads();
+  // outputs per CTA of layer l, this CTA's first one and their count
+  auto cnt = [&](int l) { return max(0, min(s_ro[l], net.sizes[l + 1] - c * s_ro[l])); };
+  for (int l = 0; l < nl; ++l) {
+    const int off = s_off[l], o0 = c * s_ro[l], no = cnt(l), in = net.sizes[l], ld = train_ld(in);
+    for (int k = tid; k < no * in; k += TNT) {
+      const int o = k / in, i = k - o * in, to = off + o * ld + i;
+      const long long g = net.woff[l] + (long long)(o0 + o) * in + i;
+      sP[to] = P[g]; sM[to] = m[g]; sV[to] = v[g];
+    }
+    for (int o = tid; o < no; o += TNT) {
+      const int to = off + s_ro[l] * ld + o;
+      const long long g = net.boff[l] + o0 + o;
+      sP[to] = P[g]; sM[to] = m[g]; sV[to] = v[g];
+    }
+  }
+  for (int k = tid; k < net.sizes[0] * 32; k += TNT) {
+    const int i = k >> 5, s = k & 31;
+    if (s < B) hT[i * TS + s] = x[(long long)s * net.sizes[0] + i];
+  }
+  const float tgt = lane < B && w < cnt(nl - 1) ? t[(long long)lane * nout + c * s_ro[nl - 1] + w] : 0.f;
+  auto slot = [&](int l, int it) { return hT + (l == 1 && (it & 1) ? nl : l) * MAXW * TS; };
+  cluster_sync();  // every CTA's buffers are zeroed before anything is stored into them
+  float lsum = 0.f;
+  for (int it = 0; it < iters; ++it) {
+    p1 *= double(0.9f);
+    p2 *= double(0.999f);
+    const AdamK ad(lr, p1, p2);
+    // ---- forward
+    for (int l = 0; l < nl; ++l) {
+      const int off = s_off[l], no = cnt(l), ld = train_ld(net.sizes[l]);
+      const float* h = slot(l, it);
+      const int og = 4 * (w & 3), kq = w >> 2, n4 = ld >> 2;
+      const int ia = 4 * (kq * n4 / 4), ib = 4 * ((kq + 1) * n4 / 4);
+      if (og < no) {
+        const float* W = sP + off + og * ld;
+        const int w1 = og + 1 < no ? ld : 0, w2 = og + 2 < no ? 2 * ld : 0, w3 = og + 3 < no ? 3 * ld : 0;
+        float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+#pragma unroll 4
+        for (int i = ia; i < ib; i += 4) {
+          const float4 q0 = *reinterpret_cast<const float4*>(W + i), q1 = *reinterpret_cast<const float4*>(W + w1 + i),
+                       q2 = *reinterpret_cast<const float4*>(W + w2 + i), q3 = *reinterpret_cast<const float4*>(W + w3 + i);
+          const float h0 = h[i * TS + lane], h1 = h[(i + 1) * TS + lane], h2 = h[(i + 2) * TS + lane],
+                      h3 = h[(i + 3) * TS + lane];
+          a0 += q0.x * h0; a1 += q1.x * h0; a2 += q2.x * h0; a3 += q3.x * h0;
+          a0 += q0.y * h1; a1 += q1.y * h1; a2 += q2.y * h1; a3 += q3.y * h1;
+          a0 += q0.z * h2; a1 += q1.z * h2; a2 += q2.z * h2; a3 += q3.z * h2;
+          a0 += q0.w * h3; a1 += q1.w * h3; a2 += q2.w * h3; a3 += q3.w * h3;
+        }
+        float* zq = zT + (kq * TRO + og) * 32 + lane;
+        zq[0] = a0; zq[32] = a1; zq[64] = a2; zq[96] = a3;
+      }
+      __syncthreads();
+      if (w < no) {
+        const float* zq = zT + w * 32 + lane;
+        const float a = sP[off + s_ro[l] * ld + w] + ((zq[0] + zq[TRO * 32]) + (zq[2 * TRO * 32] + zq[3 * TRO * 32]));
+        if (l < nl - 1) {
+          zs[(l * TRO + w) * 32 + lane] = a;
+          const float g = lane < B ? gelu(a) : 0.f;
+          const float* to = slot(l + 1, it) + (c * s_ro[l] + w) * TS + lane;
+#pragma unroll
+          for (int k = 0; k < TC; ++k) st_remote(remote(to, k), g);
+        } else {
+          const float e = lane < B ? a - tgt : 0.f;
+          lsum = e * e;
+          dT[((l & 1) * TRO + w) * TS + lane] = e * scale;
+        }
+      }
+      if (l < nl - 1) cluster_sync();
+    }
+    __syncthreads();
+    // ---- backward
+    for (int l = nl - 1; l >= 0; --l) {
+      const int off = s_off[l], no = cnt(l), in = net.sizes[l], ld = train_ld(in);
+      const float* d0 = dT + (l & 1) * TRO * TS;
+      if (l > 0) {
+        // this CTA's share of W^T d, eight inputs per warp, to the CTAs that own them
+        const int i0 = w * 8;
+        if (i0 < in) {
+          float a[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+          for (int o = 0; o < no; ++o) {
+            const float d = d0[o * TS + lane];
+            const float* W = sP + off + o * ld + i0;
+            const float4 q = *reinterpret_cast<const float4*>(W);
+            a[0] += q.x * d; a[1] += q.y * d; a[2] += q.z * d; a[3] += q.w * d;
+            if (i0 + 4 < ld) {
+              const float4 r = *reinterpret_cast<const float4*>(W + 4);
+              a[4] += r.x * d; a[5] += r.y * d; a[6] += r.z * d; a[7] += r.w * d;
+            }
+          }
+          const int rp = s_ro[l - 1];
+          const float* mine = part + ((l & 1) * TC + c) * TRO * 32 + lane;
+          int own = i0 / rp, at = i0 - own * rp;
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            if (i0 + k < in) st_remote(remote(mine + at * 32, own), a[k]);
+            if (++at == rp) { at = 0; ++own; }
+          }
+        }
+        cluster_sync();
+        // d of the layer below at this CTA's outputs there
+        if (w < cnt(l - 1)) {
+          const float* q = part + (l & 1) * TC * TRO * 32 + w * 32 + lane;
+          float a = 0.f;
+#pragma unroll
+          for (int k = 0; k < TC; ++k) a += q[k * TRO * 32];
+          dT[(((l - 1) & 1) * TRO + w) * TS + lane] = lane < B ? a * gelu_d(zs[((l - 1) * TRO + w) * 32 + lane]) : 0.f;
+        }
+      }
+      // dW, db over the samples, then Adam; thread: input i, outputs 4 og .. + 3
+      const int i = tid & (MAXW - 1), og = tid / MAXW;
+      const float* h = slot(l, it) + i * TS;
+      if (i < in && 4 * og < no) {
+        float a[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int s = 0; s < 32; s += 4) {
+          const float4 q = *reinterpret_cast<const float4*>(h + s);
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const float4 e = *reinterpret_cast<const float4*>(d0 + (4 * og + k) * TS + s);
+            a[k] += (e.x * q.x + e.y * q.y) + (e.z * q.z + e.w * q.w);
+          }
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (4 * og + k < no) {
+            const int at = off + (4 * og + k) * ld + i;
+            ad.step(sP + at, sM + at, sV + at, a[k]);
+          }
+      }
+      if (tid < no) {
+        float ab = 0.f;
+#pragma unroll
+        for (int s = 0; s < 32; s += 4) {
+          const float4 e = *reinterpret_cast<const float4*>(d0 + tid * TS + s);
+          ab += (e.x + e.y) + (e.z + e.w);
+        }
+        const int at = off + s_ro[l] * ld + tid;
+        ad.step(sP + at, sM + at, sV + at, ab);
+      }
+      __syncthreads();
+    }
+  }
+  // the loss of the last evaluated parameters, then the rows back
+  for (int k = 16; k > 0; k >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, k);
+  if (lane == 0) red[w] = lsum;
+  __syncthreads();
+  if (tid == 0) {
+    float a = 0.f;
+    for (int k = 0; k < TNT / 32; ++k) a += red[k];
+    __stcg(lossp + c, a);
+  }
+  for (int l = 0; l < nl; ++l) {
+    const int off = s_off[l], o0 = c * s_ro[l], no = cnt(l), in = net.sizes[l], ld = train_ld(in);
+    for (int k = tid; k < no * in; k += TNT) {
+      const int o = k / in, i = k - o * in, to = off + o * ld + i;
+      const long long g = net.woff[l] + (long long)(o0 + o) * in + i;
+      P[g] = sP[to]; m[g] = sM[to]; v[g] = sV[to];
+    }
+    for (int o = tid; o < no; o += TNT) {
+      const int to = off + s_ro[l] * ld + o;
+      const long long g = net.boff[l] + o0 + o;
+      P[g] = sP[to]; m[g] = sM[to]; v[g] = sV[to];
+    }
+  }
+  cluster_sync();
+  if (c == 0 && tid == 0 && iters > 0) {
+    float a = 0.f;
+    for (int k = 0; k < TC; ++k) a += __ldcg(lossp + k);
+    *loss = a / (float(B) * float(nout));
+  }
+}
+
 }  // namespace
 
 struct lbm_mlp {
@@ -461,7 +718,7 @@ struct lbm_mlp {
 };
 
 // dynamic shared memory and scratch of k_mlp_train
-static size_t train_smem(const Net& net) { return size_t(3 * train_rows(net) + (MAXW + TRO) * TS) * 4; }
+static size_t train_smem(const Net& net) { return size_t(3 * train_rows(net) + (MAXW + TRO) * TS + 4 * TRO * 32) * 4; }
 static size_t train_floats(const Net& net, int Bp) { return size_t(3 * net.nl + 2 + 2 * TC) * MAXW * Bp + TC; }
 
 static void* malloc_cb(size_t b, void*) {
@@ -606,14 +863,17 @@ extern "C" int lbm_mlp_set_data(lbm_mlp* m, const float* host_x, const float* ho
   return e == cudaSuccess ? LBM_OK : LBM_ECUDA;
 }
 
-// n iterations by k_mlp_train; false (nothing launched) if it cannot be launched
+// n iterations by k_mlp_train_one where the samples and the network fit it, else
+// by k_mlp_train; false (nothing launched) if it cannot be launched
 static bool launch_train(lbm_mlp* m, int n, float lr) {
-  const size_t smem = train_smem(m->net);
-  if (cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess) {
+  const int B = m->ndata, Bp = (B + 31) / 32 * 32;
+  const bool one = B <= 32 && size_t(one_floats(m->net)) * 4 <= size_t(227) * 1024;
+  const size_t smem = one ? size_t(one_floats(m->net)) * 4 : train_smem(m->net);
+  const void* fn = one ? reinterpret_cast<const void*>(k_mlp_train_one) : reinterpret_cast<const void*>(k_mlp_train);
+  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  const int B = m->ndata, Bp = (B + 31) / 32 * 32;
   TrainScratch sc;
   sc.h = m->train;
   sc.z = sc.h + size_t(2) * m->net.nl * MAXW * Bp;
@@ -632,8 +892,11 @@ static bool launch_train(lbm_mlp* m, int n, float lr) {
   cfg.attrs = &at;
   cfg.numAttrs = 1;
   const double p1 = std::pow(double(0.9f), double(m->adam_t)), p2 = std::pow(double(0.999f), double(m->adam_t));
-  if (cudaLaunchKernelEx(&cfg, k_mlp_train, m->net, m->P, m->m, m->v, static_cast<const float*>(m->x),
-                         static_cast<const float*>(m->t), B, Bp, sc, n, lr, p1, p2, m->loss) != cudaSuccess) {
+  const float *dx = m->x, *dt = m->t;
+  const cudaError_t e =
+      one ? cudaLaunchKernelEx(&cfg, k_mlp_train_one, m->net, m->P, m->m, m->v, dx, dt, B, sc.lossp, n, lr, p1, p2, m->loss)
+          : cudaLaunchKernelEx(&cfg, k_mlp_train, m->net, m->P, m->m, m->v, dx, dt, B, Bp, sc, n, lr, p1, p2, m->loss);
+  if (e != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
