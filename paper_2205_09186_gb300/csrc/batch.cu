@@ -24,6 +24,7 @@
 #include "../../include/lbm.h"
 #include "compact_dev.cuh"
 #include "launch.cuh"
+#include "mom2d.cuh"
 #include "step2d.cuh"
 #include "step2d_split.cuh"
 
@@ -32,6 +33,7 @@ using namespace lbmd;
 namespace {
 
 constexpr int TXB = 32, TYB = 8;
+constexpr unsigned long long BARRIER_NS = 1000000000ull;  // longest wait at a barrier
 
 struct CaseDev {
   KParams kp;
@@ -52,6 +54,9 @@ struct CaseDev {
   void* cmu;
   void* gmu;
   void* grho;
+  // steps on the moments (k_batch_mom); mom = 0: on the populations
+  int mom;
+  Mom2Geo mg;
 };
 
 // line coefficients of CFDS4, CFDS6, CFDS8, OCFDS4: [0] all PCR levels (FP64
@@ -474,6 +479,73 @@ __global__ void __launch_bounds__(NT2S, RPT >= 4 ? 1 : 2) k_batch_split(const Ca
   if (blockIdx.x == 0 && threadIdx.x == 0) ctl->t = t0 + nsteps;
 }
 
+// An even number of steps of the cases that advance on their moments (mom2d.cuh):
+// gather, then nsteps times every tile, the last time forming the populations,
+// each phase followed by the bounded barrier.  Tile b of the work list goes to
+// CTA b, further ones are claimed from the phase's counter while the one before is
+// being computed.  The moments live in the buffers the populations are not in;
+// after an even number of steps the populations belong in the buffers they
+// started in.  set_t: this launch ends the batch's step.
+template <bool FINAL>
+__device__ __forceinline__ void mom_tile(const CaseDev& cd, int par, int s, long long t, int x0, int y0, int vw, int vh,
+                                         float* smem) {
+  float* m = static_cast<float*>(cd.f[par ^ 1]);
+  float* f = static_cast<float*>(cd.f[par]);
+  float* rho = static_cast<float*>(cd.rho[par]);
+  const int a = s & 1, P = cd.mg.P;
+  const float *r = m + a * P, *j = m + (2 + 2 * a) * P;
+  float *ro = FINAL ? rho : m + (a ^ 1) * P, *jo = m + (2 + 2 * (a ^ 1)) * P;
+#define LBM_MOM_CASE(SS) \
+  case SS: mom2_tile<SS, FINAL>(cd.kp, cd.mg.LX, P, r, j, ro, jo, f, cd.bad, t, x0, y0, vw, vh, smem); break;
+  switch (cd.scheme) {
+    LBM_MOM_CASE(S_EFDS2)
+    LBM_MOM_CASE(S_EFDS4)
+    LBM_MOM_CASE(S_EFDS6)
+    LBM_MOM_CASE(S_E4)
+    LBM_MOM_CASE(S_E8)
+    default: break;
+  }
+#undef LBM_MOM_CASE
+}
+
+__global__ void __launch_bounds__(T2NT, T2_CTAS) k_batch_mom(const CaseDev* __restrict__ cases, const Item* __restrict__ tiles,
+                                                       int ntiles, int nsteps, BatchCtl* ctl,
+                                                       unsigned long long timeout_ns, int set_t) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ int s_q[2];
+  const long long t0 = *((volatile long long*)&ctl->t);
+  const int par = int(t0 & 1), w = int(threadIdx.x >> 5);
+  for (int k = 0; k <= nsteps; ++k) {  // phase 0: gather; phase k: step k - 1
+    unsigned* ctr = &ctl->work[k & 3];
+    int q = 0;
+    for (int u = int(blockIdx.x); u < ntiles; q ^= 1) {
+      // (a slot is rewritten two tiles after it was read, and every thread
+      // passes a barrier of the tile in between)
+      if (threadIdx.x == 0) s_q[q] = int(gridDim.x) + int(atomicAdd(ctr, 1u));
+      const Item itm = tiles[u];
+      const CaseDev& cd = cases[itm.c];
+      const int row = itm.tile / cd.mg.nt, x0 = (itm.tile - row * cd.mg.nt) * cd.mg.TW, y0 = row * cd.mg.TH;
+      const int vw = min(cd.mg.TW, cd.kp.nx - x0), vh = min(cd.mg.TH, cd.kp.ny - y0);
+      if (k == 0) {
+        for (int y = y0 + w; y < y0 + vh; y += T2NT / 32)
+          mom2_gather(cd.kp, cd.mg.LX, cd.mg.P, static_cast<const float*>(cd.f[par]),
+                      static_cast<const float*>(cd.rho[par]), static_cast<float*>(cd.f[par ^ 1]),
+                      static_cast<float*>(cd.f[par ^ 1]) + 2 * cd.mg.P, cd.bad, t0, x0, vw, y, y + 1);
+        __syncthreads();
+      } else if (k < nsteps) {
+        mom_tile<false>(cd, par, k - 1, t0 + k - 1, x0, y0, vw, vh, reinterpret_cast<float*>(smem));
+      } else {
+        mom_tile<true>(cd, par, k - 1, t0 + k - 1, x0, y0, vw, vh, reinterpret_cast<float*>(smem));
+      }
+      u = s_q[q];
+    }
+    if (k == nsteps) break;
+    if (blockIdx.x == 0 && threadIdx.x == 0) ctl->work[(k + 2) & 3] = 0u;
+    if (!grid_barrier(ctl, timeout_ns)) return;
+  }
+  if (set_t && blockIdx.x == 0 && threadIdx.x == 0) ctl->t = t0 + nsteps;
+}
+
 // derivative fields of the compact cases for the current state (before an
 // observation pass): mu tiles, then line groups, one CTA per item
 template <class P>
@@ -591,6 +663,10 @@ struct lbm_batch {
   int buf_split = 0;  // bytes of one item buffer of the split kernel
   int rpt = 0;        // split kernel: tile rows per thread (1, 2, 4)
   int item_cap = 0;   // capacity of d_mitems and of d_citems
+  // cases on the moments: their tiles; they come first in the work lists above,
+  // nmu_mom and ncoll_mom items of them
+  Item* d_tiles = nullptr;
+  int ntiles = 0, grid_mom = 0, nmu_mom = 0, ncoll_mom = 0;
   std::vector<int> case_order;  // split path: cases in work-list order
   // compact-scheme cases: their mu tiles (TXB x TYB), their line groups
   // (rebuilt with the group size lpb of the tile shape), longest line
@@ -660,6 +736,10 @@ static int setup_split_t(lbm_batch* b) {
     const int ct = cd.ctiles_x * ((ny + T2Y - 1) / T2Y);
     for (int tl = 0; tl < mt; ++tl) mitems.push_back({c, tl});
     for (int tl = 0; tl < ct; ++tl) citems.push_back({c, tl});
+    if (cd.mom) {
+      b->nmu_mom = int(mitems.size());
+      b->ncoll_mom = int(citems.size());
+    }
   }
   if (int(mitems.size()) > b->item_cap || int(citems.size()) > b->item_cap) return LBM_ECUDA;
   cudaError_t e = cudaMemcpyAsync(b->d_mitems, mitems.data(), sizeof(Item) * mitems.size(), cudaMemcpyHostToDevice,
@@ -700,6 +780,32 @@ static int setup_split_t(lbm_batch* b) {
   if (b->gexec) { cudaGraphExecDestroy(b->gexec); b->gexec = nullptr; }
   if (b->graph) { cudaGraphDestroy(b->graph); b->graph = nullptr; }
   b->graph_steps = -1;
+  return LBM_OK;
+}
+
+// tiles of the cases on the moments, the dearest schemes' first
+static int setup_moments(lbm_batch* b) {
+  int dev = 0, sms = 0, ps = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  std::vector<Item> tiles;
+  for (const int s : {S_E8, S_EFDS6, S_E4, S_EFDS4, S_EFDS2})
+    for (const int c : b->case_order) {
+      CaseDev& cd = b->host_cases[c];
+      if (!cd.mom || cd.scheme != s) continue;
+      for (int u = 0; u < cd.mg.nt * cd.mg.nr; ++u) tiles.push_back({c, u});
+    }
+  if (tiles.empty()) return LBM_OK;
+  if (cudaFuncSetAttribute(k_batch_mom, cudaFuncAttributeMaxDynamicSharedMemorySize, T2_SMEM) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ps, k_batch_mom, T2NT, T2_SMEM) != cudaSuccess || ps < 1)
+    return LBM_ECUDA;
+  b->ntiles = int(tiles.size());
+  b->grid_mom = std::max(1, std::min(ps * sms, b->ntiles));
+  b->d_tiles = static_cast<Item*>(balloc(b, sizeof(Item) * tiles.size()));
+  if (!b->d_tiles) return LBM_ENOMEM;
+  if (cudaMemcpyAsync(b->d_tiles, tiles.data(), sizeof(Item) * tiles.size(), cudaMemcpyHostToDevice, b->stream) != cudaSuccess ||
+      cudaStreamSynchronize(b->stream) != cudaSuccess)
+    return LBM_ECUDA;
   return LBM_OK;
 }
 
@@ -776,6 +882,9 @@ extern "C" int lbm_batch_create(const lbm_params* cases, int n, void* stream, co
     ok = cd.f[0] && cd.f[1] && cd.rho[0] && cd.rho[1] && cd.snap && cd.bad && (cd.mu || prec0 != LBM_FP32DEV || mu0);
     cd.lap = cd.lci = 0;
     cd.cmu = cd.gmu = cd.grho = nullptr;
+    cd.mom = prec0 == LBM_FP32DEV && !mu0 && mom2d_ok(cd.kp, q.scheme, 1, cd.mrt.on != 0);
+    cd.mg = Mom2Geo{};
+    if (cd.mom) cd.mg = mom2_geo(cd.kp, 1);
     if (ok && q.scheme >= LBM_CFDS4 && q.scheme <= LBM_OCFDS4) {
       b->compact = true;
       cd.lap = q.scheme == LBM_CFDS6 ? 6 : (q.scheme == LBM_CFDS8 ? 8 : 4);
@@ -792,7 +901,9 @@ extern "C" int lbm_batch_create(const lbm_params* cases, int n, void* stream, co
   if (!ok) { lbm_batch_destroy(b); return LBM_ENOMEM; }
   b->nitems = int(items.size());
   b->split = prec0 == LBM_FP32DEV && !mu0;
+  std::stable_partition(idx.begin(), idx.end(), [&](int c) { return b->host_cases[c].mom != 0; });
   b->case_order.assign(idx.begin(), idx.end());
+  if (const int rm = setup_moments(b); rm != LBM_OK) { lbm_batch_destroy(b); return rm; }
   if (b->compact) {
     // the line coefficients of the four compact schemes (the same for every batch)
     LineCoef lc[2][4];
@@ -931,23 +1042,55 @@ extern "C" int lbm_batch_init_droplets(lbm_batch* b, const double* radius, doubl
   return e == cudaSuccess ? LBM_OK : LBM_ECUDA;
 }
 
+// the split kernel over all cases, or over those not on the moments
+static cudaError_t launch_split(lbm_batch* b, int nsteps, bool all) {
+  cudaLaunchConfig_t cs{};
+  cs.gridDim = dim3(unsigned(b->grid_split));
+  cs.blockDim = dim3(NT2S);
+  cs.dynamicSmemBytes = b->smem_split;
+  cs.stream = b->stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeCooperative;
+  at[0].val.cooperative = 1;
+  cs.attrs = at;
+  cs.numAttrs = 1;
+  auto kern = b->rpt == 1 ? k_batch_split<1> : (b->rpt == 4 ? k_batch_split<4> : k_batch_split<2>);
+  const int m0 = all ? 0 : b->nmu_mom, c0 = all ? 0 : b->ncoll_mom;
+  return cudaLaunchKernelEx(&cs, kern, (const CaseDev*)b->d_cases, (const Item*)b->d_mitems + m0, b->nmu - m0,
+                            (const Item*)b->d_citems + c0, b->ncoll - c0, nsteps, b->ctl, BARRIER_NS, b->buf_split,
+                            (const Item*)b->d_litems, b->nline, b->lpb, b->lpb_shift);
+}
+
+// nsteps steps of every case: on the populations in one persistent launch, or,
+// with cases that advance on their moments, an odd step on the populations, then
+// the moments' launch and the remaining cases'
 static cudaError_t launch_persistent(lbm_batch* b, int nsteps) {
-  const unsigned long long timeout_ns = 1000000000ull;
+  const unsigned long long timeout_ns = BARRIER_NS;
+  // counters and barrier state (status and skip_block are left as they are)
+  auto reset = [&] { return cudaMemsetAsync(b->ctl, 0, offsetof(BatchCtl, status), b->stream); };
+  cudaError_t e = reset();
+  if (e != cudaSuccess) return e;
   if (b->split) {
+    const int even = b->ntiles > 0 ? nsteps / 2 * 2 : 0;
+    if (nsteps - even > 0 && (e = launch_split(b, nsteps - even, true)) != cudaSuccess) return e;
+    if (even == 0) return e;
+    const bool rest = b->nmu > b->nmu_mom;
     cudaLaunchConfig_t cs{};
-    cs.gridDim = dim3(unsigned(b->grid_split));
-    cs.blockDim = dim3(NT2S);
-    cs.dynamicSmemBytes = b->smem_split;
+    cs.gridDim = dim3(unsigned(b->grid_mom));
+    cs.blockDim = dim3(T2NT);
+    cs.dynamicSmemBytes = T2_SMEM;
     cs.stream = b->stream;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeCooperative;
     at[0].val.cooperative = 1;
     cs.attrs = at;
     cs.numAttrs = 1;
-    auto kern = b->rpt == 1 ? k_batch_split<1> : (b->rpt == 4 ? k_batch_split<4> : k_batch_split<2>);
-    return cudaLaunchKernelEx(&cs, kern, (const CaseDev*)b->d_cases, (const Item*)b->d_mitems, b->nmu,
-                              (const Item*)b->d_citems, b->ncoll, nsteps, b->ctl, timeout_ns, b->buf_split,
-                              (const Item*)b->d_litems, b->nline, b->lpb, b->lpb_shift);
+    if ((e = reset()) != cudaSuccess) return e;
+    e = cudaLaunchKernelEx(&cs, k_batch_mom, (const CaseDev*)b->d_cases, (const Item*)b->d_tiles, b->ntiles, even, b->ctl,
+                           timeout_ns, rest ? 0 : 1);
+    if (e != cudaSuccess || !rest) return e;
+    if ((e = reset()) != cudaSuccess) return e;
+    return launch_split(b, even, false);
   }
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(unsigned(b->grid));
@@ -971,8 +1114,8 @@ static cudaError_t launch_persistent(lbm_batch* b, int nsteps) {
                             b->nitems, nsteps, b->ctl, timeout_ns, cmu, b->ncmu, li, b->nline, b->lpb, b->lpb_shift);
 }
 
-// n steps = one persistent launch (preceded by the reset of the barrier and
-// work counters), captured once in a CUDA graph per distinct n and replayed
+// n steps = one persistent launch, two or three with cases on their moments
+// (each preceded by the reset of the barrier and work counters), captured once in a CUDA graph per distinct n and replayed
 extern "C" int lbm_batch_step(lbm_batch* b, long long n) {
   if (!b || n < 0 || n > INT_MAX) return LBM_EINVAL;
   if (n == 0) return LBM_OK;
@@ -985,10 +1128,9 @@ extern "C" int lbm_batch_step(lbm_batch* b, long long n) {
     b->stream = cap;
     cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-      // counters and barrier state (status and skip_block are left as they are)
-      cudaMemsetAsync(b->ctl, 0, offsetof(BatchCtl, status), cap);
-      launch_persistent(b, int(n));
+      const cudaError_t el = launch_persistent(b, int(n));
       e = cudaStreamEndCapture(cap, &b->graph);
+      if (e == cudaSuccess) e = el;
     }
     b->stream = saved;
     cudaStreamDestroy(cap);
@@ -1114,8 +1256,14 @@ extern "C" int lbm_batch_get_density(lbm_batch* b, int c, double* host) {
 
 extern "C" long long lbm_batch_get_step(const lbm_batch* b) { return b ? b->t : -1; }
 
+// CTAs of the batch's launches (the smallest, where there are two kinds)
+static int resident(const lbm_batch* b) {
+  const int g = b->split ? b->grid_split : b->grid;
+  return b->ntiles > 0 ? std::min(g, b->grid_mom) : g;
+}
+
 extern "C" int lbm_batch_inject_stall(lbm_batch* b, int cta) {
-  if (!b || cta < -1 || cta >= (b->split ? b->grid_split : b->grid)) return LBM_EINVAL;
+  if (!b || cta < -1 || cta >= resident(b)) return LBM_EINVAL;
   cudaError_t e = cudaMemcpyAsync(&b->ctl->skip_block, &cta, sizeof(int), cudaMemcpyHostToDevice, b->stream);
   int zero = 0;
   if (e == cudaSuccess) e = cudaMemcpyAsync(&b->ctl->status, &zero, sizeof(int), cudaMemcpyHostToDevice, b->stream);
@@ -1127,6 +1275,6 @@ extern "C" int lbm_batch_size(const lbm_batch* b, int* ncases, int* nitems, int*
   if (!b) return LBM_EINVAL;
   if (ncases) *ncases = b->n;
   if (nitems) *nitems = (b->split ? b->nmu + b->ncoll : b->nitems + b->ncmu) + b->nline;
-  if (grid) *grid = b->split ? b->grid_split : b->grid;
+  if (grid) *grid = resident(b);
   return LBM_OK;
 }

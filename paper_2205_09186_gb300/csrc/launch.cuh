@@ -58,6 +58,12 @@ using StepFn = cudaError_t (*)(const Launch&, int mode, int* nblocks);
 bool mom3d_ok(const KParams& kp, int scheme, int prec);
 cudaError_t mom3d_steps(const Launch& c, int scheme, int prec, long long n);
 
+// the same for D2Q9 FP32DEV, explicit and isotropic schemes (mom2d.cuh)
+struct Mom2Geo;
+Mom2Geo mom2_geo(const KParams& kp, int sms);
+bool mom2d_ok(const KParams& kp, int scheme, int prec, bool mrt);
+cudaError_t mom2d_steps(const Launch& c, int scheme, long long n);
+
 // one FP64 step on node-parallel passes (fp64.cuh), explicit and isotropic
 // schemes with mu an N-double buffer, compact ones reading c.gi
 cudaError_t step64(const Launch& c, int D, int scheme, double* mu);
@@ -108,6 +114,35 @@ cudaError_t coll3d_zero_edges(const KParams& kp, const float* rin, float* rout, 
 // cudaErrorNotSupported, nothing launched.
 bool coll3d_gf_ok(const Launch& c);
 cudaError_t coll3d_gf_step(const Launch& c, int* nblocks);
+
+// Launch a kernel that begins with pdl_wait() so that its launch overlaps the
+// end of the kernel before it in the stream (programmatic dependent launch).
+// Dependent kernels of a few microseconds otherwise start on a 2 us grid here.
+template <class... P, class... A>
+inline cudaError_t launch_pdl(void (*k)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k, P(args)...);
+}
+
+#ifdef __CUDACC__
+// lets the next kernel's blocks start (they wait in turn), then waits for the
+// kernel before this one to end with its stores visible: before any access
+__device__ __forceinline__ void pdl_wait() {
+#if __CUDA_ARCH__ >= 900
+  cudaTriggerProgrammaticLaunchCompletion();
+  cudaGridDependencySynchronize();
+#endif
+}
+#endif
 
 // Raise kernel fn's dynamic shared-memory limit to at least `bytes` on the
 // current device.  The attribute belongs to one device (context): it is set

@@ -912,13 +912,17 @@ extern "C" int lbm_autotune(lbm_handle* h, int* zc_out) {
 // needed to advance it.  A call costs gather + expand once (0.63 ms at 256^3)
 // and 0.31 ms a step against 0.608 on the populations: break-even at two.
 static bool on_moments(const lbm_handle* h, long long n) {
-  return n >= 2 && h->D == 3 && h->mu && !h->compact && !h->layer && mom3d_ok(h->kp, h->p.scheme, h->prec);
+  if (n < 2 || !h->mu || h->compact || h->layer) return false;
+  return h->D == 3 ? mom3d_ok(h->kp, h->p.scheme, h->prec) : mom2d_ok(h->kp, h->p.scheme, h->prec, h->mrt.on != 0);
+}
+static cudaError_t moment_steps(lbm_handle* h, const Launch& c, long long n) {
+  return h->D == 3 ? mom3d_steps(c, h->p.scheme, h->prec, n) : mom2d_steps(c, h->p.scheme, n);
 }
 
 extern "C" int lbm_step(lbm_handle* h, long long n) {
   if (!h || n < 0) return LBM_EINVAL;
   if (on_moments(h, n)) {
-    if (mom3d_steps(make_launch(h, 1 - h->cur), h->p.scheme, h->prec, n) != cudaSuccess) return LBM_ECUDA;
+    if (moment_steps(h, make_launch(h, 1 - h->cur), n) != cudaSuccess) return LBM_ECUDA;
     h->t += n;
     return LBM_OK;
   }
@@ -956,13 +960,13 @@ extern "C" int lbm_step_timed(lbm_handle* h, long long n, double* ms) {
       Launch c = make_launch(h, 1 - h->cur);
       c.ev_mu = e;
       cudaEventRecord(ends[0], h->stream);
-      if (mom3d_steps(c, h->p.scheme, h->prec, n) != cudaSuccess) rc = LBM_ECUDA;
+      if (moment_steps(h, c, n) != cudaSuccess) rc = LBM_ECUDA;
       cudaEventRecord(ends[1], h->stream);
       h->t += n;
     }
     if (rc == LBM_OK && cudaEventSynchronize(ends[1]) != cudaSuccess) rc = LBM_ECUDA;
     float a = 0.f;
-    for (long long s = 0; s < n && rc == LBM_OK; ++s) {
+    for (long long s = 0; s < n && rc == LBM_OK && h->D == 3; ++s) {  // (D2Q9: mu is part of the march)
       cudaEventElapsedTime(&a, e[2 * s], e[2 * s + 1]);
       ms[0] += a;
     }

@@ -25,6 +25,7 @@
 // that no stencil wraps in x; what lies past them is zero.
 #pragma once
 #include "lbm_device.cuh"
+#include "pack2.cuh"
 #include "step3d_mu.cuh"
 
 namespace lbmd {
@@ -35,11 +36,6 @@ struct MomGeo {
   int TW, nt;    // columns per tile of k_mom3d (a multiple of 4, <= 64), tiles
   int RB, nb;    // rows per band, bands
 };
-
-__device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 
 // The packed constants of a step.  Kernel parameters, not literals: a packed
 // instruction takes no immediate, and the compiler otherwise builds each pair

@@ -216,6 +216,9 @@ __device__ __forceinline__ void coll2d_compute(const KParams& p, float* __restri
       }
     } else {
       const float vv15 = 1.5f * (vx * vx + vy * vy), uu15 = 1.5f * (ux * ux + uy * uy);
+      // the rest population carries drho less the others' shares (4 w1 + 4 w2 = 5
+      // w1 in floats): no drift from weights that do not sum to one
+      const float d0 = fmaf(-5.f, float(L::w(1)) * dsv, dsv);
 #pragma unroll
       for (int i = 0; i < Q; ++i) {
         const float w = float(L::w(i));
@@ -223,11 +226,12 @@ __device__ __forceinline__ void coll2d_compute(const KParams& p, float* __restri
         const float Av = i == 0 ? -vv15 : ev * (3.f + 4.5f * ev) - vv15;
         float fs;
         if constexpr (TAU1) {
-          fs = w * (dsv + rc * Av);
+          fs = i == 0 ? d0 + w * rc * Av : w * (dsv + rc * Av);
         } else {
           const float eu = edot<L>(i, ux, uy, 0.f);
           const float Au = i == 0 ? -uu15 : eu * (3.f + 4.5f * eu) - uu15;
-          fs = (1.f - omega) * fv[i] + w * (omega * dsv + rc * (omega * Au + Av - Au));
+          const float eq = rc * (omega * Au + Av - Au);
+          fs = (1.f - omega) * fv[i] + (i == 0 ? omega * d0 + w * eq : w * (omega * dsv + eq));
         }
         s_f[i * C2N + node] = fs;
         if (interior) {

@@ -467,7 +467,10 @@ __global__ void __launch_bounds__(CX* RY_, (CollShape<S, RY_, NB_, FD_>::MINB)) 
       float* fo = fout + pz * NXY + gy * nx + gx;
       const float vv15 = 1.5f * (vx * vx + vy * vy + vz * vz);
       const float uu15 = 1.5f * (ux * ux + uy * uy + uz * uz);
-      const float wd0 = float(L::w(0)) * dsv, wd1 = float(L::w(1)) * dsv, wd2 = float(L::w(7)) * dsv;
+      // the rest population carries drho less the others' shares (6 wd1 + 12 wd2,
+      // wd2 = wd1 / 2 exactly): with rounded weights the nineteen would sum to
+      // 1.0000000xx drho, a drift of 1e-8 per step
+      const float wd1 = float(L::w(1)) * dsv, wd2 = float(L::w(7)) * dsv, wd0 = fmaf(-12.f, wd1, dsv);
       const float wr0 = float(L::w(0)) * rc, wr1 = float(L::w(1)) * rc, wr2 = float(L::w(7)) * rc;
       auto post = [&](const int i) {  // post-collision population i of this node
         const float wd = i == 0 ? wd0 : (i < 7 ? wd1 : wd2);

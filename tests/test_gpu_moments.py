@@ -62,6 +62,37 @@ def test_d3q19_steps_on_moments(L, shape, scheme, mu64, steps):
     assert np.max(np.abs(a.lbm_get_density() - o.density())) / 0.15 < 1e-5
 
 
+# tiles of up to 60 columns x 30 rows, two columns per lane: 60 x 30 fills one,
+# 61 cuts into 32 + 29, odd widths end a row in half a pair, 41 nearly fills the
+# scratch, 40 is the narrowest on the moments and 33 falls back to the
+# populations; 700 rows cut into many tiles
+@pytest.mark.parametrize("shape", [(40, 8, 1), (33, 12, 1), (41, 40, 1), (60, 30, 1), (61, 31, 1), (119, 64, 1), (230, 37, 1),
+                                   (64, 700, 1)])
+@pytest.mark.parametrize("scheme,steps", [("EFDS2", 2), ("EFDS4", 3), ("EFDS6", 20), ("E4", 5), ("E8", 8)])
+def test_d2q9_steps_on_moments(L, shape, scheme, steps):
+    kw = dict(scheme=scheme, precision=L.LBM_FP32DEV)
+    (a, rho), (b, _) = start(L, L.LBM_D2Q9, shape, **kw), start(L, L.LBM_D2Q9, shape, **kw)
+    check(L, a, b, steps, 1e-6)
+    o = O.Sim(lattice=O.D2Q9, nx=shape[0], ny=shape[1], Tr=0.9, k=0.3, kappa=0.1, scheme=scheme)
+    o.set_f(np.stack([w * rho[0] for w in O.lattice(O.D2Q9)[1]]))
+    assert o.step(steps) == 0
+    assert np.max(np.abs(a.lbm_get_density() - o.density())) / 0.15 < 1e-5
+
+
+def test_moments_with_another_equation_of_state(L):
+    # the chemical potential of a node pair takes the scalar form
+    kw = dict(lattice=L.LBM_D2Q9, nx=96, ny=60, Tr=0.85, k=0.2, kappa=0.01, scheme="EFDS4", eos="PR", a=2 / 49,
+              b=2 / 21, precision=L.LBM_FP32DEV)
+    a, b = L.Sim(L.make_params(**kw)), L.Sim(L.make_params(**kw))
+    for s in (a, b):
+        s.lbm_init_droplet(14.0)
+    a.lbm_step(30)
+    for _ in range(30):
+        b.lbm_step(1)
+    ra, rb = a.lbm_get_density(), b.lbm_get_density()
+    assert np.max(np.abs(ra - rb)) / np.max(rb) < 2e-6
+
+
 def test_moments_report_the_first_bad_step(L):
     # a cold second-order droplet: the density goes non-positive within the call
     kw = dict(lattice=L.LBM_D3Q19, nx=48, ny=40, nz=36, Tr=0.3, k=0.3, kappa=0.1, scheme="EFDS2",
