@@ -21,22 +21,20 @@ cudaError_t step(const Launch& c, double* mu) {
   if constexpr (LAT == 0 && !Sch<S>::GF) {
     const dim3 t((kp.nx + T64X - 1) / T64X, (kp.ny + T64Y - 1) / T64Y);
     if ((long long)t.x * t.y <= device_sms()) {
-      if (c.mrt.on) k64_tile<S, 2><<<t, T64N, 0, c.stream>>>(kp, fin, fout, rin, rout, c.aux, c.mrt);
-      else if (kp.omega == 1.0) k64_tile<S, 0><<<t, T64N, 0, c.stream>>>(kp, fin, fout, rin, rout, c.aux, c.mrt);
-      else k64_tile<S, 1><<<t, T64N, 0, c.stream>>>(kp, fin, fout, rin, rout, c.aux, c.mrt);
-      return cudaGetLastError();
+      auto k = c.mrt.on ? k64_tile<S, 2> : (kp.omega == 1.0 ? k64_tile<S, 0> : k64_tile<S, 1>);
+      return launch_pdl(k, t, T64N, 0, c.stream, kp, fin, fout, rin, rout, c.aux, c.mrt);
     }
   }
-  if constexpr (!Sch<S>::GF) k64_mu<S, LAT><<<g, bs, 0, c.stream>>>(kp, rin, mu);
-  if (LAT == 0 && c.mrt.on) {
-    if constexpr (LAT == 0) k64_coll<S, LAT, 2><<<g, bs, 0, c.stream>>>(kp, fin, fout, rin, mu, c.gi, c.aux, c.mrt);
-  } else if (kp.omega == 1.0) {
-    k64_coll<S, LAT, 0><<<g, bs, 0, c.stream>>>(kp, fin, fout, rin, mu, c.gi, c.aux, c.mrt);
-  } else {
-    k64_coll<S, LAT, 1><<<g, bs, 0, c.stream>>>(kp, fin, fout, rin, mu, c.gi, c.aux, c.mrt);
+  cudaError_t e = cudaSuccess;
+  if constexpr (!Sch<S>::GF) e = launch_pdl(k64_mu<S, LAT>, g, bs, 0, c.stream, kp, rin, mu);
+  if (e != cudaSuccess) return e;
+  auto k = kp.omega == 1.0 ? k64_coll<S, LAT, 0> : k64_coll<S, LAT, 1>;
+  if constexpr (LAT == 0) {
+    if (c.mrt.on) k = k64_coll<S, LAT, 2>;
   }
-  k64_rho<Lattice<LAT>::Q><<<g, bs, 0, c.stream>>>(kp, fout, rout, c.aux.bad_step, c.aux.t + 1);
-  return cudaGetLastError();
+  e = launch_pdl(k, g, bs, 0, c.stream, kp, fin, fout, rin, mu, c.gi, c.aux, c.mrt);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(k64_rho<Lattice<LAT>::Q>, g, bs, 0, c.stream, kp, fout, rout, c.aux.bad_step, c.aux.t + 1);
 }
 
 }  // namespace

@@ -13,6 +13,7 @@
 // directions share their even and odd parts.  Blocks are small on small
 // lattices, whose nodes are too few to fill 152 SMs: 32 nodes per block.
 #pragma once
+#include "launch.cuh"
 #include "lbm_device.cuh"
 #include "mrt.cuh"
 #include "step2d.cuh"
@@ -98,6 +99,7 @@ __device__ __forceinline__ void grad64(const double* q, const Node64<LAT>& c, do
 
 template <int S, int LAT>
 __global__ void k64_mu(const KParams p, const double* __restrict__ rho, double* __restrict__ mu) {
+  pdl_wait();
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= int(p.n)) return;
   const Node64<LAT> c(p, n);
@@ -201,6 +203,7 @@ template <int S, int LAT, int COLL>
 __global__ void k64_coll(const KParams p, const double* __restrict__ fin, double* __restrict__ fout,
                          const double* __restrict__ rho, const double* __restrict__ mu, const GradIn gi,
                          const StepAux aux, const Mrt mrt) {
+  pdl_wait();
   using L = Lattice<LAT>;
   constexpr int Q = L::Q, D = L::D;
   const int n = blockIdx.x * blockDim.x + threadIdx.x, N = int(p.n);
@@ -233,7 +236,7 @@ __global__ void k64_coll(const KParams p, const double* __restrict__ fin, double
 // ring, next density from the ring's and the tile's populations.  For lattices
 // whose tiles find an SM each: the redundant nodes run on pipes that would idle,
 // and one launch takes the place of three.  64^2 EFDS2 takes 8.2 us a step (16.4
-// on the three passes); with two tiles per SM the pipes are shared and the passes
+// on the three passes; 6.0 with each launch overlapping the step before); with two tiles per SM the pipes are shared and the passes
 // (16.4 us at 96^2 EFDS6) are level with it.
 constexpr int T64X = 8, T64Y = 4, T64N = 128;
 
@@ -241,6 +244,7 @@ template <int S, int COLL>
 __global__ void __launch_bounds__(T64N) k64_tile(const KParams p, const double* __restrict__ fin,
                                                  double* __restrict__ fout, const double* __restrict__ rin,
                                                  double* __restrict__ rout, const StepAux aux, const Mrt mrt) {
+  pdl_wait();
   using L = Lattice<0>;
   constexpr int Q = 9, R = Sch<S>::R, H = 2 * R + 1;
   constexpr int RW = T64X + 2 * H, RH = T64Y + 2 * H, MW = T64X + 2 * R + 2, MH = T64Y + 2 * R + 2;
@@ -301,6 +305,7 @@ __global__ void __launch_bounds__(T64N) k64_tile(const KParams p, const double* 
 template <int Q>
 __global__ void k64_rho(const KParams p, const double* __restrict__ f, double* __restrict__ rho,
                         unsigned long long* bad, long long t1) {
+  pdl_wait();
   const int n = blockIdx.x * blockDim.x + threadIdx.x, N = int(p.n);
   if (n >= N) return;
   double a = 0.0;

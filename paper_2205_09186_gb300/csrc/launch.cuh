@@ -119,10 +119,10 @@ cudaError_t coll3d_gf_step(const Launch& c, int* nblocks);
 // end of the kernel before it in the stream (programmatic dependent launch).
 // Dependent kernels of a few microseconds otherwise start on a 2 us grid here.
 template <class... P, class... A>
-inline cudaError_t launch_pdl(void (*k)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args) {
+inline cudaError_t launch_pdl(void (*k)(P...), dim3 grid, dim3 threads, size_t smem, cudaStream_t st, A... args) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;
-  cfg.blockDim = dim3(threads);
+  cfg.blockDim = threads;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute at{};

@@ -46,6 +46,8 @@ struct lbm_handle {
   void* mu = nullptr;  // mu field of the split D3Q19 FP32DEV path
   double* mu64 = nullptr;  // mu field of the FP64 step (explicit and isotropic schemes)
   signed char* layer = nullptr;  // wall layers (Appendix A): 0 fluid, 1..3, 4 deeper; null: no walls
+  int* wlist = nullptr;          // nodes of layers 1, 2, 3 in turn
+  int nwlist[3] = {0, 0, 0};     // their counts
   void* wmu = nullptr;           // mu field of the wall step (N values of the precision's mu type)
   double mu_w = 0.0;             // wall chemical potential
   alignas(64) unsigned char tmap[2][128];  // D3Q19 FP32DEV: tensor maps (CUtensorMap) of f[0], f[1]
@@ -530,6 +532,9 @@ int device_sms() {
 }  // namespace lbmd
 
 static int ck(cudaError_t e) { return e == cudaSuccess ? LBM_OK : LBM_ECUDA; }
+static size_t wlist_bytes(const lbm_handle* h) {
+  return (size_t(h->nwlist[0]) + size_t(h->nwlist[1]) + size_t(h->nwlist[2])) * sizeof(int);
+}
 
 // ------------------------------------------------------------------ create/destroy
 extern "C" void lbm_destroy(lbm_handle* h) {
@@ -548,6 +553,7 @@ extern "C" void lbm_destroy(lbm_handle* h) {
   dfree(h, h->qc, size_t(h->n_qc) * 8);
   dfree(h, h->layer, size_t(h->N));
   dfree(h, h->wmu, size_t(h->N) * 8);
+  dfree(h, h->wlist, wlist_bytes(h));
   compact_free(h->cb, [&](void* p, size_t b) { dfree(h, p, b); });
   delete h;
 }
@@ -809,7 +815,7 @@ static Launch make_launch(lbm_handle* h, int out_buf) {
 // one pass of the handle's step: walls, compact line schemes or the fused kernels
 static cudaError_t run_pass(lbm_handle* h, const Launch& c, int mode, int* nb) {
   if (h->layer) {
-    WallLaunch w{c, h->layer, h->mu_w, h->wmu};
+    WallLaunch w{c, h->layer, h->mu_w, h->wmu, h->wlist, h->nwlist};
     return wall_step(w, h->D == 2 ? 0 : 1, h->p.scheme, h->prec, mode, nb);
   }
   if (h->compact) return compact_step(h->cb, c, h->D, h->p.scheme, h->prec, mode, nb);
@@ -1180,8 +1186,10 @@ extern "C" int lbm_set_solid(lbm_handle* h, const unsigned char* mask, double mu
     cudaStreamSynchronize(h->stream);
     dfree(h, h->layer, size_t(N));
     dfree(h, h->wmu, size_t(N) * 8);
+    dfree(h, h->wlist, wlist_bytes(h));
     h->layer = nullptr;
     h->wmu = nullptr;
+    h->wlist = nullptr;
     return LBM_OK;
   }
   if (!std::isfinite(mu_w)) return LBM_EINVAL;
@@ -1219,18 +1227,36 @@ extern "C" int lbm_set_solid(lbm_handle* h, const unsigned char* mask, double mu
   }
   for (auto& v : lay)
     if (v < 0) v = 4;
+  std::vector<int> list;
+  int counts[3];
+  for (int d = 1; d <= 3; ++d) {
+    const size_t before = list.size();
+    for (long long n = 0; n < N; ++n)
+      if (lay[size_t(n)] == d) list.push_back(int(n));
+    counts[d - 1] = int(list.size() - before);
+  }
+  int* wl = static_cast<int*>(dalloc(h, list.size() * sizeof(int)));
+  if (!wl) return LBM_ENOMEM;
   if (!h->layer) {
     h->layer = static_cast<signed char*>(dalloc(h, size_t(N)));
     h->wmu = dalloc(h, size_t(N) * 8);
     if (!h->layer || !h->wmu) {
       dfree(h, h->layer, size_t(N));
       dfree(h, h->wmu, size_t(N) * 8);
+      dfree(h, wl, list.size() * sizeof(int));
       h->layer = nullptr;
       h->wmu = nullptr;
       return LBM_ENOMEM;
     }
   }
+  // (earlier work on the stream may still read the list that goes)
+  if (h->wlist) cudaStreamSynchronize(h->stream);
+  dfree(h, h->wlist, wlist_bytes(h));
+  h->wlist = wl;
+  for (int d = 0; d < 3; ++d) h->nwlist[d] = counts[d];
   int rc = ck(cudaMemcpyAsync(h->layer, lay.data(), size_t(N), cudaMemcpyHostToDevice, h->stream));
+  if (rc == LBM_OK && !list.empty())
+    rc = ck(cudaMemcpyAsync(h->wlist, list.data(), list.size() * sizeof(int), cudaMemcpyHostToDevice, h->stream));
   if (rc == LBM_OK) rc = ck(cudaStreamSynchronize(h->stream));
   h->mu_w = mu_w;
   return rc;

@@ -91,10 +91,12 @@ cudaError_t steps(const Launch& c, long long n) {
   for (long long k = 0; k < n; ++k) {
     const int a = int(k & 1);
     if (c.ev_mu) cudaEventRecord(c.ev_mu[2 * k], c.stream);
-    k_mom_mu<S, M64><<<gridm, 256, 0, c.stream>>>(kp, g, r[a], mu, zm);
+    cudaError_t e = launch_pdl(k_mom_mu<S, M64>, gridm, 256, 0, c.stream, kp, g, r[a], mu, zm);
     if (c.ev_mu) cudaEventRecord(c.ev_mu[2 * k + 1], c.stream);
-    k_mom3d<S, MW3><<<grid, Sh::NT, Sh::bytes, c.stream>>>(kp, g, r[a], mu, j[a], r[a ^ 1], j[a ^ 1], c.aux.bad_step,
-                                                           c.aux.t + k, zc, mom_const<S>());
+    if (e == cudaSuccess)
+      e = launch_pdl(k_mom3d<S, MW3>, grid, Sh::NT, Sh::bytes, c.stream, kp, g, r[a], mu, j[a], r[a ^ 1], j[a ^ 1],
+                     c.aux.bad_step, c.aux.t + k, zc, mom_const<S>());
+    if (e != cudaSuccess) return e;
   }
   const int a = int((n - 1) & 1);
   k_mom_expand<S><<<int((kp.n + 255) / 256), 256, 0, c.stream>>>(

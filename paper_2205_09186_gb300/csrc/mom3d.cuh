@@ -25,6 +25,7 @@
 // that no stencil wraps in x; what lies past them is zero.
 #pragma once
 #include "lbm_device.cuh"
+#include "launch.cuh"
 #include "pack2.cuh"
 #include "step3d_mu.cuh"
 
@@ -144,6 +145,7 @@ __device__ __forceinline__ void mom_ghost(float* fld, int o, int x, int nx, floa
 template <int S, bool M64>
 __global__ void __launch_bounds__(256) k_mom_mu(const KParams p, const MomGeo g, const float* __restrict__ rin,
                                                 float* __restrict__ mu, const int zc) {
+  pdl_wait();
   constexpr int R = Sch<S>::R;
   const int nx4 = (p.nx + 3) >> 2;
   const int c = blockIdx.x * 256 + threadIdx.x;
@@ -297,6 +299,7 @@ __global__ void __launch_bounds__(32 * W, 1) k_mom3d(const KParams p, const MomG
   const float ex = esec ? 0.f : 1.f, ey = esec ? 1.f : 0.f, sg = lane == 0 ? 1.f : -1.f;
   const bool gh = gx0 < 4 || gx0 + 1 >= nx - 4;  // rho goes beside the row too
 
+  pdl_wait();
   // planes pc0 - R .. pc0 + R (one group), then pc0 + R + 1
   for (int q = pc0 - R; q <= pc0 + R; ++q) issue(q, (q - (pc0 - R)) * Sh::plane);
   cpa_commit();

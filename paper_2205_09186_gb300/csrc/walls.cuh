@@ -11,6 +11,8 @@ struct WallLaunch {
   const signed char* layer;
   double mu_w;
   void* mu;
+  const int* list;   // nodes of layer 1, then 2, then 3
+  const int* nlist;  // their counts (host)
 };
 
 // wall densities only (layers 1..3 of c.rin, in place)

@@ -188,3 +188,25 @@ def test_scattered_obstacles_on_ragged_lattices(L, lattice, shape, scheme, preci
     g.lbm_set_solid(mask, mu_sat())
     o.set_solid(mask, mu_sat())
     compare(g, o, mask, tol, steps)
+
+
+# layers of more than 4096 nodes are filled by a launch each, smaller ones by one
+# CTA: 2 x 2100 nodes a layer on a flat wall of a wide lattice (and, 7 rows high,
+# wall layers from both sides meeting in the middle)
+@pytest.mark.parametrize("rows", [4, 7])
+@pytest.mark.parametrize("precision,tol", [(0, 1e-12), (1, 1e-5)])
+def test_wide_walls_d2q9(L, rows, precision, tol):
+    shape = (24, 2100)
+    g, o = pair(L, 2, shape, "EFDS6", precision)
+    g.lbm_init_droplet(6.0, center=[700.0, rows + 4.0, 0.0])
+    o.init_droplet(6.0, center=[700.0, rows + 4.0, 0.0])
+    mask = flat_wall(shape, rows)
+    g.lbm_set_solid(mask, mu_sat() - 0.01)
+    o.set_solid(mask, mu_sat() - 0.01)
+    compare(g, o, mask, tol, 12)
+    # a second wall on the same handle replaces the lists
+    mask2 = flat_wall(shape, 3)
+    for s in (g, o):
+        (s.lbm_init_droplet if s is g else s.init_droplet)(6.0, center=[700.0, 7.0, 0.0])
+        (s.lbm_set_solid if s is g else s.set_solid)(mask2, mu_sat())
+    compare(g, o, mask2, tol, 8)
