@@ -8,6 +8,7 @@
 
 #include "compact.cuh"
 #include "compact_dev.cuh"
+#include "iir.cuh"
 #include "step2d.cuh"
 #include "step3d.cuh"
 
@@ -439,7 +440,7 @@ cudaError_t launch_gf(const Launch& c, int D, int* nblocks) {
 }
 
 template <class P>
-cudaError_t step_prec(const CompactBufs& cb, Launch c, int D, int mode, int* nblocks) {
+cudaError_t step_prec(const CompactBufs& cb, Launch c, int D, int scheme, int mode, int* nblocks) {
   using Tm = typename P::Tm;
   using Tc = typename P::Tc;
   using Tr = typename P::Tr;
@@ -501,6 +502,16 @@ cudaError_t step_prec(const CompactBufs& cb, Launch c, int D, int mode, int* nbl
     if (forked) cudaStreamWaitEvent(c.stream, cb.join, 0);
     return e;
   }
+  if constexpr (std::is_same<P, PrecF64>::value) {
+    // steps take F / rho straight from the recursions, in the place of grad mu
+    if (mode == MODE_STEP && iir_ok(kp)) {
+      const IirGeo ig{kp.nx, kp.ny, kp.nz, kp.nx, kp.nx * kp.ny, 0, int(kp.n)};
+      if ((e = iir_acc(ig, scheme, rin, mu, gmu, 0.0, c.stream)) != cudaSuccess) return e;
+      c.gi.gmu = gmu;
+      c.gi.grho = nullptr;
+      return step64(c, D, S_CFDS4, nullptr);
+    }
+  }
   bool lines_done = false;
   if constexpr (std::is_same<P, PrecF32>::value) {
     if (forked) {
@@ -542,10 +553,9 @@ cudaError_t step_prec(const CompactBufs& cb, Launch c, int D, int mode, int* nbl
 }  // namespace
 
 cudaError_t compact_step(const CompactBufs& cb, Launch c, int D, int scheme, int prec, int mode, int* nblocks) {
-  (void)scheme;
-  if (prec == 0) return step_prec<PrecF64>(cb, c, D, mode, nblocks);
-  if (prec == 1) return step_prec<PrecF32>(cb, c, D, mode, nblocks);
-  return step_prec<PrecF32M64>(cb, c, D, mode, nblocks);
+  if (prec == 0) return step_prec<PrecF64>(cb, c, D, scheme, mode, nblocks);
+  if (prec == 1) return step_prec<PrecF32>(cb, c, D, scheme, mode, nblocks);
+  return step_prec<PrecF32M64>(cb, c, D, scheme, mode, nblocks);
 }
 
 }  // namespace lbmd

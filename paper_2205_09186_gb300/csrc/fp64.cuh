@@ -197,8 +197,8 @@ __device__ __forceinline__ void post64(const KParams& p, const Mrt& mrt, const d
   }
 }
 
-// A compact scheme (GF) reads grad mu and grad rho from gi, the others take
-// them from rho and mu.
+// A compact scheme (GF) reads grad mu and grad rho from gi, or F / rho from gi.gmu
+// where gi.grho is null; the others take them from rho and mu.
 template <int S, int LAT, int COLL>
 __global__ void k64_coll(const KParams p, const double* __restrict__ fin, double* __restrict__ fout,
                          const double* __restrict__ rho, const double* __restrict__ mu, const GradIn gi,
@@ -218,8 +218,8 @@ __global__ void k64_coll(const KParams p, const double* __restrict__ fin, double
     const double *a = static_cast<const double*>(gi.gmu), *b = static_cast<const double*>(gi.grho);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      gm[k] = k < D ? a[k * N + n] : 0.0;
-      gr[k] = k < D ? b[k * N + n] : 0.0;
+      gm[k] = k < D ? (b ? a[k * N + n] : -a[k * N + n]) : 0.0;
+      gr[k] = k < D && b ? b[k * N + n] : 0.0;
     }
   } else {
     grad64<S, LAT>(mu, c, gm);

@@ -51,7 +51,7 @@ int fast_zchunk_heuristic(const KParams& kp, int R);
 // field dump (MODE_FIELDS); returns the number of CTAs through *nblocks
 using StepFn = cudaError_t (*)(const Launch&, int mode, int* nblocks);
 
-// n >= 2 steps of the D3Q19 FP32DEV explicit line schemes at tau = 1 on the
+// n >= 2 steps of the D3Q19 FP32DEV line schemes, explicit or compact, at tau = 1 on the
 // moments rho, j (mom3d.cuh): from the populations and density fin, rin back
 // into the same buffers; fout is scratch.  mom3d_ok: whether the case and the
 // scratch (19 N floats) allow it.
@@ -63,6 +63,14 @@ struct Mom2Geo;
 Mom2Geo mom2_geo(const KParams& kp, int sms);
 bool mom2d_ok(const KParams& kp, int scheme, int prec, bool mrt);
 cudaError_t mom2d_steps(const Launch& c, int scheme, long long n);
+
+// F / rho of the compact schemes along every axis (iir.cuh) into out's component
+// fields; lines of at most 512 nodes (iir_ok)
+struct IirGeo;
+bool iir_ok(const KParams& kp);
+cudaError_t iir_acc(const IirGeo& g, int scheme, const float* rho, const float* mu, float* out, float rref, cudaStream_t st);
+cudaError_t iir_acc(const IirGeo& g, int scheme, const double* rho, const double* mu, double* out, double rref,
+                    cudaStream_t st);
 
 // one FP64 step on node-parallel passes (fp64.cuh), explicit and isotropic
 // schemes with mu an N-double buffer, compact ones reading c.gi

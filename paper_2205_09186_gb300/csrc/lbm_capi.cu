@@ -918,7 +918,7 @@ extern "C" int lbm_autotune(lbm_handle* h, int* zc_out) {
 // needed to advance it.  A call costs gather + expand once (0.63 ms at 256^3)
 // and 0.31 ms a step against 0.608 on the populations: break-even at two.
 static bool on_moments(const lbm_handle* h, long long n) {
-  if (n < 2 || !h->mu || h->compact || h->layer) return false;
+  if (n < 2 || (!h->mu && !h->compact) || h->layer || (h->compact && h->D == 2)) return false;
   return h->D == 3 ? mom3d_ok(h->kp, h->p.scheme, h->prec) : mom2d_ok(h->kp, h->p.scheme, h->prec, h->mrt.on != 0);
 }
 static cudaError_t moment_steps(lbm_handle* h, const Launch& c, long long n) {

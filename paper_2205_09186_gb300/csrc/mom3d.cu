@@ -1,7 +1,8 @@
 // Launchers of the moment steps (mom3d.cuh): D3Q19, FP32 deviations, tau = 1,
-// explicit line schemes.
+// explicit line schemes and (with the accelerations of iir.cuh) compact ones.
 #include <algorithm>
 
+#include "iir.cuh"
 #include "launch.cuh"
 #include "mom3d.cuh"
 
@@ -9,10 +10,7 @@ namespace lbmd {
 
 namespace {
 
-#ifndef MOM_W
-#define MOM_W 16
-#endif
-constexpr int MW3 = MOM_W;  // warps of a k_mom3d CTA
+constexpr int MW3 = 16;  // warps of a CTA, one CTA per SM
 
 // columns per tile: the fewest tiles of at most 64 columns, evenly cut, none
 // narrower than four columns (a row's two edge nodes then lie in two lanes)
@@ -42,7 +40,7 @@ void mom_cut(const KParams& kp, MomGeo* g, int* zc) {
     if (2 * rb < MW3 - 3 && best < 1e300) break;
     for (int n = 1; n <= kp.nz; ++n) {
       const int c = fixed > 0 ? fixed : (kp.nz + n - 1) / n;
-      if (c < 4 && n > 1) break;
+      if (c < 2 && n > 1) break;
       const long long ctas = (long long)g->nt * bands * ((kp.nz + c - 1) / c);
       const double cost = double((ctas + slots - 1) / slots) * (c + 4) * (rb + 7);
       if (cost < best - 1e-9) { best = cost; *zc = c; g->RB = rb; g->nb = bands; }
@@ -55,7 +53,7 @@ template <int S>
 MomConst mom_const() {
   auto two = [](double v) { return float2{float(v), float(v)}; };
   MomConst k{};
-  for (int m = 1; m <= Sch<S>::R; ++m) {
+  for (int m = 1; m <= Sch<S>::R && !Sch<S>::GF; ++m) {
     k.g[m - 1] = two(Sch<S>::g(m));
     k.h[m - 1] = two(Sch<S>::g(m) / 3.0);
   }
@@ -65,43 +63,57 @@ MomConst mom_const() {
   return k;
 }
 
-template <int S, bool M64>
-cudaError_t steps(const Launch& c, long long n) {
+// S: the scheme, SL: the one whose Laplacian the mu pass takes (S itself unless
+// compact, S == S_CFDS4, whose solves are those of `scheme`)
+template <int S, int SL, bool M64>
+cudaError_t steps(const Launch& c, int scheme, long long n) {
+  constexpr bool GF = Sch<S>::GF;
   const KParams& kp = c.kp;
   MomGeo g = mom_geo(kp);
   int zc = c.zc;
   mom_cut(kp, &g, &zc);
-  using Sh = MomShape<S, MW3>;
-  static_assert(Sh::bytes <= size_t(227) * 1024, "shared memory of one CTA");
-  if (cudaError_t e = ensure_smem(k_mom3d<S, MW3>, Sh::bytes); e != cudaSuccess) return e;
-  float* s = static_cast<float*>(c.fout);  // scratch: rho x 2, j x 2, mu
+  const float *fin = static_cast<const float*>(c.fin), *rin = static_cast<const float*>(c.rin);
+  float* s = static_cast<float*>(c.fout);  // scratch: rho x 2, j x 2, mu, compact: F / rho
   float* r[2] = {s, s + g.P};
   float* j[2] = {s + 2 * g.P, s + 5 * g.P};
-  float* mu = s + 8 * g.P;
+  float *mu = s + 8 * g.P, *acc = s + 9 * g.P;
   const int elems = g.PL * kp.nz;
-  k_mom_gather<<<(elems + 255) / 256, 256, 0, c.stream>>>(kp, g, static_cast<const float*>(c.fin),
-                                                          static_cast<const float*>(c.rin), r[0], j[0], r[1], mu, j[1],
-                                                          c.aux.bad_step, c.aux.t);
-  // mu pass: about eight CTAs per SM, at least eight planes each
+  k_mom_gather<<<(elems + 255) / 256, 256, 0, c.stream>>>(kp, g, fin, rin, r[0], j[0], r[1], mu, j[1], c.aux.bad_step,
+                                                          c.aux.t);
+  // mu pass: about eight CTAs per SM; at least eight planes each, down to two
+  // where that leaves SMs without a CTA (a plane is a round trip to L2)
   const int gm = ((kp.nx + 3) / 4 * kp.ny + 255) / 256;
-  const int nz8 = std::max(1, std::min((8 * device_sms() + gm - 1) / gm, (kp.nz + 7) / 8));
-  const int zm = (kp.nz + nz8 - 1) / nz8;
+  const int least = std::max(2, std::min(8, int((long long)gm * kp.nz / (2 * device_sms()))));
+  const int nzm = std::max(1, std::min((8 * device_sms() + gm - 1) / gm, (kp.nz + least - 1) / least));
+  const int zm = (kp.nz + nzm - 1) / nzm;
   const dim3 gridm(gm, (kp.nz + zm - 1) / zm);
   const dim3 grid(g.nt, g.nb, (kp.nz + zc - 1) / zc);
+  const IirGeo ig{kp.nx, kp.ny, kp.nz, g.LX, g.PL, 4, g.P};
   for (long long k = 0; k < n; ++k) {
     const int a = int(k & 1);
     if (c.ev_mu) cudaEventRecord(c.ev_mu[2 * k], c.stream);
-    cudaError_t e = launch_pdl(k_mom_mu<S, M64>, gridm, 256, 0, c.stream, kp, g, r[a], mu, zm);
+    cudaError_t e = launch_pdl(k_mom_mu<SL, M64>, gridm, 256, 0, c.stream, kp, g, r[a], mu, zm);
     if (c.ev_mu) cudaEventRecord(c.ev_mu[2 * k + 1], c.stream);
-    if (e == cudaSuccess)
-      e = launch_pdl(k_mom3d<S, MW3>, grid, Sh::NT, Sh::bytes, c.stream, kp, g, r[a], mu, j[a], r[a ^ 1], j[a ^ 1],
-                     c.aux.bad_step, c.aux.t + k, zc, mom_const<S>());
+    if constexpr (GF) {
+      constexpr size_t smem = size_t(2) * (MomCell<MW3>::XB + MomCell<MW3>::EB) * 4;
+      if (e == cudaSuccess) e = iir_acc(ig, scheme, r[a], mu, acc, float(kp.rho_ref), c.stream);
+      if (e == cudaSuccess) e = ensure_smem(k_mom3d_acc<MW3>, smem);
+      if (e == cudaSuccess)
+        e = launch_pdl(k_mom3d_acc<MW3>, grid, 32 * MW3, smem, c.stream, kp, g, r[a], acc, j[a], r[a ^ 1], j[a ^ 1],
+                       c.aux.bad_step, c.aux.t + k, zc, mom_const<S>());
+    } else {
+      using Sh = MomShape<S, MW3>;
+      static_assert(Sh::bytes <= size_t(227) * 1024, "shared memory of one CTA");
+      if (e == cudaSuccess) e = ensure_smem(k_mom3d<S, MW3>, Sh::bytes);
+      if (e == cudaSuccess)
+        e = launch_pdl(k_mom3d<S, MW3>, grid, Sh::NT, Sh::bytes, c.stream, kp, g, r[a], mu, j[a], r[a ^ 1], j[a ^ 1],
+                       c.aux.bad_step, c.aux.t + k, zc, mom_const<S>());
+    }
     if (e != cudaSuccess) return e;
   }
   const int a = int((n - 1) & 1);
-  k_mom_expand<S><<<int((kp.n + 255) / 256), 256, 0, c.stream>>>(
-      kp, g, r[a], mu, j[a], r[a ^ 1], const_cast<float*>(static_cast<const float*>(c.fin)),
-      const_cast<float*>(static_cast<const float*>(c.rin)));
+  k_mom_expand<S><<<int((kp.n + 255) / 256), 256, 0, c.stream>>>(kp, g, r[a], GF ? acc : mu, j[a], r[a ^ 1],
+                                                                 const_cast<float*>(fin), const_cast<float*>(rin));
   return cudaGetLastError();
 }
 
@@ -109,16 +121,26 @@ cudaError_t steps(const Launch& c, long long n) {
 
 bool mom3d_ok(const KParams& kp, int scheme, int prec) {
   if ((prec != 1 && prec != 2) || kp.omega != 1.0) return false;
-  if (scheme != S_EFDS2 && scheme != S_EFDS4 && scheme != S_EFDS6) return false;
+  const bool compact = scheme >= S_CFDS4 && scheme <= S_OCFDS4;
+  if (!compact && scheme != S_EFDS2 && scheme != S_EFDS4 && scheme != S_EFDS6) return false;
+  if (compact && (prec != 1 || !iir_ok(kp))) return false;
   const long long LX = (kp.nx + 3) / 4 * 4 + 8, P = (LX * kp.ny * kp.nz + 63) / 64 * 64;
-  return 9 * P <= 19 * kp.n && 19 * kp.n < (1LL << 31);
+  return (compact ? 12 : 9) * P <= 19 * kp.n && 19 * kp.n < (1LL << 31);
 }
 
 cudaError_t mom3d_steps(const Launch& c, int scheme, int prec, long long n) {
   switch (scheme) {
-    case S_EFDS2: return prec == 2 ? steps<S_EFDS2, true>(c, n) : steps<S_EFDS2, false>(c, n);
-    case S_EFDS4: return prec == 2 ? steps<S_EFDS4, true>(c, n) : steps<S_EFDS4, false>(c, n);
-    case S_EFDS6: return prec == 2 ? steps<S_EFDS6, true>(c, n) : steps<S_EFDS6, false>(c, n);
+    case S_EFDS2:
+      return prec == 2 ? steps<S_EFDS2, S_EFDS2, true>(c, scheme, n) : steps<S_EFDS2, S_EFDS2, false>(c, scheme, n);
+    case S_EFDS4:
+      return prec == 2 ? steps<S_EFDS4, S_EFDS4, true>(c, scheme, n) : steps<S_EFDS4, S_EFDS4, false>(c, scheme, n);
+    case S_EFDS6:
+      return prec == 2 ? steps<S_EFDS6, S_EFDS6, true>(c, scheme, n) : steps<S_EFDS6, S_EFDS6, false>(c, scheme, n);
+    // compact schemes: the Laplacian of their order (Sec. 2.3)
+    case S_CFDS4:
+    case S_OCFDS4: return steps<S_CFDS4, S_EFDS4, false>(c, scheme, n);
+    case S_CFDS6: return steps<S_CFDS4, S_EFDS6, false>(c, scheme, n);
+    case S_CFDS8: return steps<S_CFDS4, S_LAP8, false>(c, scheme, n);
     default: return cudaErrorNotSupported;
   }
 }

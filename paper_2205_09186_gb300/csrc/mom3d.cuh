@@ -31,6 +31,18 @@
 
 namespace lbmd {
 
+// the mu pass of CFDS8: central second derivative of order eight (Sec. 2.3)
+constexpr int S_LAP8 = 16;
+template <>
+struct Sch<S_LAP8> {
+  static constexpr int R = 4;
+  static constexpr bool ISO = false, GF = false;
+  __host__ __device__ static constexpr double g(int) { return 0.0; }
+  __host__ __device__ static constexpr double l(int m) {
+    return m == 0 ? -205.0 / 72.0 : (m == 1 ? 1.6 : (m == 2 ? -0.2 : (m == 3 ? 8.0 / 315.0 : -1.0 / 560.0)));
+  }
+};
+
 struct MomGeo {
   int LX, PL;    // row and plane strides
   int P;         // field stride (floats)
@@ -236,224 +248,132 @@ struct MomShape {
   static constexpr int KC = (GH * (GW / 4) + NT - 1) / NT;
 };
 
-template <int S, int W>
-__global__ void __launch_bounds__(32 * W, 1) k_mom3d(const KParams p, const MomGeo g, const float* __restrict__ rin,
-                                                     const float* __restrict__ muf, const float* __restrict__ jin,
-                                                     float* __restrict__ rout, float* __restrict__ jout,
-                                                     unsigned long long* bad, const long long t, const int zc,
-                                                     const __grid_constant__ MomConst kc) {
-  using Sh = MomShape<S, W>;
-  constexpr int R = Sh::R, GW = Sh::GW, NS = Sh::NS, ROWS = Sh::ROWS, NT = Sh::NT;
-  extern __shared__ __align__(16) float sm_mom[];
-  constexpr int FLD = NS * Sh::plane;           // floats of one field's ring
-  float* s_x = sm_mom + 2 * FLD;
-  float* s_e = s_x + 2 * Sh::XB;
-  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const int nx = p.nx, ny = p.ny, nz = p.nz, LX = g.LX, PL = g.PL;
-  const int x0 = blockIdx.x * g.TW, y0 = blockIdx.y * g.RB;
-  const int VW = min(g.TW, nx - x0), VH = min(g.RB, ny - y0);
-  const int z0 = blockIdx.z * zc, z1 = min(z0 + zc, nz);
-  const int pc0 = z0 - 1, pc1 = z1;
-  for (int k = tid; k < 2 * FLD; k += NT) sm_mom[k] = 0.f;
-  __syncthreads();
-  // staging: each thread's chunks of a plane (rows y0 - 1 - R .., columns x0 - 4 ..)
-  int soff[Sh::KC];
-  unsigned goff[Sh::KC];
-#pragma unroll
-  for (int k = 0; k < Sh::KC; ++k) {
-    const int e = tid + k * NT, ry = e / (GW / 4), cj = 4 * (e - ry * (GW / 4));
-    const bool in = ry < VH + 2 + 2 * R && x0 + cj + 4 <= LX;
-    soff[k] = in ? ry * GW + cj : -1;
-    goff[k] = in ? wrapn(y0 - 1 - R + ry, ny) * LX + x0 + cj : 0;
-  }
-  auto issue = [&](int q, int slot) {  // slot: offset of the ring slot
-    if (q <= pc1 + R) {
-      const unsigned zo = wrapi(q, nz) * PL;
-#pragma unroll
-      for (int k = 0; k < Sh::KC; ++k)
-        if (soff[k] >= 0) {
-          cpa16(sm_mom + slot + soff[k], rin + (zo + goff[k]));
-          cpa16(sm_mom + FLD + slot + soff[k], muf + (zo + goff[k]));
-        }
-    }
-  };
+// What a thread of the moment step holds and does once F and v of its two nodes
+// are known: spread() forms their populations and hands on what leaves, collect()
+// (behind a CTA barrier) adds up what arrives and stores the plane before.
+template <int W>
+struct MomCell {
+  static constexpr int ROWS = W - 1, XB = 8 * ROWS * 64, EB = 5 * 2 * ROWS, XK = ROWS * 32;
   // main warps: row w (0: the one below the band), columns 2 lane and 2 lane +
   // 1; the last warp: lane r holds row r's columns beyond the tile (x: left, y: right)
-  const bool edge = w == ROWS;
-  const int row = edge ? min(lane, VH + 1) : w;
-  const bool live = edge || w <= VH + 1;       // a row that is collided
-  const bool tgt = !edge && w >= 1 && w <= VH; // a row of the band
-  const unsigned gy = wrapn(y0 - 1 + row, ny) * LX + 4;
-  const int sc0 = edge ? 3 : 4 + 2 * lane;     // first node's column in a staged row
-  const int dsc = edge ? 1 + VW : 1;           // to the second node's
-  const int gx0 = edge ? (x0 == 0 ? nx - 1 : x0 - 1) : x0 + 2 * lane;
-  const int gx1 = edge ? (x0 + VW == nx ? 0 : x0 + VW) : gx0 + 1;
-  const bool in0 = edge || 2 * lane < VW, in1 = edge || 2 * lane + 1 < VW;
-  const float2 mask = make_float2(in0 ? 1.f : 0.f, in1 ? 1.f : 0.f);
-  const float mL = lane == 0 ? 0.f : 1.f, mR = lane == 31 ? 0.f : 1.f;  // what arrives by shuffle
-  const float rref = float(p.rho_ref);
-  // the edge lanes of a row take the populations of the columns beyond: the
-  // first lane into its first node, lane rl into the tile's last node
-  const int rl = (VW - 1) >> 1;
-  const bool elane = lane == 0 || lane == rl, esec = lane != 0 && ((VW - 1) & 1) != 0;
-  const float ex = esec ? 0.f : 1.f, ey = esec ? 1.f : 0.f, sg = lane == 0 ? 1.f : -1.f;
-  const bool gh = gx0 < 4 || gx0 + 1 >= nx - 4;  // rho goes beside the row too
+  int lane, w, VW, VH, row, gx0, gx1;
+  bool edge, live, tgt;  // live: a row that is collided; tgt: a row of the band
+  bool in0, in1, elane, gh, ok;
+  unsigned gy, oj0, oj1;
+  float2 mask;
+  float mL, mR, ex, ey, sg;
+  float2 *xw;  // this row's exchange values
+  float* ew;
+  float2 R0, X0, Sp, Xp, Sm, Xm;
+  float2 aR, aX, aY, aZ;  // target plane pc - 1
+  float2 bS, bX, bY;      // target plane pc: from plane pc - 1
 
-  pdl_wait();
-  // planes pc0 - R .. pc0 + R (one group), then pc0 + R + 1
-  for (int q = pc0 - R; q <= pc0 + R; ++q) issue(q, (q - (pc0 - R)) * Sh::plane);
-  cpa_commit();
-  issue(pc0 + R + 1, (2 * R + 1) * Sh::plane);
-  cpa_commit();
-  int si = (2 * R + 2) * Sh::plane;  // slot of the next plane issued
-  const int smine = (row + R) * GW + sc0;
-  int so[2 * R + 1];  // this thread's first node in planes pc - R .. pc + R
-#pragma unroll
-  for (int d = 0; d <= 2 * R; ++d) so[d] = d * Sh::plane + smine;
-  const float *j1 = jin + g.P, *j2 = jin + 2 * g.P;
-  float *q1 = jout + g.P, *q2 = jout + 2 * g.P;
-  float2 jn[3];
-  const unsigned oj0 = gy + gx0, oj1 = gy + gx1;
-  auto ldj = [&](int pc) {
-    const unsigned zo = wrapi(pc, nz) * PL;
-    if (edge) {
-      jn[0] = make_float2(__ldg(jin + (zo + oj0)), __ldg(jin + (zo + oj1)));
-      jn[1] = make_float2(__ldg(j1 + (zo + oj0)), __ldg(j1 + (zo + oj1)));
-      jn[2] = make_float2(__ldg(j2 + (zo + oj0)), __ldg(j2 + (zo + oj1)));
-    } else if (in0) {
-      jn[0] = __ldg(reinterpret_cast<const float2*>(jin + (zo + oj0)));
-      jn[1] = __ldg(reinterpret_cast<const float2*>(j1 + (zo + oj0)));
-      jn[2] = __ldg(reinterpret_cast<const float2*>(j2 + (zo + oj0)));
-    }
-  };
-  jn[0] = jn[1] = jn[2] = f2(0.f);
-  if (live) ldj(pc0);
-  cpa_wait_n<1>();
-  __syncthreads();
-  float2 aR = f2(0.f), aX = aR, aY = aR, aZ = aR;  // target plane pc - 1
-  float2 bS = aR, bX = aR, bY = aR;                // target plane pc: from plane pc - 1
-  bool ok = true;
-  float2* xw = reinterpret_cast<float2*>(s_x) + row * 32 + lane;  // this row's exchange values
-  float* ew = s_e + (edge ? row : (lane == 0 ? 0 : ROWS) + row);
-  constexpr int XK = ROWS * 32;
-  for (int pc = pc0; pc <= pc1; ++pc) {
-    issue(pc + R + 2, si);
-    cpa_commit();
-    si = si == (NS - 1) * Sh::plane ? 0 : si + Sh::plane;
-    float2 R0, X0, Sp, Xp, Sm, Xm;
-    if (live) {
-      // F_a = rho_a / 3 - rho mu_a (Eq. 12), the third folded into the stencil of rho
-      float2 gr[3], gm[3], d;
-      auto sub = [&](float2 a, float2 b) { return fma2(kc.m1, b, a); };
-      if (!edge) {
-        auto two = [&](int o) { return *reinterpret_cast<const float2*>(sm_mom + o); };
-        auto grad = [&](int f, const float2* s, float2* o, float2& mid) {
-          const float2 b = two(so[R] + f - 2), c = two(so[R] + f), e = two(so[R] + f + 2);
-          mid = c;
-          o[0] = mul2(s[0], make_float2(c.y - b.y, e.x - c.x));
-          if constexpr (R >= 2) o[0] = fma2(s[1], sub(e, b), o[0]);
-          if constexpr (R >= 3) {
-            const float2 a = two(so[R] + f - 4), h = two(so[R] + f + 4);
-            o[0] = fma2(s[2], make_float2(e.y - a.y, h.x - b.x), o[0]);
-          }
-          o[1] = mul2(s[0], sub(two(so[R] + f + GW), two(so[R] + f - GW)));
-          o[2] = mul2(s[0], sub(two(so[R + 1] + f), two(so[R - 1] + f)));
-#pragma unroll
-          for (int m = 2; m <= R; ++m) {
-            o[1] = fma2(s[m - 1], sub(two(so[R] + f + m * GW), two(so[R] + f - m * GW)), o[1]);
-            o[2] = fma2(s[m - 1], sub(two(so[R + m] + f), two(so[R - m] + f)), o[2]);
-          }
-        };
-        grad(FLD, kc.g, gm, d);
-        grad(0, kc.h, gr, d);
-      } else {
-        auto two = [&](int o) { return make_float2(sm_mom[o], sm_mom[o + dsc]); };
-        auto grad = [&](int f, const float2* s, float2* o, float2& mid) {
-          mid = two(so[R] + f);
-          o[0] = o[1] = o[2] = f2(0.f);
-#pragma unroll
-          for (int m = 1; m <= R; ++m) {
-            o[0] = fma2(s[m - 1], sub(two(so[R] + f + m), two(so[R] + f - m)), o[0]);
-            o[1] = fma2(s[m - 1], sub(two(so[R] + f + m * GW), two(so[R] + f - m * GW)), o[1]);
-            o[2] = fma2(s[m - 1], sub(two(so[R + m] + f), two(so[R - m] + f)), o[2]);
-          }
-        };
-        grad(FLD, kc.g, gm, d);
-        grad(0, kc.h, gr, d);
+  __device__ __forceinline__ MomCell(const KParams& p, const MomGeo& g, float* s_x, float* s_e) {
+    const int nx = p.nx, ny = p.ny, x0 = blockIdx.x * g.TW, y0 = blockIdx.y * g.RB;
+    lane = threadIdx.x & 31;
+    w = threadIdx.x >> 5;
+    VW = min(g.TW, nx - x0);
+    VH = min(g.RB, ny - y0);
+    edge = w == ROWS;
+    row = edge ? min(lane, VH + 1) : w;
+    live = edge || w <= VH + 1;
+    tgt = !edge && w >= 1 && w <= VH;
+    gy = wrapn(y0 - 1 + row, ny) * g.LX + 4;
+    gx0 = edge ? (x0 == 0 ? nx - 1 : x0 - 1) : x0 + 2 * lane;
+    gx1 = edge ? (x0 + VW == nx ? 0 : x0 + VW) : gx0 + 1;
+    oj0 = gy + gx0;
+    oj1 = gy + gx1;
+    in0 = edge || 2 * lane < VW;
+    in1 = edge || 2 * lane + 1 < VW;
+    mask = make_float2(in0 ? 1.f : 0.f, in1 ? 1.f : 0.f);
+    mL = lane == 0 ? 0.f : 1.f;  // what arrives by shuffle
+    mR = lane == 31 ? 0.f : 1.f;
+    // the edge lanes of a row take the populations of the columns beyond: the
+    // first lane into its first node, lane rl into the tile's last node
+    const int rl = (VW - 1) >> 1;
+    elane = lane == 0 || lane == rl;
+    const bool esec = lane != 0 && ((VW - 1) & 1) != 0;
+    ex = esec ? 0.f : 1.f;
+    ey = esec ? 1.f : 0.f;
+    sg = lane == 0 ? 1.f : -1.f;
+    gh = gx0 < 4 || gx0 + 1 >= nx - 4;  // rho goes beside the row too
+    ok = true;
+    xw = reinterpret_cast<float2*>(s_x) + row * 32 + lane;
+    ew = s_e + (edge ? row : (lane == 0 ? 0 : ROWS) + row);
+    aR = aX = aY = aZ = bS = bX = bY = f2(0.f);
+  }
+  // two nodes of a field at offset zo of a plane
+  __device__ __forceinline__ float2 load(const float* q, unsigned zo) const {
+    if (edge) return make_float2(__ldg(q + (zo + oj0)), __ldg(q + (zo + oj1)));
+    return in0 ? __ldg(reinterpret_cast<const float2*>(q + (zo + oj0))) : f2(0.f);
+  }
+  __device__ __forceinline__ void spread(const MomConst& kc, float2 d, float2 r, float2 vx, float2 vy, float2 vz) {
+    auto sub = [&](float2 a, float2 b) { return fma2(kc.m1, b, a); };
+    const float2 dm = mul2(d, mask), rm = mul2(r, mask);
+    const Post2 ps(kc, dm, rm, vx, vy, vz);
+    float2 f7, f8, f9, f10;
+    ps.diag(add2(vx, vy), f7, f8);
+    ps.diag(sub(vx, vy), f9, f10);
+    if (!edge) {
+      // the sum and the difference of a right-moving and a left-moving
+      // population at their targets in the row (nothing enters at the row's
+      // ends: that comes from the edge warp); scalar, since the shifted
+      // halves lie in two pairs
+      auto meet = [&](float2 a, float2 b, float2& s, float2& f) {
+        const float qa = __shfl_up_sync(0xffffffffu, a.y, 1), qb = __shfl_down_sync(0xffffffffu, b.x, 1);
+        s = make_float2(fmaf(qa, mL, b.y), fmaf(qb, mR, a.x));
+        f = make_float2(fmaf(qa, mL, -b.y), fmaf(qb, -mR, a.x));
+      };
+      float2 s, f;
+      {
+        float2 f3, f4;
+        ps.axis(vy, f3, f4);
+        meet(f7, f10, s, f);
+        xw[0] = add2(f3, s);
+        xw[XK] = f;
+        meet(f9, f8, s, f);
+        xw[4 * XK] = add2(f4, s);
+        xw[5 * XK] = f;
       }
-      const float2 r = add2(f2(rref), d), nr2 = mul2(kc.m1, r);
-      const float2 ir = make_float2(__fdividef(1.f, r.x), __fdividef(1.f, r.y));
-      const float2 vx = mul2(add2(jn[0], fma2(nr2, gm[0], gr[0])), ir);
-      const float2 vy = mul2(add2(jn[1], fma2(nr2, gm[1], gr[1])), ir);
-      const float2 vz = mul2(add2(jn[2], fma2(nr2, gm[2], gr[2])), ir);
-      if (pc < pc1) ldj(pc + 1);
-      const float2 dm = mul2(d, mask), rm = mul2(r, mask);
-      const Post2 ps(kc, dm, rm, vx, vy, vz);
-      float2 f7, f8, f9, f10;
-      ps.diag(add2(vx, vy), f7, f8);
-      ps.diag(sub(vx, vy), f9, f10);
-      if (!edge) {
-        // the sum and the difference of a right-moving and a left-moving
-        // population at their targets in the row (nothing enters at the row's
-        // ends: that comes from the edge warp); scalar, since the shifted
-        // halves lie in two pairs
-        auto meet = [&](float2 a, float2 b, float2& s, float2& f) {
-          const float qa = __shfl_up_sync(0xffffffffu, a.y, 1), qb = __shfl_down_sync(0xffffffffu, b.x, 1);
-          s = make_float2(fmaf(qa, mL, b.y), fmaf(qb, mR, a.x));
-          f = make_float2(fmaf(qa, mL, -b.y), fmaf(qb, -mR, a.x));
-        };
-        float2 s, f;
-        {
-          float2 f3, f4;
-          ps.axis(vy, f3, f4);
-          meet(f7, f10, s, f);
-          xw[0] = add2(f3, s);
-          xw[XK] = f;
-          meet(f9, f8, s, f);
-          xw[4 * XK] = add2(f4, s);
-          xw[5 * XK] = f;
-        }
-        {
-          float2 f15, f16, f17, f18;
-          ps.diag(add2(vy, vz), f15, f16);
-          ps.diag(sub(vy, vz), f17, f18);
-          xw[2 * XK] = f15;
-          xw[3 * XK] = f17;
-          xw[6 * XK] = f18;
-          xw[7 * XK] = f16;
-        }
-        if (tgt) {
-          float2 a, b;
-          ps.axis(vx, a, b);
-          meet(a, b, s, X0);
-          R0 = add2(ps.rest(dm, rm), s);
-          float2 f11, f12, f13, f14;
-          ps.diag(add2(vx, vz), f11, f12);
-          ps.diag(sub(vx, vz), f13, f14);
-          ps.axis(vz, a, b);
-          meet(f11, f14, s, Xp);
-          Sp = add2(a, s);
-          meet(f13, f12, s, Xm);
-          Sm = add2(b, s);
-        }
-      } else if (lane <= VH + 1) {
-        // left column: the right-moving populations; right column: the left-moving ones
-        float2 f1, f2_, f11, f12, f13, f14;
-        ps.axis(vx, f1, f2_);
+      {
+        float2 f15, f16, f17, f18;
+        ps.diag(add2(vy, vz), f15, f16);
+        ps.diag(sub(vy, vz), f17, f18);
+        xw[2 * XK] = f15;
+        xw[3 * XK] = f17;
+        xw[6 * XK] = f18;
+        xw[7 * XK] = f16;
+      }
+      if (tgt) {
+        float2 a, b;
+        ps.axis(vx, a, b);
+        meet(a, b, s, X0);
+        R0 = add2(ps.rest(dm, rm), s);
+        float2 f11, f12, f13, f14;
         ps.diag(add2(vx, vz), f11, f12);
         ps.diag(sub(vx, vz), f13, f14);
-        ew[0] = f1.x;            ew[ROWS] = f2_.y;
-        ew[2 * ROWS] = f11.x;    ew[3 * ROWS] = f14.y;
-        ew[4 * ROWS] = f13.x;    ew[5 * ROWS] = f12.y;
-        ew[6 * ROWS] = f7.x;     ew[7 * ROWS] = f10.y;
-        ew[8 * ROWS] = f9.x;     ew[9 * ROWS] = f8.y;
+        ps.axis(vz, a, b);
+        meet(f11, f14, s, Xp);
+        Sp = add2(a, s);
+        meet(f13, f12, s, Xm);
+        Sm = add2(b, s);
       }
+    } else if (lane <= VH + 1) {
+      // left column: the right-moving populations; right column: the left-moving ones
+      float2 f1, f2_, f11, f12, f13, f14;
+      ps.axis(vx, f1, f2_);
+      ps.diag(add2(vx, vz), f11, f12);
+      ps.diag(sub(vx, vz), f13, f14);
+      ew[0] = f1.x;            ew[ROWS] = f2_.y;
+      ew[2 * ROWS] = f11.x;    ew[3 * ROWS] = f14.y;
+      ew[4 * ROWS] = f13.x;    ew[5 * ROWS] = f12.y;
+      ew[6 * ROWS] = f7.x;     ew[7 * ROWS] = f10.y;
+      ew[8 * ROWS] = f9.x;     ew[9 * ROWS] = f8.y;
     }
-    cpa_wait_n<1>();
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < 2 * R; ++k) so[k] = so[k + 1];
-    so[2 * R] = so[2 * R] == (NS - 1) * Sh::plane + smine ? smine : so[2 * R] + Sh::plane;
+  }
+  // plane pc's neighbours have spread; plane pc - 1 >= z0 is complete
+  __device__ __forceinline__ void collect(const MomConst& kc, int pc, int z0, int PL, int nx, float rref, float* rout,
+                                          float* jout, float* q1, float* q2) {
     if (tgt) {
       const float2 Pu = xw[-32], Qu = xw[XK - 32], u15 = xw[2 * XK - 32], u17 = xw[3 * XK - 32];
       const float2 Pd = xw[4 * XK + 32], Qd = xw[5 * XK + 32], d18 = xw[6 * XK + 32], d16 = xw[7 * XK + 32];
@@ -506,17 +426,195 @@ __global__ void __launch_bounds__(32 * W, 1) k_mom3d(const KParams p, const MomG
       bX = Xp;
       bY = Yp;
     }
-    // the other exchange buffer
-    const int par = (pc - pc0) & 1;
-    xw += par ? -Sh::XB / 2 : Sh::XB / 2;
-    ew += par ? -Sh::EB : Sh::EB;
   }
-  if (!ok) atomicMin(bad, (unsigned long long)(t + 1));
+  // the other exchange buffer (par: which one this was)
+  __device__ __forceinline__ void flip(int par) {
+    xw += par ? -XB / 2 : XB / 2;
+    ew += par ? -EB : EB;
+  }
+};
+
+template <int S, int W>
+__global__ void __launch_bounds__(32 * W, 1) k_mom3d(const KParams p, const MomGeo g, const float* __restrict__ rin,
+                                                     const float* __restrict__ muf, const float* __restrict__ jin,
+                                                     float* __restrict__ rout, float* __restrict__ jout,
+                                                     unsigned long long* bad, const long long t, const int zc,
+                                                     const __grid_constant__ MomConst kc) {
+  using Sh = MomShape<S, W>;
+  constexpr int R = Sh::R, GW = Sh::GW, NS = Sh::NS, ROWS = Sh::ROWS, NT = Sh::NT;
+  extern __shared__ __align__(16) float sm_mom[];
+  constexpr int FLD = NS * Sh::plane;           // floats of one field's ring
+  float* s_x = sm_mom + 2 * FLD;
+  float* s_e = s_x + 2 * Sh::XB;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int nx = p.nx, ny = p.ny, nz = p.nz, LX = g.LX, PL = g.PL;
+  const int x0 = blockIdx.x * g.TW, y0 = blockIdx.y * g.RB;
+  const int VW = min(g.TW, nx - x0), VH = min(g.RB, ny - y0);
+  const int z0 = blockIdx.z * zc, z1 = min(z0 + zc, nz);
+  const int pc0 = z0 - 1, pc1 = z1;
+  for (int k = tid; k < 2 * FLD; k += NT) sm_mom[k] = 0.f;
+  __syncthreads();
+  // staging: each thread's chunks of a plane (rows y0 - 1 - R .., columns x0 - 4 ..)
+  int soff[Sh::KC];
+  unsigned goff[Sh::KC];
+#pragma unroll
+  for (int k = 0; k < Sh::KC; ++k) {
+    const int e = tid + k * NT, ry = e / (GW / 4), cj = 4 * (e - ry * (GW / 4));
+    const bool in = ry < VH + 2 + 2 * R && x0 + cj + 4 <= LX;
+    soff[k] = in ? ry * GW + cj : -1;
+    goff[k] = in ? wrapn(y0 - 1 - R + ry, ny) * LX + x0 + cj : 0;
+  }
+  auto issue = [&](int q, int slot) {  // slot: offset of the ring slot
+    if (q <= pc1 + R) {
+      const unsigned zo = wrapi(q, nz) * PL;
+#pragma unroll
+      for (int k = 0; k < Sh::KC; ++k)
+        if (soff[k] >= 0) {
+          cpa16(sm_mom + slot + soff[k], rin + (zo + goff[k]));
+          cpa16(sm_mom + FLD + slot + soff[k], muf + (zo + goff[k]));
+        }
+    }
+  };
+  MomCell<W> cell(p, g, s_x, s_e);
+  const bool edge = cell.edge, live = cell.live;
+  const int sc0 = edge ? 3 : 4 + 2 * lane;     // first node's column in a staged row
+  const int dsc = edge ? 1 + VW : 1;           // to the second node's
+  const float rref = float(p.rho_ref);
+
+  pdl_wait();
+  // planes pc0 - R .. pc0 + R (one group), then pc0 + R + 1
+  for (int q = pc0 - R; q <= pc0 + R; ++q) issue(q, (q - (pc0 - R)) * Sh::plane);
+  cpa_commit();
+  issue(pc0 + R + 1, (2 * R + 1) * Sh::plane);
+  cpa_commit();
+  int si = (2 * R + 2) * Sh::plane;  // slot of the next plane issued
+  const int smine = (cell.row + R) * GW + sc0;
+  int so[2 * R + 1];  // this thread's first node in planes pc - R .. pc + R
+#pragma unroll
+  for (int d = 0; d <= 2 * R; ++d) so[d] = d * Sh::plane + smine;
+  const float *j1 = jin + g.P, *j2 = jin + 2 * g.P;
+  float *q1 = jout + g.P, *q2 = jout + 2 * g.P;
+  float2 jn[3];
+  auto ldj = [&](int pc) {
+    const unsigned zo = wrapi(pc, nz) * PL;
+    jn[0] = cell.load(jin, zo);
+    jn[1] = cell.load(j1, zo);
+    jn[2] = cell.load(j2, zo);
+  };
+  jn[0] = jn[1] = jn[2] = f2(0.f);
+  if (live) ldj(pc0);
+  cpa_wait_n<1>();
+  __syncthreads();
+  for (int pc = pc0; pc <= pc1; ++pc) {
+    issue(pc + R + 2, si);
+    cpa_commit();
+    si = si == (NS - 1) * Sh::plane ? 0 : si + Sh::plane;
+    if (live) {
+      // F_a = rho_a / 3 - rho mu_a (Eq. 12), the third folded into the stencil of rho
+      float2 gr[3], gm[3], d;
+      auto sub = [&](float2 a, float2 b) { return fma2(kc.m1, b, a); };
+      if (!edge) {
+        auto two = [&](int o) { return *reinterpret_cast<const float2*>(sm_mom + o); };
+        auto grad = [&](int f, const float2* s, float2* o, float2& mid) {
+          const float2 b = two(so[R] + f - 2), c = two(so[R] + f), e = two(so[R] + f + 2);
+          mid = c;
+          o[0] = mul2(s[0], make_float2(c.y - b.y, e.x - c.x));
+          if constexpr (R >= 2) o[0] = fma2(s[1], sub(e, b), o[0]);
+          if constexpr (R >= 3) {
+            const float2 a = two(so[R] + f - 4), h = two(so[R] + f + 4);
+            o[0] = fma2(s[2], make_float2(e.y - a.y, h.x - b.x), o[0]);
+          }
+          o[1] = mul2(s[0], sub(two(so[R] + f + GW), two(so[R] + f - GW)));
+          o[2] = mul2(s[0], sub(two(so[R + 1] + f), two(so[R - 1] + f)));
+#pragma unroll
+          for (int m = 2; m <= R; ++m) {
+            o[1] = fma2(s[m - 1], sub(two(so[R] + f + m * GW), two(so[R] + f - m * GW)), o[1]);
+            o[2] = fma2(s[m - 1], sub(two(so[R + m] + f), two(so[R - m] + f)), o[2]);
+          }
+        };
+        grad(FLD, kc.g, gm, d);
+        grad(0, kc.h, gr, d);
+      } else {
+        auto two = [&](int o) { return make_float2(sm_mom[o], sm_mom[o + dsc]); };
+        auto grad = [&](int f, const float2* s, float2* o, float2& mid) {
+          mid = two(so[R] + f);
+          o[0] = o[1] = o[2] = f2(0.f);
+#pragma unroll
+          for (int m = 1; m <= R; ++m) {
+            o[0] = fma2(s[m - 1], sub(two(so[R] + f + m), two(so[R] + f - m)), o[0]);
+            o[1] = fma2(s[m - 1], sub(two(so[R] + f + m * GW), two(so[R] + f - m * GW)), o[1]);
+            o[2] = fma2(s[m - 1], sub(two(so[R + m] + f), two(so[R - m] + f)), o[2]);
+          }
+        };
+        grad(FLD, kc.g, gm, d);
+        grad(0, kc.h, gr, d);
+      }
+      const float2 r = add2(f2(rref), d), nr2 = mul2(kc.m1, r);
+      const float2 ir = make_float2(__fdividef(1.f, r.x), __fdividef(1.f, r.y));
+      const float2 vx = mul2(add2(jn[0], fma2(nr2, gm[0], gr[0])), ir);
+      const float2 vy = mul2(add2(jn[1], fma2(nr2, gm[1], gr[1])), ir);
+      const float2 vz = mul2(add2(jn[2], fma2(nr2, gm[2], gr[2])), ir);
+      if (pc < pc1) ldj(pc + 1);
+      cell.spread(kc, d, r, vx, vy, vz);
+    }
+    cpa_wait_n<1>();
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 2 * R; ++k) so[k] = so[k + 1];
+    so[2 * R] = so[2 * R] == (NS - 1) * Sh::plane + smine ? smine : so[2 * R] + Sh::plane;
+    if (cell.tgt) cell.collect(kc, pc, z0, PL, nx, rref, rout, jout, q1, q2);
+    cell.flip((pc - pc0) & 1);
+  }
+  if (!cell.ok) atomicMin(bad, (unsigned long long)(t + 1));
+}
+
+// The same with F / rho from the line solves of a compact scheme (acc: three
+// fields): nothing is staged but the exchange, so two planes' loads (seven
+// fields of the thread's own nodes) are all that is in flight.  192^3: 0.088 ms,
+// 230 instructions per node at 52% issue; 24 warps of 80 registers, or two CTAs of
+// 12, spill and take half as long again.
+template <int W>
+__global__ void __launch_bounds__(32 * W, 1) k_mom3d_acc(const KParams p, const MomGeo g, const float* __restrict__ rin,
+                                                         const float* __restrict__ acc, const float* __restrict__ jin,
+                                                         float* __restrict__ rout, float* __restrict__ jout,
+                                                         unsigned long long* bad, const long long t, const int zc,
+                                                         const __grid_constant__ MomConst kc) {
+  extern __shared__ __align__(16) float sm_mom[];
+  MomCell<W> cell(p, g, sm_mom, sm_mom + 2 * MomCell<W>::XB);
+  const int nx = p.nx, nz = p.nz, PL = g.PL, P = g.P;
+  const int z0 = blockIdx.z * zc, z1 = min(z0 + zc, nz), pc0 = z0 - 1, pc1 = z1;
+  const float rref = float(p.rho_ref);
+  float *q1 = jout + P, *q2 = jout + 2 * P;
+  float2 n[7];  // the next plane's rho, j, F / rho
+  auto ld = [&](int pc) {
+    const unsigned zo = wrapi(pc, nz) * PL;
+    n[0] = cell.load(rin, zo);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      n[1 + a] = cell.load(jin + a * P, zo);
+      n[4 + a] = cell.load(acc + a * P, zo);
+    }
+  };
+  pdl_wait();
+  if (cell.live) ld(pc0);
+  for (int pc = pc0; pc <= pc1; ++pc) {
+    if (cell.live) {
+      const float2 d = n[0], r = add2(f2(rref), d);
+      const float2 ir = make_float2(__fdividef(1.f, r.x), __fdividef(1.f, r.y));
+      const float2 vx = fma2(n[1], ir, n[4]), vy = fma2(n[2], ir, n[5]), vz = fma2(n[3], ir, n[6]);
+      if (pc < pc1) ld(pc + 1);
+      cell.spread(kc, d, r, vx, vy, vz);
+    }
+    __syncthreads();
+    if (cell.tgt) cell.collect(kc, pc, z0, PL, nx, rref, rout, jout, q1, q2);
+    cell.flip((pc - pc0) & 1);
+  }
+  if (!cell.ok) atomicMin(bad, (unsigned long long)(t + 1));
 }
 
 // ------------------------------------------------------------------ expand
 // The populations after the last step, pushed from the state before it (rin,
-// muf, jin), and the last density rlast copied into the unpadded field.  One
+// muf, jin; with a compact scheme muf holds F / rho, three fields), and the last density rlast copied into the unpadded field.  One
 // thread per node, stencils through L1: bound by the 76-byte stores.
 template <int S>
 __global__ void __launch_bounds__(256) k_mom_expand(const KParams p, const MomGeo g, const float* __restrict__ rin,
@@ -531,22 +629,30 @@ __global__ void __launch_bounds__(256) k_mom_expand(const KParams p, const MomGe
   const int row = n / nx, x = n - row * nx, z = row / ny, y = row - z * ny;
   const int o = z * g.PL + y * g.LX + 4 + x;
   const float d = __ldg(rin + o), r = float(p.rho_ref) + d;
-  float gx = 0.f, gy = 0.f, gz = 0.f, mx = 0.f, my = 0.f, mz = 0.f;
-#pragma unroll
-  for (int m = 1; m <= R; ++m) {
-    const float c = float(Sch<S>::g(m));
-    const int yp = o + (wrapi(y + m, ny) - y) * g.LX, ym = o + (wrapi(y - m, ny) - y) * g.LX;
-    const int zp = o + (wrapi(z + m, nz) - z) * g.PL, zm = o + (wrapi(z - m, nz) - z) * g.PL;
-    gx += c * (__ldg(rin + o + m) - __ldg(rin + o - m));
-    mx += c * (__ldg(muf + o + m) - __ldg(muf + o - m));
-    gy += c * (__ldg(rin + yp) - __ldg(rin + ym));
-    my += c * (__ldg(muf + yp) - __ldg(muf + ym));
-    gz += c * (__ldg(rin + zp) - __ldg(rin + zm));
-    mz += c * (__ldg(muf + zp) - __ldg(muf + zm));
-  }
   const float ir = __fdividef(1.f, r);
-  const float vx = (jin[o] + (gx * (1.f / 3.f) - r * mx)) * ir, vy = (jin[o + g.P] + (gy * (1.f / 3.f) - r * my)) * ir,
-              vz = (jin[o + 2 * g.P] + (gz * (1.f / 3.f) - r * mz)) * ir;
+  float vx, vy, vz;
+  if constexpr (Sch<S>::GF) {
+    vx = jin[o] * ir + muf[o];
+    vy = jin[o + g.P] * ir + muf[o + g.P];
+    vz = jin[o + 2 * g.P] * ir + muf[o + 2 * g.P];
+  } else {
+    float gx = 0.f, gy = 0.f, gz = 0.f, mx = 0.f, my = 0.f, mz = 0.f;
+#pragma unroll
+    for (int m = 1; m <= R; ++m) {
+      const float c = float(Sch<S>::g(m));
+      const int yp = o + (wrapi(y + m, ny) - y) * g.LX, ym = o + (wrapi(y - m, ny) - y) * g.LX;
+      const int zp = o + (wrapi(z + m, nz) - z) * g.PL, zm = o + (wrapi(z - m, nz) - z) * g.PL;
+      gx += c * (__ldg(rin + o + m) - __ldg(rin + o - m));
+      mx += c * (__ldg(muf + o + m) - __ldg(muf + o - m));
+      gy += c * (__ldg(rin + yp) - __ldg(rin + ym));
+      my += c * (__ldg(muf + yp) - __ldg(muf + ym));
+      gz += c * (__ldg(rin + zp) - __ldg(rin + zm));
+      mz += c * (__ldg(muf + zp) - __ldg(muf + zm));
+    }
+    vx = (jin[o] + (gx * (1.f / 3.f) - r * mx)) * ir;
+    vy = (jin[o + g.P] + (gy * (1.f / 3.f) - r * my)) * ir;
+    vz = (jin[o + 2 * g.P] + (gz * (1.f / 3.f) - r * mz)) * ir;
+  }
   const float nvv = -1.5f * (vx * vx + (vy * vy + vz * vz));
   rout[n] = rlast[o];
   const int dxp = (x + 1 < nx) ? 1 : 1 - nx, dxm = (x > 0) ? -1 : nx - 1;

@@ -62,6 +62,34 @@ def test_d3q19_steps_on_moments(L, shape, scheme, mu64, steps):
     assert np.max(np.abs(a.lbm_get_density() - o.density())) / 0.15 < 1e-5
 
 
+# compact schemes: lines cut into segments on 32 lanes (along x) and on 4, 8 or 16
+# warps (y, z; from 64 and 128 nodes on): lengths that do not divide, shorter
+# than the lanes, of exactly 64 and 128, longer than the periodic wrap of what
+# enters a segment; 12 x 9 x 30 falls back to the populations
+@pytest.mark.parametrize("shape", [(33, 8, 21), (12, 9, 30), (100, 64, 9), (40, 63, 128), (65, 130, 10), (513, 8, 8)])
+@pytest.mark.parametrize("scheme,precision,steps", [("OCFDS4", 1, 6), ("CFDS4", 1, 2), ("CFDS6", 1, 3), ("CFDS8", 1, 5),
+                                                    ("OCFDS4", 0, 4), ("CFDS8", 0, 3)])
+def test_d3q19_compact_steps(L, shape, scheme, precision, steps):
+    kw = dict(scheme=scheme, precision=precision)
+    (a, rho), (b, _) = start(L, L.LBM_D3Q19, shape, **kw), start(L, L.LBM_D3Q19, shape, **kw)
+    check(L, a, b, steps, 1e-6 if precision else 1e-12)
+    o = O.Sim(lattice=O.D3Q19, nx=shape[0], ny=shape[1], nz=shape[2], Tr=0.9, k=0.3, kappa=0.1, scheme=scheme)
+    o.set_f(np.stack([w * rho for w in O.lattice(O.D3Q19)[1]]))
+    assert o.step(steps) == 0
+    assert np.max(np.abs(a.lbm_get_density() - o.density())) / 0.15 < (1e-5 if precision else 1e-12)
+
+
+@pytest.mark.parametrize("shape", [(48, 70, 1), (300, 150, 1)])
+def test_d2q9_fp64_compact_steps(L, shape):
+    kw = dict(scheme="OCFDS4", precision=0, tau=0.8)
+    a, rho = start(L, L.LBM_D2Q9, shape, **kw)
+    a.lbm_step(5)
+    o = O.Sim(lattice=O.D2Q9, nx=shape[0], ny=shape[1], Tr=0.9, k=0.3, kappa=0.1, scheme="OCFDS4", tau=0.8)
+    o.set_f(np.stack([w * rho[0] for w in O.lattice(O.D2Q9)[1]]))
+    assert o.step(5) == 0
+    assert np.max(np.abs(a.lbm_get_density() - o.density())) / 0.15 < 1e-12
+
+
 # tiles of up to 60 columns x 30 rows, two columns per lane: 60 x 30 fills one,
 # 61 cuts into 32 + 29, odd widths end a row in half a pair, 41 nearly fills the
 # scratch, 40 is the narrowest on the moments and 33 falls back to the
