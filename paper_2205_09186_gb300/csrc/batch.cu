@@ -23,6 +23,7 @@
 
 #include "../../include/lbm.h"
 #include "compact_dev.cuh"
+#include "iir.cuh"
 #include "launch.cuh"
 #include "mom2d.cuh"
 #include "step2d.cuh"
@@ -63,7 +64,7 @@ struct CaseDev {
 // lines), [1] the levels that move a float (FP32 lines)
 __constant__ LineCoef c_lines[2][4];
 
-__device__ __forceinline__ bool is_compact(int scheme) { return scheme >= S_CFDS4 && scheme <= S_OCFDS4; }
+__host__ __device__ __forceinline__ bool is_compact(int scheme) { return scheme >= S_CFDS4 && scheme <= S_OCFDS4; }
 
 struct Item {
   int c, tile;
@@ -481,14 +482,25 @@ __global__ void __launch_bounds__(NT2S, RPT >= 4 ? 1 : 2) k_batch_split(const Ca
 
 // An even number of steps of the cases that advance on their moments (mom2d.cuh):
 // gather, then nsteps times every tile, the last time forming the populations,
-// each phase followed by the bounded barrier.  Tile b of the work list goes to
-// CTA b, further ones are claimed from the phase's counter while the one before is
-// being computed.  The moments live in the buffers the populations are not in;
-// after an even number of steps the populations belong in the buffers they
-// started in.  set_t: this launch ends the batch's step.
+// each phase followed by the bounded barrier.  Compact cases make a step three
+// phases: their mu, F / rho along their lines (iir.cuh) with the other cases'
+// tiles behind them, their tiles. (48 cases, 8 of them compact: 79 us a step so; 85
+// with the other cases' tiles beside the mu or the compact tiles, 86 with a third
+// in each phase, whose ends then all wait for part-filled waves. On the populations
+// the batch took 231; its 40 explicit cases alone 125 and now 44.)
+// Item b of a phase goes to CTA b, further ones are
+// claimed from the phase's counter while the one before is being computed.  The
+// moments live in the buffers the populations are not in; after an even number of
+// steps the populations belong in the buffers they started in.  set_t: this
+// launch ends the batch's step.
+struct IirAll {
+  IirK<float> k[4];  // CFDS4, CFDS6, CFDS8, OCFDS4
+};
+
 template <bool FINAL>
-__device__ __forceinline__ void mom_tile(const CaseDev& cd, int par, int s, long long t, int x0, int y0, int vw, int vh,
-                                         float* smem) {
+__device__ __forceinline__ void mom_tile(const CaseDev& cd, int par, int s, long long t, int tile, float* smem) {
+  const int row = tile / cd.mg.nt, x0 = (tile - row * cd.mg.nt) * cd.mg.TW, y0 = row * cd.mg.TH;
+  const int vw = min(cd.mg.TW, cd.kp.nx - x0), vh = min(cd.mg.TH, cd.kp.ny - y0);
   float* m = static_cast<float*>(cd.f[par ^ 1]);
   float* f = static_cast<float*>(cd.f[par]);
   float* rho = static_cast<float*>(cd.rho[par]);
@@ -503,43 +515,93 @@ __device__ __forceinline__ void mom_tile(const CaseDev& cd, int par, int s, long
     LBM_MOM_CASE(S_EFDS6)
     LBM_MOM_CASE(S_E4)
     LBM_MOM_CASE(S_E8)
-    default: break;
+    default:
+      mom2_tile<S_CFDS4, FINAL>(cd.kp, cd.mg.LX, P, r, j, ro, jo, f, cd.bad, t, x0, y0, vw, vh, smem,
+                                static_cast<const float*>(cd.gmu));
+      break;
   }
 #undef LBM_MOM_CASE
 }
 
-__global__ void __launch_bounds__(T2NT, T2_CTAS) k_batch_mom(const CaseDev* __restrict__ cases, const Item* __restrict__ tiles,
-                                                       int ntiles, int nsteps, BatchCtl* ctl,
-                                                       unsigned long long timeout_ns, int set_t) {
-  extern __shared__ __align__(16) unsigned char smem[];
+// mu of a compact case: 64 columns x 32 rows per CTA (tiles across: ceil(nx / 64))
+__device__ __forceinline__ void mom_cmu(const CaseDev& cd, int par, int s, int tile) {
+  const int nt = (cd.kp.nx + 63) / 64, row = tile / nt, w = int(threadIdx.x >> 5);
+  const int x0 = (tile - row * nt) * 64 + 32 * (w & 1), y0 = row * 32 + 8 * (w >> 1);
+  const float* r = static_cast<const float*>(cd.f[par ^ 1]) + (s & 1) * cd.mg.P;
+  if (cd.lap == 4) mom2_mu_rows<4>(cd.kp, cd.mg.LX, r, cd.mu, x0, y0);
+  else if (cd.lap == 6) mom2_mu_rows<6>(cd.kp, cd.mg.LX, r, cd.mu, x0, y0);
+  else mom2_mu_rows<8>(cd.kp, cd.mg.LX, r, cd.mu, x0, y0);
+}
+
+// F / rho of a compact case: groups of lines along x, then of columns
+__device__ __noinline__ void mom_acc(const CaseDev& cd, const IirAll& ia, int par, int s, int g, float* smem) {
+  const int nx = cd.kp.nx, ny = cd.kp.ny, rows = (ny + IIR_CTA_ROWS - 1) / IIR_CTA_ROWS, LX = cd.mg.LX;
+  const float* r = static_cast<const float*>(cd.f[par ^ 1]) + (s & 1) * cd.mg.P;
+  const float rref = float(cd.kp.rho_ref);
+  float* acc = static_cast<float*>(cd.gmu);
+  float* kf = smem + IIR_CTA_FLOATS;
+  const IirK<float>& c = *reinterpret_cast<const IirK<float>*>(kf);
+  if (threadIdx.x < sizeof(IirK<float>) / 4) kf[threadIdx.x] = reinterpret_cast<const float*>(&ia.k[cd.lci])[threadIdx.x];
+  __syncthreads();
+  if (g < rows) {
+    iir_cta_rows(c, nx, ny, LX, 8, r, cd.mu, acc, rref, g * IIR_CTA_ROWS, smem);
+  } else {
+    const int x0 = (g - rows) * iir_cta_cols_n(ny);
+    acc += cd.kp.n;
+    if (ny <= 256) iir_cta_cols<16>(c, nx, ny, LX, 8, r, cd.mu, acc, rref, x0, smem);
+    else iir_cta_cols<8>(c, nx, ny, LX, 8, r, cd.mu, acc, rref, x0, smem);
+  }
+}
+
+static_assert(sizeof(float) * IIR_CTA_FLOATS + sizeof(IirK<float>) <= T2_SMEM, "line groups of a batch");
+
+// work lists of k_batch_mom: tiles of the explicit cases; the compact cases' mu
+// tiles, line groups and tiles
+struct MomWork {
+  const Item *tiles, *cmp[3];
+  int ntiles, ncmp[3];
+};
+
+__global__ void __launch_bounds__(T2NT, T2_CTAS) k_batch_mom(const CaseDev* __restrict__ cases, const MomWork work,
+                                                             int nsteps, BatchCtl* ctl, unsigned long long timeout_ns,
+                                                             int set_t, const __grid_constant__ IirAll ia) {
+  extern __shared__ __align__(16) unsigned char smem_[];
+  float* smem = reinterpret_cast<float*>(smem_);
   __shared__ int s_q[2];
   const long long t0 = *((volatile long long*)&ctl->t);
   const int par = int(t0 & 1), w = int(threadIdx.x >> 5);
-  for (int k = 0; k <= nsteps; ++k) {  // phase 0: gather; phase k: step k - 1
+  const int ph = work.ncmp[2] > 0 ? 3 : 1;  // phases of a step
+  int q = 0;
+  for (int k = 0; k <= ph * nsteps; ++k) {  // phase 0: gather
+    const int s = k > 0 ? (k - 1) / ph : 0, f = k > 0 ? (k - 1) - s * ph : 2;
+    const bool last = s == nsteps - 1;
+    const Item* cmp = work.cmp[f];
+    const int nc = work.ncmp[f], n = nc + (k == 0 || ph == 1 || f == 1 ? work.ntiles : 0);
     unsigned* ctr = &ctl->work[k & 3];
-    int q = 0;
-    for (int u = int(blockIdx.x); u < ntiles; q ^= 1) {
-      // (a slot is rewritten two tiles after it was read, and every thread
-      // passes a barrier of the tile in between)
+    for (int u = int(blockIdx.x); u < n;) {
+      // (a slot is rewritten two items after it was read, past the barrier below)
       if (threadIdx.x == 0) s_q[q] = int(gridDim.x) + int(atomicAdd(ctr, 1u));
-      const Item itm = tiles[u];
+      const Item itm = u < nc ? cmp[u] : work.tiles[u - nc];
       const CaseDev& cd = cases[itm.c];
-      const int row = itm.tile / cd.mg.nt, x0 = (itm.tile - row * cd.mg.nt) * cd.mg.TW, y0 = row * cd.mg.TH;
-      const int vw = min(cd.mg.TW, cd.kp.nx - x0), vh = min(cd.mg.TH, cd.kp.ny - y0);
       if (k == 0) {
+        const int row = itm.tile / cd.mg.nt, x0 = (itm.tile - row * cd.mg.nt) * cd.mg.TW, y0 = row * cd.mg.TH;
+        const int vw = min(cd.mg.TW, cd.kp.nx - x0), vh = min(cd.mg.TH, cd.kp.ny - y0);
         for (int y = y0 + w; y < y0 + vh; y += T2NT / 32)
           mom2_gather(cd.kp, cd.mg.LX, cd.mg.P, static_cast<const float*>(cd.f[par]),
                       static_cast<const float*>(cd.rho[par]), static_cast<float*>(cd.f[par ^ 1]),
                       static_cast<float*>(cd.f[par ^ 1]) + 2 * cd.mg.P, cd.bad, t0, x0, vw, y, y + 1);
-        __syncthreads();
-      } else if (k < nsteps) {
-        mom_tile<false>(cd, par, k - 1, t0 + k - 1, x0, y0, vw, vh, reinterpret_cast<float*>(smem));
+      } else if (u < nc && f < 2) {
+        if (f == 0) mom_cmu(cd, par, s, itm.tile);
+        else mom_acc(cd, ia, par, s, itm.tile, smem);
       } else {
-        mom_tile<true>(cd, par, k - 1, t0 + k - 1, x0, y0, vw, vh, reinterpret_cast<float*>(smem));
+        if (last) mom_tile<true>(cd, par, s, t0 + s, itm.tile, smem);
+        else mom_tile<false>(cd, par, s, t0 + s, itm.tile, smem);
       }
+      __syncthreads();
       u = s_q[q];
+      q ^= 1;
     }
-    if (k == nsteps) break;
+    if (k == ph * nsteps) break;
     if (blockIdx.x == 0 && threadIdx.x == 0) ctl->work[(k + 2) & 3] = 0u;
     if (!grid_barrier(ctl, timeout_ns)) return;
   }
@@ -666,7 +728,8 @@ struct lbm_batch {
   // cases on the moments: their tiles; they come first in the work lists above,
   // nmu_mom and ncoll_mom items of them
   Item* d_tiles = nullptr;
-  int ntiles = 0, grid_mom = 0, nmu_mom = 0, ncoll_mom = 0;
+  MomWork work{};
+  int grid_mom = 0, nmu_mom = 0, ncoll_mom = 0, nline_mom = 0;
   std::vector<int> case_order;  // split path: cases in work-list order
   // compact-scheme cases: their mu tiles (TXB x TYB), their line groups
   // (rebuilt with the group size lpb of the tile shape), longest line
@@ -693,6 +756,7 @@ static int build_line_items(lbm_batch* b, int lpb) {
       for (int g = 0; g < groups; ++g)
         for (int field = 0; field < 2; ++field) li.push_back({c, g * 4 + 2 * axis + field});
     }
+    if (cd.mom) b->nline_mom = int(li.size());
   }
   if (int(li.size()) > b->line_cap) return LBM_ECUDA;
   if (!li.empty() && cudaMemcpyAsync(b->d_litems, li.data(), sizeof(Item) * li.size(), cudaMemcpyHostToDevice,
@@ -783,27 +847,41 @@ static int setup_split_t(lbm_batch* b) {
   return LBM_OK;
 }
 
-// tiles of the cases on the moments, the dearest schemes' first
+// work lists of the cases on the moments, the dearest schemes' tiles first
 static int setup_moments(lbm_batch* b) {
   int dev = 0, sms = 0, ps = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  std::vector<Item> tiles;
-  for (const int s : {S_E8, S_EFDS6, S_E4, S_EFDS4, S_EFDS2})
+  std::vector<Item> list, cmp[3];
+  MomWork& wk = b->work;
+  wk = MomWork{};
+  for (const int s : {S_E8, S_EFDS6, S_E4, S_EFDS4, S_EFDS2, S_CFDS4})
     for (const int c : b->case_order) {
-      CaseDev& cd = b->host_cases[c];
-      if (!cd.mom || cd.scheme != s) continue;
-      for (int u = 0; u < cd.mg.nt * cd.mg.nr; ++u) tiles.push_back({c, u});
+      const CaseDev& cd = b->host_cases[c];
+      if (!cd.mom || (is_compact(cd.scheme) ? int(S_CFDS4) : cd.scheme) != s) continue;
+      for (int u = 0; u < cd.mg.nt * cd.mg.nr; ++u) (s == S_CFDS4 ? cmp[2] : list).push_back({c, u});
+      if (s != S_CFDS4) continue;
+      const int nx = cd.kp.nx, ny = cd.kp.ny;
+      for (int u = 0; u < (nx + 63) / 64 * ((ny + 31) / 32); ++u) cmp[0].push_back({c, u});
+      const int groups = (ny + IIR_CTA_ROWS - 1) / IIR_CTA_ROWS + (nx + iir_cta_cols_n(ny) - 1) / iir_cta_cols_n(ny);
+      for (int g = groups - 1; g >= 0; --g) cmp[1].push_back({c, g});
     }
-  if (tiles.empty()) return LBM_OK;
+  if (list.empty() && cmp[2].empty()) return LBM_OK;
   if (cudaFuncSetAttribute(k_batch_mom, cudaFuncAttributeMaxDynamicSharedMemorySize, T2_SMEM) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ps, k_batch_mom, T2NT, T2_SMEM) != cudaSuccess || ps < 1)
     return LBM_ECUDA;
-  b->ntiles = int(tiles.size());
-  b->grid_mom = std::max(1, std::min(ps * sms, b->ntiles));
-  b->d_tiles = static_cast<Item*>(balloc(b, sizeof(Item) * tiles.size()));
+  wk.ntiles = int(list.size());
+  const int most = int(list.size() + std::max(cmp[1].size(), cmp[2].size()));
+  for (int f = 0; f < 3; ++f) {
+    wk.ncmp[f] = int(cmp[f].size());
+    list.insert(list.end(), cmp[f].begin(), cmp[f].end());
+  }
+  b->grid_mom = std::max(1, std::min(ps * sms, most));
+  b->d_tiles = static_cast<Item*>(balloc(b, sizeof(Item) * list.size()));
   if (!b->d_tiles) return LBM_ENOMEM;
-  if (cudaMemcpyAsync(b->d_tiles, tiles.data(), sizeof(Item) * tiles.size(), cudaMemcpyHostToDevice, b->stream) != cudaSuccess ||
+  wk.tiles = b->d_tiles;
+  for (int f = 0, at = wk.ntiles; f < 3; at += wk.ncmp[f++]) wk.cmp[f] = wk.tiles + at;
+  if (cudaMemcpyAsync(b->d_tiles, list.data(), sizeof(Item) * list.size(), cudaMemcpyHostToDevice, b->stream) != cudaSuccess ||
       cudaStreamSynchronize(b->stream) != cudaSuccess)
     return LBM_ECUDA;
   return LBM_OK;
@@ -882,7 +960,10 @@ extern "C" int lbm_batch_create(const lbm_params* cases, int n, void* stream, co
     ok = cd.f[0] && cd.f[1] && cd.rho[0] && cd.rho[1] && cd.snap && cd.bad && (cd.mu || prec0 != LBM_FP32DEV || mu0);
     cd.lap = cd.lci = 0;
     cd.cmu = cd.gmu = cd.grho = nullptr;
-    cd.mom = prec0 == LBM_FP32DEV && !mu0 && mom2d_ok(cd.kp, q.scheme, 1, cd.mrt.on != 0);
+    // (compact cases: the fit and tau as for an explicit scheme, lines of at most 512)
+    const bool comp = is_compact(q.scheme);
+    cd.mom = prec0 == LBM_FP32DEV && !mu0 && (!comp || iir_ok(cd.kp)) &&
+             mom2d_ok(cd.kp, comp ? S_EFDS4 : q.scheme, 1, cd.mrt.on != 0);
     cd.mg = Mom2Geo{};
     if (cd.mom) cd.mg = mom2_geo(cd.kp, 1);
     if (ok && q.scheme >= LBM_CFDS4 && q.scheme <= LBM_OCFDS4) {
@@ -1055,10 +1136,10 @@ static cudaError_t launch_split(lbm_batch* b, int nsteps, bool all) {
   cs.attrs = at;
   cs.numAttrs = 1;
   auto kern = b->rpt == 1 ? k_batch_split<1> : (b->rpt == 4 ? k_batch_split<4> : k_batch_split<2>);
-  const int m0 = all ? 0 : b->nmu_mom, c0 = all ? 0 : b->ncoll_mom;
+  const int m0 = all ? 0 : b->nmu_mom, c0 = all ? 0 : b->ncoll_mom, l0 = all ? 0 : b->nline_mom;
   return cudaLaunchKernelEx(&cs, kern, (const CaseDev*)b->d_cases, (const Item*)b->d_mitems + m0, b->nmu - m0,
                             (const Item*)b->d_citems + c0, b->ncoll - c0, nsteps, b->ctl, BARRIER_NS, b->buf_split,
-                            (const Item*)b->d_litems, b->nline, b->lpb, b->lpb_shift);
+                            (const Item*)b->d_litems + l0, b->nline - l0, b->lpb, b->lpb_shift);
 }
 
 // nsteps steps of every case: on the populations in one persistent launch, or,
@@ -1071,7 +1152,7 @@ static cudaError_t launch_persistent(lbm_batch* b, int nsteps) {
   cudaError_t e = reset();
   if (e != cudaSuccess) return e;
   if (b->split) {
-    const int even = b->ntiles > 0 ? nsteps / 2 * 2 : 0;
+    const int even = b->work.tiles ? nsteps / 2 * 2 : 0;
     if (nsteps - even > 0 && (e = launch_split(b, nsteps - even, true)) != cudaSuccess) return e;
     if (even == 0) return e;
     const bool rest = b->nmu > b->nmu_mom;
@@ -1086,8 +1167,9 @@ static cudaError_t launch_persistent(lbm_batch* b, int nsteps) {
     cs.attrs = at;
     cs.numAttrs = 1;
     if ((e = reset()) != cudaSuccess) return e;
-    e = cudaLaunchKernelEx(&cs, k_batch_mom, (const CaseDev*)b->d_cases, (const Item*)b->d_tiles, b->ntiles, even, b->ctl,
-                           timeout_ns, rest ? 0 : 1);
+    IirAll ia;
+    for (int k = 0; k < 4; ++k) ia.k[k] = iir_coef(S_CFDS4 + k);
+    e = cudaLaunchKernelEx(&cs, k_batch_mom, (const CaseDev*)b->d_cases, b->work, even, b->ctl, timeout_ns, rest ? 0 : 1, ia);
     if (e != cudaSuccess || !rest) return e;
     if ((e = reset()) != cudaSuccess) return e;
     return launch_split(b, even, false);
@@ -1259,7 +1341,7 @@ extern "C" long long lbm_batch_get_step(const lbm_batch* b) { return b ? b->t : 
 // CTAs of the batch's launches (the smallest, where there are two kinds)
 static int resident(const lbm_batch* b) {
   const int g = b->split ? b->grid_split : b->grid;
-  return b->ntiles > 0 ? std::min(g, b->grid_mom) : g;
+  return b->work.tiles ? std::min(g, b->grid_mom) : g;
 }
 
 extern "C" int lbm_batch_inject_stall(lbm_batch* b, int cta) {

@@ -67,6 +67,8 @@ cudaError_t run(const IirGeo& g, int scheme, const T* rho, const T* mu, T* out, 
 
 }  // namespace
 
+IirK<float> iir_coef(int scheme) { return coef<float>(scheme); }
+
 // segments: at most 16 nodes on 32 lanes along x, 32 on 16 warps along y and z
 bool iir_ok(const KParams& kp) { return kp.nx <= 512 && kp.ny <= 512 && kp.nz <= 512; }
 

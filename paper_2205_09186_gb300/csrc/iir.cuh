@@ -207,4 +207,136 @@ __global__ void __launch_bounds__(256) k_iir_row(const IirGeo g, const T* __rest
   for (int i = lane; i < L; i += 32) out[base + i] = sr[i + (i >> 5)];
 }
 
+// ------------------------------------------------------------------ CTAs of a batch
+// The same for D2Q9 lattices in a persistent launch, by a CTA of 256 threads: eight
+// lines along x (a warp each), or Q columns (256 / Q segments each). rho is padded
+// (row stride ldr, first column at off), mu and out are not. Written earlier in the
+// launch, so read by ordinary loads. All threads take part (barriers inside); c and
+// smem (IIR_CTA_FLOATS) in shared memory.
+//
+// The segments lie in shared memory, not in registers as above: the registers are
+// the tile kernel's 80, its shared memory leaves the L1 a few KB, and spilled
+// segments went to L2 and back (48 cases, 8 of them compact: 111 us a step).
+constexpr int IIR_CTA_ROWS = 8, IIR_CTA_LP = 512 + 6 + 16 + 1;  // rows, a padded line
+__host__ __device__ constexpr int iir_cta_cols_n(int ny) { return ny <= 256 ? 16 : 8; }
+constexpr int IIR_CTA_FLOATS = 4 * (256 + 6) * 16 + 1024 + 64;
+static_assert(IIR_CTA_FLOATS >= 4 * IIR_CTA_ROWS * IIR_CTA_LP && IIR_CTA_FLOATS >= 4 * (512 + 6) * 8 + 1024, "fits");
+
+// a segment of both fields: r and u (nodes -3 .. len + 2 about at(0)), y scratch;
+// enter(ends, dir): what enters it from the segments before (-1) and after (1)
+template <class At, class Enter, class Emit>
+__device__ __forceinline__ void iir_cta_seg(const IirK<float>& c, const float* r, const float* u, float* yr, float* yu,
+                                            At at, int len, Enter enter, Emit emit) {
+  const float a1 = c.a1, a2 = c.a2, a3 = c.a3, nr = c.nr;
+  float2 y = make_float2(0.f, 0.f);
+  {
+    float r0 = r[at(-3)], r1 = r[at(-2)], r2 = r[at(-1)], r3 = r[at(0)], r4 = r[at(1)], r5 = r[at(2)];
+    float u0 = u[at(-3)], u1 = u[at(-2)], u2 = u[at(-1)], u3 = u[at(0)], u4 = u[at(1)], u5 = u[at(2)];
+#pragma unroll 2
+    for (int k = 0; k < len; ++k) {
+      const float r6 = r[at(k + 3)], u6 = u[at(k + 3)];
+      y.x = a1 * (r4 - r2) + a2 * (r5 - r1) + a3 * (r6 - r0) + nr * y.x;
+      y.y = a1 * (u4 - u2) + a2 * (u5 - u1) + a3 * (u6 - u0) + nr * y.y;
+      yr[at(k)] = y.x;
+      yu[at(k)] = y.y;
+      r0 = r1, r1 = r2, r2 = r3, r3 = r4, r4 = r5, r5 = r6;
+      u0 = u1, u1 = u2, u2 = u3, u3 = u4, u4 = u5, u5 = u6;
+    }
+  }
+  float2 e = enter(y, -1);
+  y = make_float2(0.f, 0.f);
+#pragma unroll 2
+  for (int k = len - 1; k >= 0; --k) {
+    const float p = c.p[k + 1];
+    y.x = yr[at(k)] + e.x * p + nr * y.x;
+    y.y = yu[at(k)] + e.y * p + nr * y.y;
+    yr[at(k)] = y.x;
+    yu[at(k)] = y.y;
+  }
+  e = enter(y, 1);
+#pragma unroll 2
+  for (int k = len - 1; k >= 0; --k) {
+    e.x *= nr;
+    e.y *= nr;
+    emit(k, yr[at(k)] + e.x, yu[at(k)] + e.y);
+  }
+}
+
+__device__ __forceinline__ void iir_cta_rows(const IirK<float>& c, int nx, int ny, int ldr, int off, const float* rho,
+                                             const float* mu, float* out, float rref, int y0, float* smem) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, y = y0 + w;
+  float *sr = smem + w * 4 * IIR_CTA_LP, *su = sr + IIR_CTA_LP, *yr = su + IIR_CTA_LP, *yu = yr + IIR_CTA_LP;
+  if (y < ny) {
+    for (int k = lane; k < nx + 6; k += 32) {
+      int i = k - 3;
+      i = i < 0 ? i + nx : (i >= nx ? i - nx : i);
+      sr[k + (k >> 5)] = rho[y * ldr + off + i];
+      su[k + (k >> 5)] = mu[y * nx + i];
+    }
+    __syncwarp();
+    const int i0 = lane * nx / 32, len = (lane + 1) * nx / 32 - i0, J = (c.K * 32 + nx - 1) / nx + 1;
+    const float pl = c.p[len];
+    auto at = [&](int k) { return i0 + 3 + k + ((i0 + 3 + k) >> 5); };
+    // -r^nx closes the period (doubling sums all 32 segments when J asks for it)
+    auto enter = [&](float2 a, int dir) {
+      float f = pl;
+      int n = 1;
+      for (; n < J && n < 32; n *= 2) {
+        const int from = (lane + dir * n) & 31;
+        const float ax = __shfl_sync(0xffffffffu, a.x, from), ay = __shfl_sync(0xffffffffu, a.y, from);
+        const float f1 = __shfl_sync(0xffffffffu, f, from);
+        a.x += f * ax;
+        a.y += f * ay;
+        f *= f1;
+      }
+      a.x = __shfl_sync(0xffffffffu, a.x, (lane + dir) & 31);
+      a.y = __shfl_sync(0xffffffffu, a.y, (lane + dir) & 31);
+      return n == 32 ? make_float2(a.x / (1.f - f), a.y / (1.f - f)) : a;
+    };
+    iir_cta_seg(c, sr, su, yr, yu, at, len, enter,
+                [&](int k, float dr, float du) { yu[at(k)] = __fdividef(dr, 3.f * (rref + sr[at(k)])) - du; });
+    __syncwarp();
+    for (int i = lane; i < nx; i += 32) out[y * nx + i] = yu[i + 3 + ((i + 3) >> 5)];
+  }
+}
+
+template <int Q>
+__device__ __forceinline__ void iir_cta_cols(const IirK<float>& c, int nx, int ny, int ldr, int off, const float* rho,
+                                             const float* mu, float* out, float rref, int x0, float* smem) {
+  constexpr int S = 256 / Q;
+  const int q = threadIdx.x % Q, s = threadIdx.x / Q, x = min(x0 + q, nx - 1), F = (ny + 6) * Q;
+  float *sr = smem, *su = sr + F, *yr = su + F, *yu = yr + F;
+  float2* se = reinterpret_cast<float2*>(smem + IIR_CTA_FLOATS - 1024);  // [2][S][Q] of ends, forward and back
+  for (int r = s; r < ny + 6; r += S) {
+    int i = r - 3;
+    i = i < 0 ? i + ny : (i >= ny ? i - ny : i);
+    sr[r * Q + q] = rho[i * ldr + off + x];
+    su[r * Q + q] = mu[i * nx + x];
+  }
+  __syncthreads();
+  const int i0 = s * ny / S, len = (s + 1) * ny / S - i0, lo = ny / S, J = (c.K * S + ny - 1) / ny + 1;
+  const float plo = c.p[lo], phi = c.p[lo + 1];
+  auto at = [&](int k) { return (i0 + 3 + k) * Q + q; };
+  auto enter = [&](float2 v, int dir) {
+    float2* f = se + (dir > 0 ? S * Q : 0);
+    f[threadIdx.x] = v;
+    __syncthreads();
+    float2 a = make_float2(0.f, 0.f);
+    for (int j = J; j >= 1; --j) {
+      const int t = (s + dir * j) & (S - 1);
+      const float p = (t + 1) * ny / S - t * ny / S > lo ? phi : plo;
+      const float2 b = f[t * Q + q];
+      a.x = b.x + p * a.x;
+      a.y = b.y + p * a.y;
+    }
+    return a;
+  };
+  iir_cta_seg(c, sr, su, yr, yu, at, len, enter, [&](int k, float dr, float du) {
+    if (x0 + q < nx) out[(i0 + k) * nx + x] = __fdividef(dr, 3.f * (rref + sr[at(k)])) - du;
+  });
+}
+
+// coefficients of a scheme (host)
+IirK<float> iir_coef(int scheme);
+
 }  // namespace lbmd

@@ -100,39 +100,52 @@ __device__ __forceinline__ float2 mu_pair(float2 rho, float2 lap, const EosF& e,
 template <int S, bool FINAL>
 __device__ __forceinline__ void mom2_tile(const KParams& p, int LX, int P, const float* rin, const float* jin, float* rout,
                                           float* jout, float* fout, unsigned long long* bad, long long t, int x0, int y0,
-                                          int VW, int VH, float* smem) {
+                                          int VW, int VH, float* smem, const float* acc = nullptr) {
   using Sh = Mom2Shape<S>;
+  constexpr bool GF = Sch<S>::GF;  // compact: F / rho from acc (two unpadded fields)
   constexpr int R = Sh::R, H = Sh::H, RW = Sh::RW, MW = Sh::MW, XK = Sh::XR * 32;
   constexpr bool ISO = Sch<S>::ISO;
   const Mom2Const& kc = c_mom2<S>;
   float* s_r = smem;                                        // row k: y0 - H + k; column j: x0 - 8 + j
   float* s_m = s_r + Sh::RR * RW;                           // row k: y0 - 1 - R + k; column j: x0 - 4 + j
-  float2* s_x = reinterpret_cast<float2*>(s_m + Sh::MR * MW);  // [6][XR][32]
+  float2* s_x = reinterpret_cast<float2*>(GF ? smem : s_m + Sh::MR * MW);  // [6][XR][32]
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, nx = p.nx, ny = p.ny;
   const float rref = float(p.rho_ref);
-  // ---- rho (16-byte chunks; those past the padded row are zeroed)
-  for (int e = tid; e < (VH + 2 * H) * 19; e += T2NT) {
-    const int k = e / 19, j = 4 * (e - k * 19);
-    if (x0 + j + 4 <= LX) cpa16(s_r + k * RW + j, rin + (unsigned(wrapn(y0 - H + k, ny)) * LX + x0 + j));
-    else *reinterpret_cast<float4*>(s_r + k * RW + j) = make_float4(0.f, 0.f, 0.f, 0.f);
+  if constexpr (!GF) {
+    // ---- rho (16-byte chunks; those past the padded row are zeroed)
+    for (int e = tid; e < (VH + 2 * H) * 19; e += T2NT) {
+      const int k = e / 19, j = 4 * (e - k * 19);
+      if (x0 + j + 4 <= LX) cpa16(s_r + k * RW + j, rin + (unsigned(wrapn(y0 - H + k, ny)) * LX + x0 + j));
+      else *reinterpret_cast<float4*>(s_r + k * RW + j) = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    cpa_commit();
   }
-  cpa_commit();
   auto two = [](const float* q) { return *reinterpret_cast<const float2*>(q); };
   // momentum of the warp's next row of the ring, loaded a row ahead
-  float2 jx = f2(0.f), jy = f2(0.f);
+  float2 jx = f2(0.f), jy = f2(0.f), dn = f2(0.f), ax = f2(0.f), ay = f2(0.f);
+  const int xa = GF ? wrapn(x0 - 2 + 2 * lane, nx) : 0, xb = GF ? wrapn(x0 - 1 + 2 * lane, nx) : 0;
   auto ldj = [&](int k) {
     if (k < VH + 2 && x0 + 8 + 2 * lane <= LX) {  // inside the padded row
-      const unsigned o = unsigned(wrapn(y0 - 1 + k, ny)) * LX + 6 + x0 + 2 * lane;
+      const int y = wrapn(y0 - 1 + k, ny);
+      const unsigned o = unsigned(y) * LX + 6 + x0 + 2 * lane;
       jx = two(jin + o);
       jy = two(jin + P + o);
+      if constexpr (GF) {
+        dn = two(rin + o);
+        const float* a = acc + y * nx;
+        ax = make_float2(a[xa], a[xb]);
+        ay = make_float2(a[int(p.n) + xa], a[int(p.n) + xb]);
+      }
     }
   };
   ldj(w);
-  cpa_wait_all();
-  __syncthreads();
+  if constexpr (!GF) {
+    cpa_wait_all();
+    __syncthreads();
+  }
   auto sub = [&](float2 a, float2 b) { return fma2(kc.m1, b, a); };
   // ---- mu of the pairs -4 .. 63
-  {
+  if constexpr (!GF) {
     const float k2 = float(p.k2), kap = float(p.kappa);
     const EosF ef = eos_f(p);
     for (int e = tid; e < (VH + 2 + 2 * R) * 34; e += T2NT) {
@@ -172,15 +185,17 @@ __device__ __forceinline__ void mom2_tile(const KParams& p, int LX, int P, const
       }
       *reinterpret_cast<float2*>(s_m + k * MW + j) = mu_pair(add2(f2(rref), c), lap, ef, k2, kap);
     }
+    __syncthreads();
   }
-  __syncthreads();
   // ---- collision: row k of the ring and the tile, columns -2 .. 61
   for (int k = w; k < VH + 2; k += T2NT / 32) {
+    float2 d, gmx, gmy, grx, gry;  // grad mu, grad rho / 3
     const float* q = s_r + (k + H - 1) * RW + 6 + 2 * lane;
     const float* m = s_m + (k + R) * MW + 2 + 2 * lane;
-    const float2 d = two(q);
-    float2 gmx, gmy, grx, gry;  // grad mu, grad rho / 3
-    if constexpr (ISO) {
+    d = GF ? dn : two(q);
+    if constexpr (GF) {
+      gmx = gmy = grx = gry = f2(0.f);
+    } else if constexpr (ISO) {
       auto grad = [&](const float* b, int W, float2& gx, float2& gy) {
         float x0_ = 0.f, x1 = 0.f, y0_ = 0.f, y1 = 0.f;
 #pragma unroll
@@ -233,7 +248,14 @@ __device__ __forceinline__ void mom2_tile(const KParams& p, int LX, int P, const
     }
     const float2 r = add2(f2(rref), d), nr = mul2(kc.m1, r);
     const float2 ir = make_float2(__fdividef(1.f, r.x), __fdividef(1.f, r.y));
-    const float2 vx = mul2(add2(jx, fma2(nr, gmx, grx)), ir), vy = mul2(add2(jy, fma2(nr, gmy, gry)), ir);
+    float2 vx, vy;
+    if constexpr (GF) {
+      vx = fma2(jx, ir, ax);
+      vy = fma2(jy, ir, ay);
+    } else {
+      vx = mul2(add2(jx, fma2(nr, gmx, grx)), ir);
+      vy = mul2(add2(jy, fma2(nr, gmy, gry)), ir);
+    }
     ldj(k + T2NT / 32);
     // post-collision populations (Eq. 2's order); opposite ones share all but
     // the sign of the linear term; the rest population carries drho less the
@@ -319,6 +341,32 @@ __device__ __forceinline__ void mom2_tile(const KParams& p, int LX, int P, const
     }
   }
   if (!ok) atomicMin(bad, (unsigned long long)(t + 1));
+}
+
+// mu of a compact scheme (central Laplacian of order LO) at 8 rows x 32 columns by a
+// warp, from the padded rho into the unpadded mu; ordinary loads (mom2_tile)
+template <int LO>
+__device__ __forceinline__ void mom2_mu_rows(const KParams& p, int LX, const float* rin, float* mu, int x0, int y0) {
+  constexpr int R = LO / 2, U = 8;
+  constexpr double l0 = LO == 4 ? -2.5 : (LO == 6 ? -49.0 / 18.0 : -205.0 / 72.0);
+  constexpr double l[5] = {l0, LO == 4 ? 4.0 / 3.0 : (LO == 6 ? 1.5 : 1.6), LO == 4 ? -1.0 / 12.0 : (LO == 6 ? -0.15 : -0.2),
+                           LO == 6 ? 1.0 / 90.0 : (LO == 8 ? 8.0 / 315.0 : 0.0), LO == 8 ? -1.0 / 560.0 : 0.0};
+  const int x = x0 + int(threadIdx.x & 31), nx = p.nx, ny = p.ny;
+  if (x >= nx || y0 >= ny) return;
+  const float k2 = float(p.k2), kap = float(p.kappa), rref = float(p.rho_ref);
+  const EosF ef = eos_f(p);
+  float c[U + 2 * R];
+#pragma unroll
+  for (int k = 0; k < U + 2 * R; ++k) c[k] = rin[wrapn(y0 - R + k, ny) * LX + 8 + x];
+#pragma unroll
+  for (int r = 0; r < U; ++r) {
+    if (y0 + r >= ny) break;
+    const float* q = rin + (y0 + r) * LX + 8 + x;
+    float lap = float(2.0 * l[0]) * c[r + R];
+#pragma unroll
+    for (int m = 1; m <= R; ++m) lap += float(l[m]) * ((q[m] + q[-m]) + (c[r + R + m] + c[r + R - m]));
+    mu[(y0 + r) * nx + x] = k2 * eos_mu_f(rref + c[r + R], ef) - kap * lap;
+  }
 }
 
 // moments of the populations f at rows ya .. yb - 1, columns xs .. xs + ow - 1
