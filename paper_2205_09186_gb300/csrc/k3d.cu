@@ -9,6 +9,7 @@
 #include "launch.cuh"
 #include "step3d.cuh"
 #include "step3d_fast.cuh"
+#include "step3d_node.cuh"
 #include "step3d_split.cuh"
 #include "coll3d_launch.cuh"
 
@@ -136,11 +137,51 @@ cudaError_t launch_mu(const Launch& c, bool zero_edges = false) {
   return cudaGetLastError();
 }
 
+// Whether a step runs on node-parallel passes (step3d_node.cuh) or on the mu and
+// collision passes. By nodes: rows of whole 16-byte chunks suit the collision pass's
+// tensor copies, so it takes over where one population array (76 bytes a node)
+// outgrows about two thirds of the L2; on other rows it issues four times as many
+// copies and is worth its halo only well beyond the L2. Measured, tau 0.8, us a step
+// on the two passes and here: 96^3 58 and 51, 104^3 83 and 70, 128^3 105 and 126;
+// 97^3 80 and 54, 129^3 143 and 131, 161^3 271 and 251, 193^3 412 and 425. With
+// observables, whose sums cost small blocks more: 125 x 70 x 43 63 and 39, 64^3 61
+// and 36, 96^3 79 and 87.
+bool node_rule(const KParams& kp, bool vec, bool obs) {
+  return kp.n <= (obs ? 600000 : (vec ? 1200000 : 4200000));
+}
+
+// the three node-parallel passes (step3d_node.cuh)
+template <int S, bool TAU1, bool M64>
+cudaError_t launch_node(const Launch& c, int* nblocks, bool obs) {
+  const KParams& kp = c.kp;
+  const int g = int((kp.n + NODE_T - 1) / NODE_T), go = std::min(g, 8 * num_sms());
+  if (nblocks) {
+    if (obs && go > *nblocks) return cudaErrorNotSupported;
+    *nblocks = obs ? go : g;
+  } else if (obs) {
+    return cudaErrorInvalidValue;
+  }
+  const unsigned mx = unsigned(((1ull << 32) + kp.nx - 1) / kp.nx), my = unsigned(((1ull << 32) + kp.ny - 1) / kp.ny);
+  const float *fin = static_cast<const float*>(c.fin), *rin = static_cast<const float*>(c.rin);
+  float *fout = static_cast<float*>(c.fout), *rout = static_cast<float*>(c.rout), *mu = static_cast<float*>(c.mu);
+  cudaError_t e = launch_pdl(k_node_mu<S, M64>, g, NODE_T, 0, c.stream, kp, mx, my, rin, mu);
+  if (e != cudaSuccess) return e;
+  if (c.ev_mid) cudaEventRecord(c.ev_mid, c.stream);
+  auto k = obs ? k_node_coll<S, TAU1, true> : k_node_coll<S, TAU1, false>;
+  e = launch_pdl(k, obs ? go : g, NODE_T, 0, c.stream, kp, mx, my, fin, fout, rin, mu, c.aux.bad_step, c.aux.t,
+                 obs ? static_cast<float*>(const_cast<void*>(c.aux.rho_snap)) : nullptr, c.aux.partials);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(k_node_rho, g, NODE_T, 0, c.stream, kp, fout, rout, c.aux.bad_step, c.aux.t + 1);
+}
+
 // mu pass + collision pass (line schemes, FP32DEV, FP32 mu); with obs the
 // collision pass also reduces the observables of the state it advances
 template <int S, bool TAU1, bool M64 = false>
 cudaError_t launch_split(const Launch& c, int* nblocks, bool obs) {
   if (!c.mu) return cudaErrorInvalidValue;
+  // 16-byte copies need rows of whole chunks and aligned bases
+  const bool vec = c.kp.nx % 4 == 0 && aligned16(c.fin) && aligned16(c.rin) && aligned16(c.mu) && c.tmap;
+  if (node_rule(c.kp, vec, obs)) return launch_node<S, TAU1, M64>(c, nblocks, obs);
   const int zc = c.zc > 0 ? c.zc : split_zchunk_heuristic(c.kp, Sch<S>::R, TYC, CollShape<S, CY, 2, COLL_FD>::MINB);
   const long long ctas = coll3d_ctas(c.kp, zc);
   if (nblocks) {
@@ -153,8 +194,6 @@ cudaError_t launch_split(const Launch& c, int* nblocks, bool obs) {
   cudaError_t em = launch_mu<S, M64>(c, true);
   if (em != cudaSuccess) return em;
   if (c.ev_mid) cudaEventRecord(c.ev_mid, c.stream);
-  // 16-byte copies need rows of whole chunks and aligned bases
-  const bool vec = c.kp.nx % 4 == 0 && aligned16(c.fin) && aligned16(c.rin) && aligned16(c.mu) && c.tmap;
   if (obs)
     return vec ? launch_coll<S, TAU1, true, true>(c, zc) : launch_coll<S, TAU1, false, true>(c, zc);
   return vec ? launch_coll<S, TAU1, true, false>(c, zc) : launch_coll<S, TAU1, false, false>(c, zc);

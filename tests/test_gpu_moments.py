@@ -134,3 +134,39 @@ def test_moments_report_the_first_bad_step(L):
     oa, ob = a.lbm_observables(), b.lbm_observables()
     assert oa["status"] == ob["status"] == L.LBM_EUNSTABLE
     assert abs(oa["step"] - ob["step"]) <= 2
+
+
+# node-parallel D3Q19 steps: 512 nodes, a last block of part of its threads, sizes
+# either side of the ranges (rows of whole 16-byte chunks up to 1.2 million nodes,
+# others up to 4.2, with observables 0.6) against the oracle
+@pytest.mark.parametrize("shape", [(8, 8, 8), (9, 11, 13), (33, 20, 17), (64, 40, 24)])
+@pytest.mark.parametrize("scheme,tau,mu64", [("EFDS2", 0.8, 0), ("EFDS4", 1.3, 0), ("EFDS6", 1.0, 0), ("EFDS4", 0.7, 1)])
+def test_d3q19_node_steps(L, shape, scheme, tau, mu64):
+    kw = dict(scheme=scheme, precision=L.LBM_FP32DEV, mu_fp64=mu64, tau=tau)
+    (a, rho), (b, _) = start(L, L.LBM_D3Q19, shape, **kw), start(L, L.LBM_D3Q19, shape, **kw)
+    o = O.Sim(lattice=O.D3Q19, nx=shape[0], ny=shape[1], nz=shape[2], Tr=0.9, k=0.3, kappa=0.1, scheme=scheme, tau=tau)
+    o.set_f(np.stack([w * rho for w in O.lattice(O.D3Q19)[1]]))
+    for _ in range(4):
+        a.lbm_step(1)
+        oo = o.observables()
+        ob = b.lbm_step_observe(1)  # of the state before the step, like the oracle's
+        assert o.step(1) == 0
+        for key in ("max_v", "max_u"):
+            assert ob[key] == pytest.approx(oo[key], rel=1e-3, abs=1e-6), key
+        assert ob["mass"] == pytest.approx(oo["mass"], rel=1e-6)
+    # FP32: a few roundings of 2^-24 of a population a step
+    assert np.max(np.abs(a.lbm_get_density() - o.density())) / 0.15 < 1e-5
+    assert np.max(np.abs(a.lbm_get_f() - o.get_f().reshape(a.lbm_get_f().shape))) / 0.15 < 1e-5
+    assert np.array_equal(a.lbm_get_f(), b.lbm_get_f())
+
+
+@pytest.mark.parametrize("shape", [(104, 104, 108), (160, 100, 75), (161, 161, 162), (161, 161, 161), (80, 75, 100), (84, 75, 100)])
+def test_d3q19_node_range(L, shape):
+    kw = dict(scheme="EFDS4", precision=L.LBM_FP32DEV, tau=0.8)
+    a, rho = start(L, L.LBM_D3Q19, shape, **kw)
+    b, _ = start(L, L.LBM_D3Q19, shape, **dict(kw, precision=L.LBM_FP64))
+    ob = [a.lbm_step_observe(1), b.lbm_step_observe(1)]
+    assert ob[0]["max_u"] == pytest.approx(ob[1]["max_u"], rel=1e-3, abs=1e-6)
+    a.lbm_step(2)
+    b.lbm_step(2)
+    assert np.max(np.abs(a.lbm_get_density() - b.lbm_get_density())) / 0.15 < 1e-5
