@@ -127,7 +127,8 @@ cudaError_t coll3d_gf_step(const Launch& c, int* nblocks);
 // end of the kernel before it in the stream (programmatic dependent launch).
 // Dependent kernels of a few microseconds otherwise start on a 2 us grid here.
 template <class... P, class... A>
-inline cudaError_t launch_pdl(void (*k)(P...), dim3 grid, dim3 threads, size_t smem, cudaStream_t st, A... args) {
+inline cudaError_t launch_if_pdl(bool pdl, void (*k)(P...), dim3 grid, dim3 threads, size_t smem, cudaStream_t st,
+                                 A... args) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;
   cfg.blockDim = threads;
@@ -137,8 +138,12 @@ inline cudaError_t launch_pdl(void (*k)(P...), dim3 grid, dim3 threads, size_t s
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = pdl ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, k, P(args)...);
+}
+template <class... P, class... A>
+inline cudaError_t launch_pdl(void (*k)(P...), dim3 grid, dim3 threads, size_t smem, cudaStream_t st, A... args) {
+  return launch_if_pdl(true, k, grid, threads, smem, st, args...);
 }
 
 #ifdef __CUDACC__

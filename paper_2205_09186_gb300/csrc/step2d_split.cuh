@@ -15,6 +15,7 @@
 // Both are device functions so that the single-case kernels and the
 // persistent batch kernel share them.
 #pragma once
+#include "launch.cuh"
 #include "lbm_device.cuh"
 #include "step2d.cuh"
 
@@ -326,6 +327,7 @@ template <int S>
 __global__ void __launch_bounds__(YMT) k_mu2d_ym(const KParams p, const float* __restrict__ rin,
                                                  float* __restrict__ mu, const int rpt) {
   static_assert(!Sch<S>::ISO && Sch<S>::R <= 4, "line schemes, stencil within one chunk on each side");
+  pdl_wait();
   constexpr int R = Sch<S>::R;
   const int nx = p.nx, ny = p.ny;
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
@@ -413,6 +415,7 @@ template <int S, int RPT>
 __global__ void __launch_bounds__(NT2S) k_mu2d(const KParams p, const float* __restrict__ rin, float* __restrict__ mu) {
   [[maybe_unused]] constexpr int M2Y = Tile2<RPT>::M2Y, C2Y = Tile2<RPT>::C2Y, T2Y = Tile2<RPT>::T2Y, C2N = Tile2<RPT>::C2N;
   extern __shared__ __align__(16) unsigned char smem[];
+  pdl_wait();
   mu2d_tile<S, RPT>(p, rin, mu, blockIdx.x * M2X, blockIdx.y * M2Y, smem);
 }
 
@@ -423,6 +426,7 @@ __global__ void __launch_bounds__(NT2S) k_coll2d(const KParams p, const float* _
                                                  const StepAux aux, const Mrt mrt) {
   [[maybe_unused]] constexpr int M2Y = Tile2<RPT>::M2Y, C2Y = Tile2<RPT>::C2Y, T2Y = Tile2<RPT>::T2Y, C2N = Tile2<RPT>::C2N;
   extern __shared__ __align__(16) unsigned char smem[];
+  pdl_wait();
   coll2d_tile<S, TAU1, RPT>(p, fin, fout, rin, mu, rout, aux.bad_step, aux.t, blockIdx.x * T2X, blockIdx.y * T2Y, smem,
                        mrt);
 }

@@ -170,3 +170,28 @@ def test_d3q19_node_range(L, shape):
     a.lbm_step(2)
     b.lbm_step(2)
     assert np.max(np.abs(a.lbm_get_density() - b.lbm_get_density())) / 0.15 < 1e-5
+
+
+# D2Q9 steps at any tau and MRT: node-parallel up to 32768 nodes (181^2 and 128 x 256
+# below and at the line, 129 x 255 beyond it), then tiles with overlapped launches
+# (350 x 400: more tiles than SMs), against the oracle
+@pytest.mark.parametrize("shape", [(8, 8, 1), (33, 17, 1), (181, 181, 1), (128, 256, 1), (129, 255, 1), (350, 400, 1)])
+@pytest.mark.parametrize("scheme,tau,mrt", [("EFDS2", 0.8, 0), ("EFDS4", 1.0, 1), ("EFDS6", 1.3, 0), ("E4", 0.9, 1), ("E8", 0.9, 0)])
+def test_d2q9_steps_with_relaxation(L, shape, scheme, tau, mrt):
+    kw = dict(scheme=scheme, precision=L.LBM_FP32DEV, tau=tau, collision=mrt)
+    a, rho = start(L, L.LBM_D2Q9, shape, **kw)
+    b, _ = start(L, L.LBM_D2Q9, shape, **dict(kw, precision=L.LBM_FP64))
+    a.lbm_step(3)
+    a.lbm_step(1)
+    b.lbm_step(4)
+    # FP32: a few roundings of 2^-24 of a population a step
+    assert np.max(np.abs(a.lbm_get_density() - b.lbm_get_density())) / 0.15 < 1e-5
+    assert np.max(np.abs(a.lbm_get_f() - b.lbm_get_f())) / 0.15 < 1e-5
+    oa, ob = a.lbm_observables(), b.lbm_observables()
+    assert oa["status"] == ob["status"] == 0
+    assert oa["mass"] == pytest.approx(ob["mass"], rel=1e-6)
+    if shape[0] * shape[1] < 1000 and not mrt:
+        o = O.Sim(lattice=O.D2Q9, nx=shape[0], ny=shape[1], Tr=0.9, k=0.3, kappa=0.1, scheme=scheme, tau=tau)
+        o.set_f(np.stack([w * rho[0] for w in O.lattice(O.D2Q9)[1]]))
+        assert o.step(4) == 0
+        assert np.max(np.abs(a.lbm_get_density() - o.density())) / 0.15 < 1e-5
