@@ -457,7 +457,11 @@ __global__ void k_import_f(KParams p, int Q, const double* in, Tf* f) {
 template <typename Tr>
 __global__ void k_obs_final(const double* part, int nb, const Tr* rho, double rho_ref, long long center,
                             const unsigned long long* bad, double* out, lbm_obs* rec, long long t_obs, long long dt) {
+  pdl_wait();
   __shared__ double red[4][256];
+  // maxima of magnitudes, never NaN (the partials' own maxima pass it over): ordered
+  // as the integers of their bits (an FP64 instruction takes 64 clocks here)
+  auto fmax = [](double x, double y) { return __double_as_longlong(x) > __double_as_longlong(y) ? x : y; };
   double a = 0, b = 0, c = 0, d = 0;
   for (int i = threadIdx.x; i < nb; i += blockDim.x) {
     a = fmax(a, part[4 * i]);
@@ -1027,11 +1031,11 @@ static int finish_observables(lbm_handle* h, int nb, const void* rho_obs, long l
   lbm_obs* rec = async ? reinterpret_cast<lbm_obs*>(h->d_obs + 8) : nullptr;
   const long long dt = t_obs > h->t_snap ? t_obs - h->t_snap : 0;
   if (h->p.precision == LBM_FP64)
-    k_obs_final<double><<<1, 256, 0, h->stream>>>(h->d_partials, nb, static_cast<const double*>(rho_obs), 0.0, center,
-                                                  h->d_bad, h->d_obs, rec, t_obs, dt);
+    launch_pdl(k_obs_final<double>, 1, 256, 0, h->stream, h->d_partials, nb, static_cast<const double*>(rho_obs), 0.0,
+               center, h->d_bad, h->d_obs, rec, t_obs, dt);
   else
-    k_obs_final<float><<<1, 256, 0, h->stream>>>(h->d_partials, nb, static_cast<const float*>(rho_obs),
-                                                 h->kp.rho_ref, center, h->d_bad, h->d_obs, rec, t_obs, dt);
+    launch_pdl(k_obs_final<float>, 1, 256, 0, h->stream, h->d_partials, nb, static_cast<const float*>(rho_obs),
+               h->kp.rho_ref, center, h->d_bad, h->d_obs, rec, t_obs, dt);
   if (async) {
     h->t_snap = t_obs;
     return ck(cudaMemcpyAsync(out, rec, sizeof(lbm_obs), cudaMemcpyDefault, h->stream));

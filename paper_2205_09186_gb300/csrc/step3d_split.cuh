@@ -171,6 +171,7 @@ __global__ void __launch_bounds__(CX* RY_, (CollShape<S, RY_, NB_, FD_>::MINB)) 
                                                     const __grid_constant__ CUtensorMap tmf,
                                                     const float* __restrict__ gmu, const float* __restrict__ grho,
                                                     unsigned long long* __restrict__ qc, const float qscale) {
+  pdl_wait();
   using L = Lattice<1>;
   using Sh = CollShape<S, RY_, NB_, FD_>;
   constexpr int Q = 19, R = Sh::R, GW = Sh::GW, NS = Sh::NS, FPL = Sh::FPL;
@@ -659,16 +660,16 @@ __global__ void __launch_bounds__(CX* RY_, (CollShape<S, RY_, NB_, FD_>::MINB)) 
 __global__ void __launch_bounds__(256) k_coll3d_corners(const KParams p, int ry, unsigned long long* __restrict__ qc,
                                                         float* __restrict__ rout, const float inv_qscale,
                                                         unsigned long long* bad, long long t1) {
+  pdl_wait();
   const ColTiles tiles(p.nx);
   const RowBands bands(p.ny, ry);
-  const long long n = 4LL * tiles.nt * bands.nb * p.nz;
+  const unsigned n = 4u * tiles.nt * bands.nb * p.nz;  // (fewer than the nodes: 32 bits)
   const float rref = float(p.rho_ref);
-  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
-    const int c = int(k & 3);
-    const long long r = k >> 2;
-    const int t = int(r % tiles.nt);
-    const long long r2 = r / tiles.nt;
-    const int b = int(r2 % bands.nb), z = int(r2 / bands.nb);
+  for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+    const int c = int(k & 3u);
+    const unsigned r = k >> 2, r2 = r / unsigned(tiles.nt);
+    const int t = int(r - r2 * tiles.nt);
+    const int z = int(r2 / unsigned(bands.nb)), b = int(r2 - unsigned(z) * bands.nb);
     const int x = (c & 1) ? tiles.start(t + 1) - 1 : tiles.start(t);
     const int y = (c & 2) ? bands.start(b + 1) - 1 : bands.start(b);
     const long long q = (long long)qc[k];
