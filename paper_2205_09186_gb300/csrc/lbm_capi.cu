@@ -868,9 +868,12 @@ extern "C" int lbm_autotune(lbm_handle* h, int* zc_out) {
     for (int round = 0; round < 3 && rc == LBM_OK; ++round) {
       for (int j = 0; j < 3; ++j) {
         h->rpt2d = shapes[j];
-        if ((rc = lbm_step(h, 2)) != LBM_OK) break;  // warm up
+        // single steps: at tau = 1 longer calls run on the moments, whose tiles
+        // these shapes are not
+        if ((rc = lbm_step(h, 1)) != LBM_OK) break;  // warm up
         cudaEventRecord(e0, h->stream);
-        if ((rc = lbm_step(h, 10)) != LBM_OK) break;
+        for (int k = 0; k < 10 && rc == LBM_OK; ++k) rc = lbm_step(h, 1);
+        if (rc != LBM_OK) break;
         cudaEventRecord(e1, h->stream);
         if (cudaEventSynchronize(e1) != cudaSuccess) { rc = LBM_ECUDA; break; }
         float ms = 0.f;
@@ -900,9 +903,11 @@ extern "C" int lbm_autotune(lbm_handle* h, int* zc_out) {
     if (zc == prev || (zc < 4 && nzc > 1)) continue;
     prev = zc;
     h->zc = zc;
-    if (lbm_step(h, 1) != LBM_OK) break;
+    // single steps: at tau = 1 longer calls run on the moments, which this does not cut
+    int rc = lbm_step(h, 1);
     cudaEventRecord(e0, h->stream);
-    if (lbm_step(h, 3) != LBM_OK) break;
+    for (int k = 0; k < 3 && rc == LBM_OK; ++k) rc = lbm_step(h, 1);
+    if (rc != LBM_OK) break;
     cudaEventRecord(e1, h->stream);
     if (cudaEventSynchronize(e1) != cudaSuccess) break;
     float ms = 0.f;
