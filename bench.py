@@ -1,5 +1,5 @@
 #!/usr/bin/env python
-"""Benchmark: fused D3Q19 chemical-potential LBM step on one GB300.
+"""Benchmark: D3Q19 chemical-potential LBM step on one GB300.
 
 Workload (one step = one full time step of the hot path over the lattice):
 D3Q19, 256^3 periodic, droplet r0 = 60, Carnahan-Starling EOS (a=1, b=4,
@@ -31,14 +31,15 @@ METRIC = "MLUPS & HBM-peak fraction of fused step; device-s to converged sweep v
 UNIT = "MLUPS"
 WORKLOAD = dict(lattice="D3Q19", nx=256, ny=256, nz=256, radius=60.0, Tr=0.8, k=0.25, kappa=0.1, tau=1.0,
                 scheme="EFDS6", precision="FP32DEV", mu="fp32")
-# algorithmic bytes per lattice update of the step: read + write the 19 FP32
-# populations (152), read + write the FP32 density deviation (8), write + read
-# the FP32 chemical potential field of the mu pass (8)
-B_ALG = 19 * 4 * 2 + 4 * 2 + 4 * 2
-# of which the collision/streaming pass (the dominant kernel) moves: populations
-# read + write, density read + write, mu read
-B_COLL = 19 * 4 * 2 + 4 * 2 + 4
+# algorithmic bytes per lattice update of a step of one lbm_step call at tau = 1,
+# which carries the moments (density deviation and momentum, FP32): the mu pass
+# reads the density and writes mu, the moment pass reads density, momentum and mu
+# and writes density and momentum
 B_MU = 4 + 4
+B_MOM = 4 * (1 + 3 + 1) + 4 * (1 + 3)
+# and once per call, beside the steps: the 19 populations and the density into
+# moments, and back
+B_CALL = (19 * 4 + 4 + 16) + (20 + 19 * 4 + 4)
 SAMPLE_N = 128  # oracle sample lattice (same parameters, radius scaled)
 
 
@@ -115,10 +116,9 @@ class ClockSampler:
                 "reasons": reasons, "samples": len(rows)}
 
 
-KERNEL_SOURCES = ["paper_2205_09186_gb300/csrc/step3d_split.cuh", "paper_2205_09186_gb300/csrc/lbm_device.cuh",
-                  "paper_2205_09186_gb300/csrc/step3d_fast.cuh", "paper_2205_09186_gb300/csrc/step3d.cuh",
-                  "paper_2205_09186_gb300/csrc/step3d_mu.cuh", "paper_2205_09186_gb300/csrc/coll3d_launch.cuh"]
-TRAFFIC_FILE = "profiles/k_coll3d_d3q19_fp32dev_traffic.txt"
+KERNEL_SOURCES = ["paper_2205_09186_gb300/csrc/mom3d.cuh", "paper_2205_09186_gb300/csrc/mom3d.cu",
+                  "paper_2205_09186_gb300/csrc/pack2.cuh"]
+TRAFFIC_FILE = "profiles/k_mom3d_d3q19_fp32dev_traffic.txt"
 
 
 def kernel_hash():
@@ -131,7 +131,7 @@ def kernel_hash():
 
 
 def captured_traffic(n_nodes):
-    """DRAM bytes per launch of the collision pass from the committed ncu
+    """DRAM bytes per launch of the moment pass from the committed ncu
     capture, scaled to n_nodes by bytes per lattice update; None when the
     kernel sources changed since the capture."""
     try:
@@ -226,7 +226,7 @@ def run_batch(L, steps=50, warmup=10, ncases=512, schemes=None):
             "schemes": sorted(by_scheme), "nodes": nodes, "steps": steps, "ms": ms,
             "mlups": nodes * steps / (ms * 1e-3) / 1e6,
             "mlups_stable_cases": stable_nodes * steps / (ms * 1e-3) / 1e6,
-            "hbm_frac": nodes * steps * (9 * 4 * 2 + 4 * 2) / (ms * 1e-3) / 1e9 / measured_peak()[0],
+            "hbm_frac": nodes * (steps * (3 + 3) * 4 + 80) / (ms * 1e-3) / 1e9 / measured_peak()[0],
             "stable_cases": stable, "cases_stable_by_scheme": by_scheme, "work_items": nitems,
             "resident_ctas": grid, "tile_rows_per_thread": rows, "status": rc}
 
@@ -263,7 +263,8 @@ def run_cfg2_sweep(L, steps=50, warmup=5):
 def run_2d(L, steps=200, warmup=20):
     """D2Q9 512^2 droplet (r0 = 100, T_r = 0.8, k = 0.25, EFDS6, FP32 deviation
     storage): BGK and the MRT operator of Eq. 1, 3-5; MLUPS and the roofline of
-    the collision pass (84 B per lattice update); the same droplet on a wall."""
+    the step: BGK at tau = 1 on the moments (24 B per lattice update, and 80 a call),
+    MRT's collision pass (84 B); the same droplet on a wall."""
     import numpy as np
     import torch
     out = {"workload": "D2Q9 512^2 droplet r0=100, T_r 0.8, k 0.25, EFDS6, FP32DEV, tau 1"}
@@ -280,7 +281,7 @@ def run_2d(L, steps=200, warmup=20):
         coll_ms = ms[1] / steps
         out[col.lower()] = {"mlups": n * steps / (ms[2] * 1e-3) / 1e6, "ms_per_step": ms[2] / steps,
                             "coll_ms": coll_ms, "mu_ms": ms[0] / steps,
-                            "coll_frac": 84 * n / (coll_ms * 1e-3) / 1e9 / measured_peak()[0],
+                            "coll_frac": (84 if col == "MRT" else 24 + 80 / steps) * n / (coll_ms * 1e-3) / 1e9 / measured_peak()[0],
                             "tile_rows_per_thread": rows, "status": s.lbm_observables()["status"]}
         s.close()
     # a lattice larger than L2: 4096^2 (1.2 GB of populations), r0 = 800
@@ -294,7 +295,7 @@ def run_2d(L, steps=200, warmup=20):
     ms = s.lbm_step_timed(20)
     n = 4096 * 4096
     out["bgk_4096"] = {"mlups": n * 20 / (ms[2] * 1e-3) / 1e6, "ms_per_step": ms[2] / 20, "coll_ms": ms[1] / 20,
-                       "mu_ms": ms[0] / 20, "coll_frac": 84 * n / (ms[1] / 20 * 1e-3) / 1e9 / measured_peak()[0],
+                       "mu_ms": ms[0] / 20, "coll_frac": (24 + 80 / 20) * n / (ms[1] / 20 * 1e-3) / 1e9 / measured_peak()[0],
                        "tile_rows_per_thread": rows,
                        "status": s.lbm_observables()["status"]}
     s.close()
@@ -342,7 +343,7 @@ def run_compact(L, steps=20, warmup=5, n=192):
 def run_cfg3_legs(L, zc, steps=20, warmup=5, n=256, check_steps=300):
     """The 256^3 droplet (r0 = 60, EFDS6, FP32 deviation storage) at the other
     temperatures of the configuration and with the FP64 chemical potential:
-    MLUPS, the step's HBM fraction at 168 B per lattice update, and the status
+    MLUPS, the step's HBM fraction at its bytes per lattice update, and the status
     after check_steps steps (first bad step if unstable).  At T_r 0.2 the
     k = 0.25 droplet goes unstable (the oracle on the same droplet scaled to
     96^3 fails at the same step as the GPU there); it is recorded, and the
@@ -365,7 +366,7 @@ def run_cfg3_legs(L, zc, steps=20, warmup=5, n=256, check_steps=300):
         o = s.lbm_observables()
         out[name] = {"Tr": Tr, "k": k, "mu": "fp64" if mu64 else "fp32", "mlups": n ** 3 * steps / (ms[2] * 1e-3) / 1e6,
                      "ms_per_step": ms[2] / steps,
-                     "step_frac": B_ALG * n ** 3 / (ms[2] / steps * 1e-3) / 1e9 / peak,
+                     "step_frac": (B_MU + B_MOM + B_CALL / steps) * n ** 3 / (ms[2] / steps * 1e-3) / 1e9 / peak,
                      "status": o["status"], "steps_checked": check_steps,
                      "first_bad_step": o["step"] if o["status"] != 0 else None,
                      "rho_center": o["rho_center"], "rho_corner": o["rho_corner"], "max_v": o["max_v"]}
@@ -467,8 +468,8 @@ def run_gpu(args):
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     with ClockSampler(local) as clk:
         e0.record(stream)
-        # one step per launch group; CUDA events between the mu pass and the
-        # collision pass time the dominant kernel on the handle's own stream
+        # CUDA events around the mu passes time them and the rest, on the handle's
+        # own stream
         phase_ms = sim.lbm_step_timed(args.steps)
         e1.record(stream)
         torch.cuda.synchronize()
@@ -479,9 +480,11 @@ def run_gpu(args):
     obs = sim.lbm_observables()
     ok = obs["status"] == 0 and abs(obs["mass"] / obs0["mass"] - 1) < 1e-6
     mlups = job_mlups(N, args.steps, world, total_ms)
-    coll_ms = phase_ms[1] / args.steps   # collision/streaming pass (dominant kernel), per launch
+    coll_ms = phase_ms[1] / args.steps   # moment pass (dominant kernel), with gather and expansion / steps
     mu_ms = phase_ms[0] / args.steps     # mu pass, per launch
-    achieved = B_COLL * N / (coll_ms * 1e-3) / 1e9
+    # the moment passes with the call's gather and expansion, whose bytes count once
+    b_mom = B_MOM + B_CALL / args.steps
+    achieved = b_mom * N / (coll_ms * 1e-3) / 1e9
     peak, peak_kind = measured_peak()
 
     # end to end through the public API with pinned host buffers: upload the
@@ -560,13 +563,13 @@ def run_gpu(args):
                            **WORKLOAD),
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "traffic": captured_traffic(N), "peak_kind": peak_kind,
-                         "bytes_per_lu": B_COLL,
-                         "kernel": "k_coll3d (grad mu, grad rho, force, BGK+EDM, push, next density)"
-                                   " + k_coll3d_corners (tile-corner densities), timed together",
-                         "kernel_ms": coll_ms, "mu_pass": {"kernel": "k_mu3d_zm", "ms": mu_ms, "bytes_per_lu": B_MU,
+                         "bytes_per_lu": b_mom,
+                         "kernel": "k_mom3d (grad mu, grad rho, force, equilibrium, streaming of the moments)"
+                                   " + k_mom_gather and k_mom_expand once per call, timed together",
+                         "kernel_ms": coll_ms, "mu_pass": {"kernel": "k_mom_mu", "ms": mu_ms, "bytes_per_lu": B_MU,
                                                            "achieved": B_MU * N / (mu_ms * 1e-3) / 1e9 if mu_ms > 0 else None},
-                         "step_bytes_per_lu": B_ALG, "step_frac": B_ALG * N / (total_ms / args.steps * 1e-3) / 1e9 / peak},
-            "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": 3 * args.steps,
+                         "step_bytes_per_lu": B_MU + b_mom, "step_frac": (B_MU + b_mom) * N / (total_ms / args.steps * 1e-3) / 1e9 / peak},
+            "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": 2 * args.steps + 2,
             "clocks": clk.summary(), "check": {"status": obs["status"], "mass_rel_change": obs["mass"] / obs0["mass"] - 1,
                                                "ok": ok},
             "extra": extra}

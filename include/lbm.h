@@ -269,9 +269,9 @@ long long lbm_get_step(const lbm_handle* h);
  * next lbm_step. */
 int lbm_device_state(lbm_handle* h, void** f, void** rho);
 
-/* Work decomposition.  D3Q19 FP32DEV step (explicit schemes, and the
- * compact schemes' collision pass when nx % 4 == 0): each CTA
- * marches through a chunk of zc planes; lbm_set_zchunk fixes zc (0 = the
+/* Work decomposition.  D3Q19 FP32DEV step on the populations (explicit schemes
+ * above about a million nodes, and the compact schemes' collision pass when nx % 4
+ * == 0): each CTA marches through a chunk of zc planes; lbm_set_zchunk fixes zc (0 = the
  * built-in heuristic, which balances the last wave of CTAs against the
  * per-chunk prologue).  D2Q9 FP32DEV split step (explicit and isotropic
  * schemes, no walls): tiles of 16 x rows-per-thread rows; lbm_set_tile_rows
@@ -373,13 +373,14 @@ int lbm_observables_noalloc(const lbm_params* p, const void* d_f, const void* d_
  * must share lattice (LBM_D2Q9), precision and mu_fp64; schemes may differ
  * freely, the compact ones included (Eq. 21-24 and OCFDS4 of Sec. 3.1: their
  * steps add a chemical-potential phase where the precision needs one, and a
- * phase of periodic tridiagonal line solves along x and y, groups of lines
+ * phase of periodic line solves along x and y, groups of lines
  * being work items of the same launch, each phase behind the barrier).  Each
  * case owns its own populations and density; lbm_batch_step runs n steps of
- * every case in ONE persistent kernel launch whose resident CTAs fetch
+ * every case in one persistent kernel launch whose resident CTAs fetch
  * (case, tile) work items dynamically and meet at a device-wide barrier
- * between steps; the launch is captured in a CUDA graph (one per distinct n)
- * and replayed.  Barrier waits are bounded (about one second): if a wait runs
+ * between steps (FP32DEV cases at tau = 1 advance on their moments, in a launch
+ * of their own; an odd step, and the other cases, in another); the launches are
+ * captured in a CUDA graph (one per distinct n) and replayed.  Barrier waits are bounded (about one second): if a wait runs
  * out the kernel returns and lbm_batch_observables reports LBM_ETIMEOUT.
  */
 typedef struct lbm_batch lbm_batch;
