@@ -1,5 +1,7 @@
 // Batched D2Q9 droplets of uneven sizes and parameters in one persistent
-// launch.  In FP32-deviation batches (k_batch_split) the CTAs (collision
+// launch.  Cases of FP32-deviation batches at tau = 1 advance on their moments, an
+// even number of steps per call (k_batch_mom, a launch of its own); an odd step and
+// the other cases run on the populations.  There (k_batch_split) the CTAs (collision
 // items) and warps (mu units) claim the work of each phase from an atomic
 // counter in guided runs; other precisions (k_batch_persistent) fetch their
 // (case, tile) items one at a time from an atomic counter per phase.
@@ -11,7 +13,7 @@
 // fields.
 // Steps and phases are separated by a device-wide barrier whose waits are
 // bounded (about one second), after which the kernel records LBM_ETIMEOUT and
-// returns.  lbm_batch_step captures the launch (plus the counter reset) in a
+// returns.  lbm_batch_step captures the launches (plus the counter resets) in a
 // CUDA graph and replays it; lbm_batch_autotune picks the tile shape.
 #include <cuda_runtime.h>
 

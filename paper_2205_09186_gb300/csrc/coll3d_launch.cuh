@@ -35,10 +35,11 @@ cudaError_t launch_coll(const Launch& c, int zc) {
   const ColTiles tiles(c.kp.nx);
   const RowBands bands(c.kp.ny, RY);
   const dim3 grid(tiles.nt, bands.nb, (c.kp.nz + zc - 1) / zc);
-  // overlapped with the mu pass only where all CTAs are resident at once: dealt early,
-  // the CTAs of a longer grid no longer march neighbouring tiles together (256^3
-  // EFDS6: 664 us a step so, 610 with the corner kernel overlapped, 613 with neither).
-  // The mu pass itself is not: some runs at 256^3 then took 8% longer.
+  // overlapped with the mu pass, and the corner kernel with it, only where all CTAs
+  // are resident at once (3D lattices of 1 to 2 million nodes: 4 to 7% off a step).
+  // Dealt early, the CTAs of a longer grid no longer march neighbouring tiles together
+  // (256^3 EFDS6: 664 us a step against 613; with the corner kernel overlapped 610,
+  // but some runs 5% more).
   const bool pdl = (long long)grid.x * grid.y * grid.z <= (long long)Sh::MINB * device_sms();
   cudaError_t e = launch_if_pdl(pdl, kc, grid, Sh::NT, by, c.stream, c.kp, static_cast<const float*>(c.fin),
                              static_cast<float*>(c.fout), static_cast<const float*>(c.rin),
@@ -48,8 +49,8 @@ cudaError_t launch_coll(const Launch& c, int zc) {
   if (e != cudaSuccess) return e;
   const long long ncorner = 4LL * tiles.nt * bands.nb * c.kp.nz;
   const int nblk = int(std::min<long long>((ncorner + 255) / 256, 4096LL));
-  return launch_pdl(k_coll3d_corners, nblk, 256, 0, c.stream, c.kp, RY, c.qc, static_cast<float*>(c.rout), 1.f / c.qscale,
-                    c.aux.bad_step, c.aux.t + 1);
+  return launch_if_pdl(pdl, k_coll3d_corners, nblk, 256, 0, c.stream, c.kp, RY, c.qc, static_cast<float*>(c.rout), 1.f / c.qscale,
+                       c.aux.bad_step, c.aux.t + 1);
 }
 
 }  // namespace lbmd
