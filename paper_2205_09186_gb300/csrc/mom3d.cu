@@ -78,8 +78,8 @@ cudaError_t steps(const Launch& c, int scheme, long long n) {
   float* j[2] = {s + 2 * g.P, s + 5 * g.P};
   float *mu = s + 8 * g.P, *acc = s + 9 * g.P;
   const int elems = g.PL * kp.nz;
-  k_mom_gather<<<(elems + 255) / 256, 256, 0, c.stream>>>(kp, g, fin, rin, r[0], j[0], r[1], mu, j[1], c.aux.bad_step,
-                                                          c.aux.t);
+  k_mom_gather<<<(elems + 255) / 256, 256, 0, c.stream>>>(kp, g, fin, rin, r[0], j[0], r[1], mu, j[1],
+                                                          GF ? acc : nullptr, c.aux.bad_step, c.aux.t);
   // mu pass: about eight CTAs per SM; at least eight planes each, down to two
   // where that leaves SMs without a CTA (a plane is a round trip to L2)
   const int gm = ((kp.nx + 3) / 4 * kp.ny + 255) / 256;

@@ -102,12 +102,14 @@ struct Post2 {
 // ------------------------------------------------------------------ gather
 // One thread per element of a padded row: the moments at the lattice's nodes,
 // the periodic copies of rho beside them, zeros in the rest of every field
-// (rb, mu and jb are the step's other buffers).
+// (rb, mu, jb and, with a compact scheme, the three fields acc are the step's
+// other buffers).  A row's last pair of nodes reads one element of it where nx is
+// odd; its populations are masked by a factor of zero, so it has to be finite.
 __global__ void __launch_bounds__(256) k_mom_gather(const KParams p, const MomGeo g, const float* __restrict__ f,
                                                     const float* __restrict__ rho, float* __restrict__ ra,
                                                     float* __restrict__ ja, float* __restrict__ rb,
                                                     float* __restrict__ mu, float* __restrict__ jb,
-                                                    unsigned long long* bad, long long t) {
+                                                    float* __restrict__ acc, unsigned long long* bad, long long t) {
   using L = Lattice<1>;
   const int e = blockIdx.x * 256 + threadIdx.x;
   if (e >= g.PL * p.nz) return;
@@ -137,7 +139,10 @@ __global__ void __launch_bounds__(256) k_mom_gather(const KParams p, const MomGe
     rb[e] = 0.f;
     mu[e] = 0.f;
 #pragma unroll
-    for (int a = 0; a < 3; ++a) ja[e + a * g.P] = jb[e + a * g.P] = 0.f;
+    for (int a = 0; a < 3; ++a) {
+      ja[e + a * g.P] = jb[e + a * g.P] = 0.f;
+      if (acc) acc[e + a * g.P] = 0.f;
+    }
   }
 }
 
