@@ -275,8 +275,10 @@ int lbm_device_state(lbm_handle* h, void** f, void** rho);
  * built-in heuristic, which balances the last wave of CTAs against the
  * per-chunk prologue).  D2Q9 FP32DEV split step (explicit and isotropic
  * schemes, no walls): tiles of 16 x rows-per-thread rows; lbm_set_tile_rows
- * fixes rows per thread (1, 2 or 4; 0 = 2).  lbm_autotune times the
- * candidates on this handle's lattice and keeps the fastest: chunk lengths
+ * fixes rows per thread (1, 2 or 4; 0 = 2).  Neither reaches the steps that carry
+ * the moments (lbm_step) or those of small lattices, which run one thread per
+ * node.  lbm_autotune times the
+ * candidates on this handle's lattice, on the passes they cut, and keeps the fastest: chunk lengths
  * over a few steps each, tile rows in three interleaved rounds of ten steps
  * (each shape's fastest round counting); the steps run on the handle's
  * state, which is left undefined (initialise after tuning).  *zc_out

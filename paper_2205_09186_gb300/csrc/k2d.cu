@@ -109,7 +109,7 @@ cudaError_t launch_split2d(const Launch& c, int* nblocks) {
 template <int S, class P>
 cudaError_t launch(const Launch& c, int mode, int* nblocks) {
   if constexpr (std::is_same<P, PrecF32>::value) {
-    if (mode == MODE_STEP && c.mu && node2_rule(c.kp)) return launch_node2<S>(c, nblocks);
+    if (mode == MODE_STEP && c.mu && !c.tiled && node2_rule(c.kp)) return launch_node2<S>(c, nblocks);
     if (mode == MODE_STEP && c.mu)
       return c.kp.omega == 1.0 ? launch_split2d<S, true>(c, nblocks) : launch_split2d<S, false>(c, nblocks);
   }

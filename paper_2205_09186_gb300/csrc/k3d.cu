@@ -181,7 +181,7 @@ cudaError_t launch_split(const Launch& c, int* nblocks, bool obs) {
   if (!c.mu) return cudaErrorInvalidValue;
   // 16-byte copies need rows of whole chunks and aligned bases
   const bool vec = c.kp.nx % 4 == 0 && aligned16(c.fin) && aligned16(c.rin) && aligned16(c.mu) && c.tmap;
-  if (node_rule(c.kp, vec, obs)) return launch_node<S, TAU1, M64>(c, nblocks, obs);
+  if (!c.tiled && node_rule(c.kp, vec, obs)) return launch_node<S, TAU1, M64>(c, nblocks, obs);
   const int zc = c.zc > 0 ? c.zc : split_zchunk_heuristic(c.kp, Sch<S>::R, TYC, CollShape<S, CY, 2, COLL_FD>::MINB);
   const long long ctas = coll3d_ctas(c.kp, zc);
   if (nblocks) {

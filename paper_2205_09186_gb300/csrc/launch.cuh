@@ -25,6 +25,7 @@ struct Launch {
   cudaEvent_t* ev_mu;  // mom3d_steps, if set: recorded before and after each step's mu pass (2 n events)
   const void* tmap;    // D3Q19 FP32DEV: tensor map (CUtensorMap) of the populations fin, or null
   int rpt2d;           // D2Q9 FP32DEV split tiles: rows per thread (1, 2, 4; 0 = default 2)
+  bool tiled;          // the tiled passes on every lattice (what lbm_autotune times), node-parallel ones on none
   // D3Q19 FP32DEV collision pass: corner accumulators (coll3d_corner_count
   // 64-bit integers, zero between passes) and their fixed-point scale
   unsigned long long* qc;

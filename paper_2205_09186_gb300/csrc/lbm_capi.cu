@@ -55,6 +55,7 @@ struct lbm_handle {
   unsigned long long* qc = nullptr;  // D3Q19 FP32DEV: corner accumulators of the collision pass
   long long n_qc = 0;
   float qscale = 0.f;
+  bool tuning = false;  // lbm_autotune: steps run on the tiled passes
   int rpt2d = 0;  // D2Q9 FP32DEV split tiles: rows per thread (0 = default)
 };
 
@@ -811,6 +812,7 @@ static Launch make_launch(lbm_handle* h, int out_buf) {
   c.mrt = h->mrt;
   c.tmap = h->has_tmap ? h->tmap[h->cur] : nullptr;
   c.rpt2d = h->rpt2d;
+  c.tiled = h->tuning;
   c.qc = h->qc;
   c.qscale = h->qscale;
   return c;
@@ -865,11 +867,12 @@ extern "C" int lbm_autotune(lbm_handle* h, int* zc_out) {
     const int shapes[3] = {1, 2, 4};
     float shape_ms[3] = {1e30f, 1e30f, 1e30f};
     int rc = LBM_OK;
+    h->tuning = true;
     for (int round = 0; round < 3 && rc == LBM_OK; ++round) {
       for (int j = 0; j < 3; ++j) {
         h->rpt2d = shapes[j];
-        // single steps: at tau = 1 longer calls run on the moments, whose tiles
-        // these shapes are not
+        // single steps on the tiled passes: at tau = 1 longer calls run on the
+        // moments, on small lattices node-parallel, neither of which these shapes cut
         if ((rc = lbm_step(h, 1)) != LBM_OK) break;  // warm up
         cudaEventRecord(e0, h->stream);
         for (int k = 0; k < 10 && rc == LBM_OK; ++k) rc = lbm_step(h, 1);
@@ -881,6 +884,7 @@ extern "C" int lbm_autotune(lbm_handle* h, int* zc_out) {
         shape_ms[j] = std::min(shape_ms[j], ms);
       }
     }
+    h->tuning = false;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     int best = 0;
@@ -898,12 +902,14 @@ extern "C" int lbm_autotune(lbm_handle* h, int* zc_out) {
   const long long t_saved = h->t;
   int prev = 0, best_zc = 0;
   float best = 1e30f;
+  h->tuning = true;
   for (int nzc = 1; nzc <= 32 && nzc <= h->p.nz; ++nzc) {
     const int zc = (h->p.nz + nzc - 1) / nzc;
     if (zc == prev || (zc < 4 && nzc > 1)) continue;
     prev = zc;
     h->zc = zc;
-    // single steps: at tau = 1 longer calls run on the moments, which this does not cut
+    // single steps on the tiled passes: at tau = 1 longer calls run on the moments, on
+    // smaller lattices node-parallel, neither of which this cuts
     int rc = lbm_step(h, 1);
     cudaEventRecord(e0, h->stream);
     for (int k = 0; k < 3 && rc == LBM_OK; ++k) rc = lbm_step(h, 1);
@@ -914,6 +920,7 @@ extern "C" int lbm_autotune(lbm_handle* h, int* zc_out) {
     cudaEventElapsedTime(&ms, e0, e1);
     if (ms < best) { best = ms; best_zc = zc; }
   }
+  h->tuning = false;
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   h->t = t_saved;

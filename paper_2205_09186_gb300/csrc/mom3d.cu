@@ -26,25 +26,25 @@ MomGeo mom_geo(const KParams& kp) {
   return g;
 }
 
-// rows per band and planes per chunk (zc > 0: that many) together: the waves
+// rows per band and planes per chunk together (the chunk of lbm_set_zchunk belongs to
+// the collision pass on the populations, another kernel): the waves
 // of CTAs (one per SM) times a CTA's planes (two collided beyond the chunk,
 // the prologue worth two more) times the time of a plane, which grows with
 // the rows held (the band, one beyond either side, the edge warp, and about
 // four rows' worth of barrier and latency)
 void mom_cut(const KParams& kp, MomGeo* g, int* zc) {
   const long long slots = device_sms();
-  const int fixed = *zc;
   double best = 1e300;
   for (int nb = (kp.ny + MW3 - 4) / (MW3 - 3); nb <= kp.ny; ++nb) {
     const int rb = (kp.ny + nb - 1) / nb, bands = (kp.ny + rb - 1) / rb;
     if (2 * rb < MW3 - 3 && best < 1e300) break;
     for (int n = 1; n <= kp.nz; ++n) {
-      const int c = fixed > 0 ? fixed : (kp.nz + n - 1) / n;
+      const int c = (kp.nz + n - 1) / n;
       if (c < 2 && n > 1) break;
       const long long ctas = (long long)g->nt * bands * ((kp.nz + c - 1) / c);
       const double cost = double((ctas + slots - 1) / slots) * (c + 4) * (rb + 7);
       if (cost < best - 1e-9) { best = cost; *zc = c; g->RB = rb; g->nb = bands; }
-      if (fixed > 0 || ctas > 8 * slots) break;
+      if (ctas > 8 * slots) break;
     }
   }
 }
@@ -70,7 +70,7 @@ cudaError_t steps(const Launch& c, int scheme, long long n) {
   constexpr bool GF = Sch<S>::GF;
   const KParams& kp = c.kp;
   MomGeo g = mom_geo(kp);
-  int zc = c.zc;
+  int zc = 0;
   mom_cut(kp, &g, &zc);
   const float *fin = static_cast<const float*>(c.fin), *rin = static_cast<const float*>(c.rin);
   float* s = static_cast<float*>(c.fout);  // scratch: rho x 2, j x 2, mu, compact: F / rho

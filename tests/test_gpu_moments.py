@@ -243,3 +243,52 @@ def test_moments_do_not_read_what_memory_held(L, monkeypatch, lattice, shape, sc
 
     for a, b in zip(run(0), run(255)):  # zeros, NaN
         assert np.array_equal(a, b)
+
+
+def best_ms(call, repeats=5, calls=8):
+    import torch
+    out = []
+    for _ in range(repeats):
+        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        call()
+        e0.record()
+        for _ in range(calls):
+            call()
+        e1.record()
+        torch.cuda.synchronize()
+        out.append(e0.elapsed_time(e1) / calls)
+    return min(out)
+
+
+def test_zchunk_does_not_reach_the_moments(L):
+    # chunks of one plane collide three planes for each of theirs (and five more in
+    # the prologue): two to four times the time where they are used
+    kw = dict(lattice=L.LBM_D3Q19, nx=128, ny=128, nz=128, Tr=0.9, k=0.3, kappa=0.1, scheme="EFDS6",
+              precision=L.LBM_FP32DEV)
+    ms = []
+    for zc in (0, 1):
+        s = L.Sim(L.make_params(**kw))
+        s.lbm_set_zchunk(zc)
+        s.lbm_init_droplet(30.0)
+        ms.append(best_ms(lambda: s.lbm_step(20)))
+    assert ms[1] < 1.4 * ms[0], ms
+
+
+def test_autotune_times_the_passes_it_cuts(L):
+    # a million nodes: single steps run node-parallel, observed ones on the tiled
+    # collision pass, whose time depends on the chunk by a factor of two; steps that
+    # do not use it would leave the choice to chance
+    kw = dict(lattice=L.LBM_D3Q19, nx=100, ny=100, nz=100, Tr=0.9, k=0.3, kappa=0.1, scheme="EFDS6",
+              precision=L.LBM_FP32DEV)
+    s = L.Sim(L.make_params(**kw))
+    fixed = {}
+    for zc in (100, 50, 25, 20, 13, 10, 7, 5):
+        s.lbm_set_zchunk(zc)
+        s.lbm_init_droplet(25.0)
+        fixed[zc] = best_ms(lambda: s.lbm_step_observe(1))
+    for _ in range(6):
+        zc = s.lbm_autotune()
+        assert zc > 0
+        s.lbm_init_droplet(25.0)
+        ms = best_ms(lambda: s.lbm_step_observe(1))
+        assert ms < 1.25 * min(fixed.values()), (zc, ms, fixed)
