@@ -422,7 +422,9 @@ int lbm_batch_inject_stall(lbm_batch* b, int cta);
  * it; lbm_batch_autotune times `steps` steps of every shape that has a
  * resident launch configuration (after one captured warm-up launch each), in
  * three interleaved rounds, and keeps the shape with the fastest launch,
- * reported in *rows_out (18 launches of `steps` steps).  The tuning steps run on the
+ * reported in *rows_out (18 launches of `steps` steps; where all cases advance on
+ * their moments, which the shape does not cut, the timed steps run on the
+ * populations as their odd steps do).  The tuning steps run on the
  * batch's state, which they advance: initialise before tuning (the timing
  * is only representative of a physical state) and again after it.  The shapes
  * give identical results (same arithmetic per node).  Errors: LBM_EINVAL,

@@ -732,6 +732,7 @@ struct lbm_batch {
   Item* d_tiles = nullptr;
   MomWork work{};
   int grid_mom = 0, nmu_mom = 0, ncoll_mom = 0, nline_mom = 0;
+  bool populations = false;  // lbm_batch_autotune: every case on the populations
   std::vector<int> case_order;  // split path: cases in work-list order
   // compact-scheme cases: their mu tiles (TXB x TYB), their line groups
   // (rebuilt with the group size lpb of the tile shape), longest line
@@ -1154,7 +1155,7 @@ static cudaError_t launch_persistent(lbm_batch* b, int nsteps) {
   cudaError_t e = reset();
   if (e != cudaSuccess) return e;
   if (b->split) {
-    const int even = b->work.tiles ? nsteps / 2 * 2 : 0;
+    const int even = b->work.tiles && !b->populations ? nsteps / 2 * 2 : 0;
     if (nsteps - even > 0 && (e = launch_split(b, nsteps - even, true)) != cudaSuccess) return e;
     if (even == 0) return e;
     const bool rest = b->nmu > b->nmu_mom;
@@ -1246,6 +1247,9 @@ extern "C" int lbm_batch_autotune(lbm_batch* b, int steps, int* rows_out) {
   const int shapes[3] = {1, 2, 4};
   float shape_ms[3] = {1e30f, 1e30f, 1e30f};
   int rc = LBM_OK;
+  // where every case advances on its moments, only odd steps run on the tiles that
+  // are tuned: all of the timed ones do
+  b->populations = b->nmu == b->nmu_mom;
   for (int round = 0; round < 3 && rc == LBM_OK; ++round) {
     for (int j = 0; j < 3; ++j) {
       if (setup_split(b, shapes[j]) != LBM_OK) continue;  // shape without a resident configuration
@@ -1261,6 +1265,8 @@ extern "C" int lbm_batch_autotune(lbm_batch* b, int steps, int* rows_out) {
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
+  b->populations = false;
+  b->graph_steps = -1;
   if (rc != LBM_OK) return rc;
   int best = 0;
   float best_ms = 1e30f;

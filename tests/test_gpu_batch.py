@@ -274,3 +274,35 @@ def test_batch_compact_on_moments(L, scheme, steps):
         assert np.max(np.abs(da - db)) / np.max(ro) < 1e-6, c
         assert np.max(np.abs(da - ro)) / np.max(ro) < 1e-5, c
         assert oa[i]["mass"] == pytest.approx(ob[i]["mass"], rel=1e-6)
+
+
+def test_batch_autotune_times_the_tiles(L):
+    # every case on its moments: an even number of steps runs none of the tiles that
+    # are tuned, and the choice was chance; odd steps do, and on two small
+    # lattices the taller tiles leave more SMs without one (15 and 40% slower)
+    import torch
+    cases = [dict(nx=100, ny=100, Tr=0.9, k=0.3, scheme="EFDS6", r=25.0)] * 2
+    b = L.Batch([params(L, c, 1) for c in cases])
+
+    def ms():
+        b.lbm_batch_init_droplets([c["r"] for c in cases])
+        out = []
+        for _ in range(5):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            b.lbm_batch_step(1)
+            e0.record()
+            for _ in range(20):
+                b.lbm_batch_step(1)
+            e1.record()
+            torch.cuda.synchronize()
+            out.append(e0.elapsed_time(e1) / 20)
+        return min(out)
+
+    fixed = {}
+    for rows in (1, 2, 4):
+        b.lbm_batch_set_tiles(rows)
+        fixed[rows] = ms()
+    for _ in range(8):
+        rows = b.lbm_batch_autotune(steps=10)
+        t = ms()
+        assert t < 1.08 * min(fixed.values()), (rows, t, fixed)
