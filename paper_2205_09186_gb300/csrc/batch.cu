@@ -777,10 +777,6 @@ static void* balloc(lbm_batch* b, size_t bytes) {
   if (p) b->blocks.push_back({p, bytes ? bytes : 256});
   return p;
 }
-static void* cuda_alloc_b(size_t bytes, void*) {
-  void* p = nullptr;
-  return cudaMalloc(&p, bytes) == cudaSuccess ? p : nullptr;
-}
 static void cuda_free_b(void* p, size_t, void*) { cudaFree(p); }
 
 extern "C" void lbm_batch_destroy(lbm_batch* b) {
@@ -918,7 +914,7 @@ extern "C" int lbm_batch_create(const lbm_params* cases, int n, void* stream, co
   b->n = n;
   b->stream = static_cast<cudaStream_t>(stream);
   if (alloc && alloc->alloc && alloc->free) b->alloc = *alloc;
-  else { b->alloc.alloc = cuda_alloc_b; b->alloc.free = cuda_free_b; b->alloc.ctx = nullptr; }
+  else { b->alloc.alloc = device_malloc; b->alloc.free = cuda_free_b; b->alloc.ctx = nullptr; }
   b->prec = prec0 == LBM_FP64 ? 0 : (mu0 ? 2 : 1);
   b->p.assign(cases, cases + n);
   b->host_cases.resize(n);

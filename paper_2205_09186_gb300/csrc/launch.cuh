@@ -171,6 +171,9 @@ inline cudaError_t ensure_smem(K* fn, size_t bytes) { return ensure_smem(reinter
 // multiprocessor count of the current device (looked up once per device)
 int device_sms();
 
+// cudaMalloc as an allocation callback: null where it fails, with no error left behind
+void* device_malloc(size_t bytes, void*);
+
 // number of CTAs (hence partial results) of the observation pass
 long long step2d_obs_ctas(const KParams& kp);
 long long step3d_obs_ctas(const KParams& kp);

@@ -67,10 +67,6 @@ static void* dalloc(lbm_handle* h, size_t bytes) {
 static void dfree(lbm_handle* h, void* p, size_t bytes) {
   if (p) h->alloc.free(p, bytes == 0 ? 256 : bytes, h->alloc.ctx);
 }
-static void* cuda_alloc_cb(size_t bytes, void*) {
-  void* p = nullptr;
-  return cudaMalloc(&p, bytes) == cudaSuccess ? p : nullptr;
-}
 static void cuda_free_cb(void* p, size_t, void*) { cudaFree(p); }
 
 static size_t f_bytes(const lbm_handle* h) {
@@ -520,6 +516,14 @@ cudaError_t ensure_smem(const void* fn, size_t bytes) {
   return e;
 }
 
+// the allocation callback of handles that bring none
+void* device_malloc(size_t bytes, void*) {
+  void* p = nullptr;
+  if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
+  cudaGetLastError();  // reported by the null pointer: the next launch is not to report it again
+  return nullptr;
+}
+
 int device_sms() {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return 1;
@@ -597,7 +601,7 @@ extern "C" int lbm_create(const lbm_params* params, void* stream, const lbm_allo
   if (alloc && alloc->alloc && alloc->free) {
     h->alloc = *alloc;
   } else {
-    h->alloc.alloc = cuda_alloc_cb;
+    h->alloc.alloc = device_malloc;
     h->alloc.free = cuda_free_cb;
     h->alloc.ctx = nullptr;
     h->own_alloc = true;

@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "../../include/lbm.h"
+#include "launch.cuh"
 
 namespace {
 
@@ -721,10 +722,6 @@ struct lbm_mlp {
 static size_t train_smem(const Net& net) { return size_t(3 * train_rows(net) + (MAXW + TRO) * TS + 4 * TRO * 32) * 4; }
 static size_t train_floats(const Net& net, int Bp) { return size_t(3 * net.nl + 2 + 2 * TC) * MAXW * Bp + TC; }
 
-static void* malloc_cb(size_t b, void*) {
-  void* p = nullptr;
-  return cudaMalloc(&p, b) == cudaSuccess ? p : nullptr;
-}
 static void free_cb(void* p, size_t, void*) { cudaFree(p); }
 
 static float* mget(lbm_mlp* m, size_t floats) {
@@ -751,7 +748,7 @@ extern "C" int lbm_mlp_create(const int* sizes, int nlayers, int max_batch, void
   if (!m) return LBM_ENOMEM;
   m->stream = static_cast<cudaStream_t>(stream);
   if (alloc && alloc->alloc && alloc->free) m->alloc = *alloc;
-  else { m->alloc.alloc = malloc_cb; m->alloc.free = free_cb; m->alloc.ctx = nullptr; }
+  else { m->alloc.alloc = lbmd::device_malloc; m->alloc.free = free_cb; m->alloc.ctx = nullptr; }
   m->net.nl = nlayers;
   long long off = 0;
   size_t act = 0;
