@@ -98,7 +98,7 @@ __device__ __forceinline__ void grad64(const double* q, const Node64<LAT>& c, do
 }
 
 template <int S, int LAT>
-__global__ void k64_mu(const KParams p, const double* __restrict__ rho, double* __restrict__ mu) {
+__global__ void k64_mu(const KParams p, const double* rho, double* __restrict__ mu) {
   pdl_wait();
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= int(p.n)) return;
@@ -200,8 +200,8 @@ __device__ __forceinline__ void post64(const KParams& p, const Mrt& mrt, const d
 // A compact scheme (GF) reads grad mu and grad rho from gi, or F / rho from gi.gmu
 // where gi.grho is null; the others take them from rho and mu.
 template <int S, int LAT, int COLL>
-__global__ void k64_coll(const KParams p, const double* __restrict__ fin, double* __restrict__ fout,
-                         const double* __restrict__ rho, const double* __restrict__ mu, const GradIn gi,
+__global__ void k64_coll(const KParams p, const double* fin, double* __restrict__ fout,
+                         const double* rho, const double* mu, const GradIn gi,
                          const StepAux aux, const Mrt mrt) {
   pdl_wait();
   using L = Lattice<LAT>;
@@ -241,8 +241,8 @@ __global__ void k64_coll(const KParams p, const double* __restrict__ fin, double
 constexpr int T64X = 8, T64Y = 4, T64N = 128;
 
 template <int S, int COLL>
-__global__ void __launch_bounds__(T64N) k64_tile(const KParams p, const double* __restrict__ fin,
-                                                 double* __restrict__ fout, const double* __restrict__ rin,
+__global__ void __launch_bounds__(T64N) k64_tile(const KParams p, const double* fin,
+                                                 double* __restrict__ fout, const double* rin,
                                                  double* __restrict__ rout, const StepAux aux, const Mrt mrt) {
   pdl_wait();
   using L = Lattice<0>;
@@ -303,7 +303,7 @@ __global__ void __launch_bounds__(T64N) k64_tile(const KParams p, const double* 
 }
 
 template <int Q>
-__global__ void k64_rho(const KParams p, const double* __restrict__ f, double* __restrict__ rho,
+__global__ void k64_rho(const KParams p, const double* f, double* __restrict__ rho,
                         unsigned long long* bad, long long t1) {
   pdl_wait();
   const int n = blockIdx.x * blockDim.x + threadIdx.x, N = int(p.n);

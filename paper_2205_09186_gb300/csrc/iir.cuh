@@ -78,8 +78,8 @@ __device__ __forceinline__ double iir_quot(double a, double b) { return a * rcp6
 
 // LS: log2 of the segments; J: how many of them reach (K nodes of at least L >> LS each)
 template <class T, int M, int LS>
-__global__ void __launch_bounds__(32 << LS) k_iir_col(const IirGeo g, const int axis, const T* __restrict__ rho,
-                                                      const T* __restrict__ mu, T* __restrict__ out, const T rref,
+__global__ void __launch_bounds__(32 << LS) k_iir_col(const IirGeo g, const int axis, const T* rho,
+                                                      const T* mu, T* __restrict__ out, const T rref,
                                                       const int J, const IirK<T> c) {
   constexpr int S = 1 << LS;
   __shared__ T s_f[2][S][32], s_b[2][S][32];
@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(32 << LS) k_iir_col(const IirGeo g, const int 
 }
 
 template <class T, int M>
-__global__ void __launch_bounds__(256) k_iir_row(const IirGeo g, const T* __restrict__ rho, const T* __restrict__ mu,
+__global__ void __launch_bounds__(256) k_iir_row(const IirGeo g, const T* rho, const T* mu,
                                                  T* __restrict__ out, const T rref, const int J, const T close,
                                                  const IirK<T> c) {
   extern __shared__ __align__(16) unsigned char sm_iir[];

@@ -127,6 +127,13 @@ cudaError_t coll3d_gf_step(const Launch& c, int* nblocks);
 // Launch a kernel that begins with pdl_wait() so that its launch overlaps the
 // end of the kernel before it in the stream (programmatic dependent launch).
 // Dependent kernels of a few microseconds otherwise start on a 2 us grid here.
+//
+// Such a kernel is resident while the ones before it in the stream still write, so it
+// reads what they wrote by ordinary loads, which the wait orders behind those
+// writes: its inputs are neither const __restrict__ nor read by __ldg.  Either would
+// take the read-only path, which is defined only for data that stays as it is for as
+// long as the reading kernel is resident, its wait included.  (What is constant over
+// the whole chain, such as wall layers, may take it.)
 template <class... P, class... A>
 inline cudaError_t launch_if_pdl(bool pdl, void (*k)(P...), dim3 grid, dim3 threads, size_t smem, cudaStream_t st,
                                  A... args) {

@@ -157,10 +157,11 @@ __device__ __forceinline__ void mom_ghost(float* fld, int o, int x, int nx, floa
 // neighbours in a register queue, x and y neighbours by 16-byte loads that
 // hit L1 (the rows of a CTA are adjacent).  No shared memory and no barrier:
 // the padded rows need no wrap in x and the queue's next plane is loaded one
-// plane ahead.  At 256^3 0.057 ms (the zeroing mu pass of
-// the population steps takes 0.060), bound by issue (69% of cycles).
+// plane ahead.  (__ldca: an ordinary load that the compiler leaves in its place;
+// left to it, EFDS6 takes 0.060 ms at 256^3.)  At 256^3 0.058 ms (the zeroing mu pass
+// of the population steps takes 0.060), bound by issue (69% of cycles).
 template <int S, bool M64>
-__global__ void __launch_bounds__(256) k_mom_mu(const KParams p, const MomGeo g, const float* __restrict__ rin,
+__global__ void __launch_bounds__(256) k_mom_mu(const KParams p, const MomGeo g, const float* rin,
                                                 float* __restrict__ mu, const int zc) {
   pdl_wait();
   constexpr int R = Sch<S>::R;
@@ -176,7 +177,7 @@ __global__ void __launch_bounds__(256) k_mom_mu(const KParams p, const MomGeo g,
     yo[m - 1] = wrapi(y + m, ny) * g.LX + 4 + x;
     yo[R + m - 1] = wrapi(y - m, ny) * g.LX + 4 + x;
   }
-  auto ld = [&](int zo, int o) { return __ldg(reinterpret_cast<const float4*>(rin + zo + o)); };
+  auto ld = [&](int zo, int o) { return __ldca(reinterpret_cast<const float4*>(rin + zo + o)); };
   const float k2 = float(p.k2), kap = float(p.kappa), rref = float(p.rho_ref);
   const EosF ef = eos_f(p);
   const MuConst<M64> mc(p);
@@ -309,8 +310,8 @@ struct MomCell {
   }
   // two nodes of a field at offset zo of a plane
   __device__ __forceinline__ float2 load(const float* q, unsigned zo) const {
-    if (edge) return make_float2(__ldg(q + (zo + oj0)), __ldg(q + (zo + oj1)));
-    return in0 ? __ldg(reinterpret_cast<const float2*>(q + (zo + oj0))) : f2(0.f);
+    if (edge) return make_float2(q[zo + oj0], q[zo + oj1]);
+    return in0 ? *reinterpret_cast<const float2*>(q + (zo + oj0)) : f2(0.f);
   }
   __device__ __forceinline__ void spread(const MomConst& kc, float2 d, float2 r, float2 vx, float2 vy, float2 vz) {
     auto sub = [&](float2 a, float2 b) { return fma2(kc.m1, b, a); };
@@ -440,8 +441,8 @@ struct MomCell {
 };
 
 template <int S, int W>
-__global__ void __launch_bounds__(32 * W, 1) k_mom3d(const KParams p, const MomGeo g, const float* __restrict__ rin,
-                                                     const float* __restrict__ muf, const float* __restrict__ jin,
+__global__ void __launch_bounds__(32 * W, 1) k_mom3d(const KParams p, const MomGeo g, const float* rin,
+                                                     const float* muf, const float* jin,
                                                      float* __restrict__ rout, float* __restrict__ jout,
                                                      unsigned long long* bad, const long long t, const int zc,
                                                      const __grid_constant__ MomConst kc) {
@@ -579,8 +580,8 @@ __global__ void __launch_bounds__(32 * W, 1) k_mom3d(const KParams p, const MomG
 // 230 instructions per node at 52% issue; 24 warps of 80 registers, or two CTAs of
 // 12, spill and take half as long again.
 template <int W>
-__global__ void __launch_bounds__(32 * W, 1) k_mom3d_acc(const KParams p, const MomGeo g, const float* __restrict__ rin,
-                                                         const float* __restrict__ acc, const float* __restrict__ jin,
+__global__ void __launch_bounds__(32 * W, 1) k_mom3d_acc(const KParams p, const MomGeo g, const float* rin,
+                                                         const float* acc, const float* jin,
                                                          float* __restrict__ rout, float* __restrict__ jout,
                                                          unsigned long long* bad, const long long t, const int zc,
                                                          const __grid_constant__ MomConst kc) {

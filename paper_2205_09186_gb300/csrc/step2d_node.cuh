@@ -33,7 +33,7 @@ struct Node2 {
 };
 
 template <int S>
-__global__ void __launch_bounds__(NODE2_T) k_node2_mu(const KParams p, const unsigned mx, const float* __restrict__ rin,
+__global__ void __launch_bounds__(NODE2_T) k_node2_mu(const KParams p, const unsigned mx, const float* rin,
                                                       float* __restrict__ mu) {
   pdl_wait();
   using Sc = Sch<S>;
@@ -61,9 +61,9 @@ __global__ void __launch_bounds__(NODE2_T) k_node2_mu(const KParams p, const uns
 
 // COLL: 0 single relaxation at tau = 1, 1 at any tau, 2 MRT
 template <int S, int COLL>
-__global__ void __launch_bounds__(NODE2_T) k_node2_coll(const KParams p, const unsigned mx, const float* __restrict__ fin,
-                                                        float* __restrict__ fout, const float* __restrict__ rin,
-                                                        const float* __restrict__ mu, unsigned long long* bad,
+__global__ void __launch_bounds__(NODE2_T) k_node2_coll(const KParams p, const unsigned mx, const float* fin,
+                                                        float* __restrict__ fout, const float* rin,
+                                                        const float* mu, unsigned long long* bad,
                                                         const long long t, const Mrt mrt) {
   pdl_wait();
   using L = Lattice<0>;
@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(NODE2_T) k_node2_coll(const KParams p, const u
   }
 }
 
-__global__ void __launch_bounds__(NODE2_T) k_node2_rho(const KParams p, const float* __restrict__ f,
+__global__ void __launch_bounds__(NODE2_T) k_node2_rho(const KParams p, const float* f,
                                                        float* __restrict__ rho, unsigned long long* bad, const long long t1) {
   pdl_wait();
   const int n = blockIdx.x * NODE2_T + threadIdx.x, N = int(p.n);

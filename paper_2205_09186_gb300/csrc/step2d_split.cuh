@@ -324,7 +324,7 @@ __device__ __forceinline__ void mu2d_rows(const KParams& p, const float* rin, fl
 constexpr int YMT = 256;
 
 template <int S>
-__global__ void __launch_bounds__(YMT) k_mu2d_ym(const KParams p, const float* __restrict__ rin,
+__global__ void __launch_bounds__(YMT) k_mu2d_ym(const KParams p, const float* rin,
                                                  float* __restrict__ mu, const int rpt) {
   static_assert(!Sch<S>::ISO && Sch<S>::R <= 4, "line schemes, stencil within one chunk on each side");
   pdl_wait();
@@ -339,7 +339,7 @@ __global__ void __launch_bounds__(YMT) k_mu2d_ym(const KParams p, const float* _
   const bool own = x < nx;
   const bool need_lo = tx == 0, need_hi = tx == 15 || x + 4 >= nx;
   auto ld = [&](int xx, int yy) {
-    return __ldg(reinterpret_cast<const float4*>(rin + wrapn(yy, ny) * nx + wrapn(xx, nx)));
+    return *reinterpret_cast<const float4*>(rin + wrapn(yy, ny) * nx + wrapn(xx, nx));
   };
   const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
   float4 q[2 * R + 1];
@@ -412,7 +412,7 @@ __device__ __forceinline__ void coll2d_tile(const KParams& p, const float* __res
 }
 
 template <int S, int RPT>
-__global__ void __launch_bounds__(NT2S) k_mu2d(const KParams p, const float* __restrict__ rin, float* __restrict__ mu) {
+__global__ void __launch_bounds__(NT2S) k_mu2d(const KParams p, const float* rin, float* __restrict__ mu) {
   [[maybe_unused]] constexpr int M2Y = Tile2<RPT>::M2Y, C2Y = Tile2<RPT>::C2Y, T2Y = Tile2<RPT>::T2Y, C2N = Tile2<RPT>::C2N;
   extern __shared__ __align__(16) unsigned char smem[];
   pdl_wait();
@@ -420,9 +420,9 @@ __global__ void __launch_bounds__(NT2S) k_mu2d(const KParams p, const float* __r
 }
 
 template <int S, bool TAU1, int RPT>
-__global__ void __launch_bounds__(NT2S) k_coll2d(const KParams p, const float* __restrict__ fin,
-                                                 float* __restrict__ fout, const float* __restrict__ rin,
-                                                 const float* __restrict__ mu, float* __restrict__ rout,
+__global__ void __launch_bounds__(NT2S) k_coll2d(const KParams p, const float* fin,
+                                                 float* __restrict__ fout, const float* rin,
+                                                 const float* mu, float* __restrict__ rout,
                                                  const StepAux aux, const Mrt mrt) {
   [[maybe_unused]] constexpr int M2Y = Tile2<RPT>::M2Y, C2Y = Tile2<RPT>::C2Y, T2Y = Tile2<RPT>::T2Y, C2N = Tile2<RPT>::C2N;
   extern __shared__ __align__(16) unsigned char smem[];

@@ -40,7 +40,7 @@ struct Node3 {
 
 template <int S, bool M64>
 __global__ void __launch_bounds__(NODE_T) k_node_mu(const KParams p, const unsigned mx, const unsigned my,
-                                                    const float* __restrict__ rin, float* __restrict__ mu) {
+                                                    const float* rin, float* __restrict__ mu) {
   pdl_wait();
   constexpr int R = Sch<S>::R;
   const int n = blockIdx.x * NODE_T + threadIdx.x;
@@ -59,8 +59,8 @@ __global__ void __launch_bounds__(NODE_T) k_node_mu(const KParams p, const unsig
 // block into partials, and snap overwritten with that state's density deviation
 template <int S, bool TAU1, bool OBS>
 __global__ void __launch_bounds__(NODE_T) k_node_coll(const KParams p, const unsigned mx, const unsigned my,
-                                                      const float* __restrict__ fin, float* __restrict__ fout,
-                                                      const float* __restrict__ rin, const float* __restrict__ mu,
+                                                      const float* fin, float* __restrict__ fout,
+                                                      const float* rin, const float* mu,
                                                       unsigned long long* bad, const long long t,
                                                       float* __restrict__ snap, double* __restrict__ partials) {
   pdl_wait();
@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(NODE_T) k_node_coll(const KParams p, const uns
   }
 }
 
-__global__ void __launch_bounds__(NODE_T) k_node_rho(const KParams p, const float* __restrict__ f, float* __restrict__ rho,
+__global__ void __launch_bounds__(NODE_T) k_node_rho(const KParams p, const float* f, float* __restrict__ rho,
                                                      unsigned long long* bad, const long long t1) {
   pdl_wait();
   const int n = blockIdx.x * NODE_T + threadIdx.x, N = int(p.n);

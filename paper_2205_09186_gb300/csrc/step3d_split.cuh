@@ -164,12 +164,12 @@ __device__ __forceinline__ bool mbar_wait_bounded(unsigned bar, unsigned parity)
 // integers (v * qscale rounded), into the corner accumulators qc
 // (k_coll3d_corners indexing); rout is not touched at corner nodes.
 template <int S, bool TAU1, bool VEC, bool OBS, int RY_ = CY, int NB_ = 2, int FD_ = COLL_FD>
-__global__ void __launch_bounds__(CX* RY_, (CollShape<S, RY_, NB_, FD_>::MINB)) k_coll3d(const KParams p, const float* __restrict__ fin,
-                                                    float* __restrict__ fout, const float* __restrict__ rin,
-                                                    const float* __restrict__ muf, float* __restrict__ rout,
+__global__ void __launch_bounds__(CX* RY_, (CollShape<S, RY_, NB_, FD_>::MINB)) k_coll3d(const KParams p, const float* fin,
+                                                    float* __restrict__ fout, const float* rin,
+                                                    const float* muf, float* __restrict__ rout,
                                                     const StepAux aux, const int zc, float* __restrict__ snap,
                                                     const __grid_constant__ CUtensorMap tmf,
-                                                    const float* __restrict__ gmu, const float* __restrict__ grho,
+                                                    const float* gmu, const float* grho,
                                                     unsigned long long* __restrict__ qc, const float qscale) {
   pdl_wait();
   using L = Lattice<1>;

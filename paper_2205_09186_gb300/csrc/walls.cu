@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(1024) k_wall_fill(Geo g, const signed char* __
 
 template <int LAT, int S, class P>
 __global__ void __launch_bounds__(WT) k_wall_mu(Geo g, KParams p, const signed char* __restrict__ layer,
-                                                const typename P::Tr* __restrict__ rho, double mu_w,
+                                                const typename P::Tr* rho, double mu_w,
                                                 typename P::Tm* mu) {
   pdl_wait();
   using Tm = typename P::Tm;
@@ -134,10 +134,10 @@ __global__ void __launch_bounds__(WT) k_wall_mu(Geo g, KParams p, const signed c
 // mode 0: collide and stream; mode 1: F (D x N) and mu (N) as FP64 fields
 template <int LAT, int S, class P>
 __global__ void __launch_bounds__(WT) k_wall_coll(Geo g, KParams p, Mrt mrt, const signed char* __restrict__ layer,
-                                                  const typename P::Tf* __restrict__ fin,
+                                                  const typename P::Tf* fin,
                                                   typename P::Tf* __restrict__ fout,
-                                                  const typename P::Tr* __restrict__ rho,
-                                                  const typename P::Tm* __restrict__ mu, unsigned long long* bad,
+                                                  const typename P::Tr* rho,
+                                                  const typename P::Tm* mu, unsigned long long* bad,
                                                   long long t, int mode, double* F, double* muo) {
   pdl_wait();
   using Lt = Lattice<LAT>;
@@ -218,7 +218,7 @@ __global__ void __launch_bounds__(WT) k_wall_coll(Geo g, KParams p, Mrt mrt, con
 
 template <int LAT, class P>
 __global__ void __launch_bounds__(WT) k_wall_dens(Geo g, KParams p, const signed char* __restrict__ layer,
-                                                  const typename P::Tf* __restrict__ f, typename P::Tr* rho,
+                                                  const typename P::Tf* f, typename P::Tr* rho,
                                                   unsigned long long* bad, long long t) {
   pdl_wait();
   constexpr int Q = LAT == 0 ? 9 : 19;

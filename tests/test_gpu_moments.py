@@ -292,3 +292,50 @@ def test_autotune_times_the_passes_it_cuts(L):
         s.lbm_init_droplet(25.0)
         ms = best_ms(lambda: s.lbm_step_observe(1))
         assert ms < 1.25 * min(fixed.values()), (zc, ms, fixed)
+
+
+# launches that overlap the end of the one before read what it wrote: the same bits as
+# from steps that are waited for one by one (and, on the moments, from launches with
+# events between them)
+@pytest.mark.parametrize("lattice,shape,kw,steps", [
+    ("D3", (8, 9, 10), dict(scheme="EFDS6", precision=1, tau=0.8), 3000),
+    ("D3", (33, 20, 17), dict(scheme="EFDS2", precision=1, tau=0.8), 2000),
+    ("D2", (16, 12, 1), dict(scheme="EFDS6", precision=1, tau=0.8), 3000),
+    ("D2", (96, 70, 1), dict(scheme="E8", precision=1, collision=1), 2000),
+    ("D2", (300, 150, 1), dict(scheme="EFDS4", precision=1, tau=0.9), 1000),
+    ("D2", (64, 64, 1), dict(scheme="EFDS2", precision=0), 2000),
+    ("D2", (100, 130, 1), dict(scheme="EFDS4", precision=0, tau=0.9), 500),
+    ("D3", (12, 13, 14), dict(scheme="EFDS4", precision=0), 500),
+    ("D3", (24, 20, 16), dict(scheme="OCFDS4", precision=0), 300),
+    ("D2", (64, 48, 1), dict(scheme="EFDS4", precision=1, walls=True), 400),  # (the oracle diverges at 590)
+    ("D3", (16, 12, 1), dict(scheme="EFDS2", precision=1, walls=True), 500),
+    ("D3", (32, 24, 20), dict(scheme="EFDS6", precision=1, moments=True), 1000),
+    ("D3", (33, 20, 21), dict(scheme="OCFDS4", precision=1, moments=True), 500),
+    ("D2", (64, 60, 1), dict(scheme="EFDS6", precision=1, moments=True), 2000)])
+def test_overlapped_launches_agree_with_separate_ones(L, lattice, shape, kw, steps):
+    import torch
+    kw = dict(kw)
+    walls, moments = kw.pop("walls", False), kw.pop("moments", False)
+    nx, ny, nz = shape if lattice == "D2" or shape[2] > 1 else shape[:2] + (12,)
+    out = []
+    for overlapped in (True, False):
+        p = L.make_params(lattice=L.LBM_D3Q19 if lattice == "D3" else L.LBM_D2Q9, nx=nx, ny=ny, nz=nz, Tr=0.9, k=0.2,
+                          kappa=0.1, **kw)
+        s = L.Sim(p)
+        s.lbm_init_droplet(min(d for d in (nx, ny, nz) if d > 1) / 4.0)
+        if walls:
+            mask = np.zeros(s.shape, np.uint8)
+            mask[:3] = 1
+            s.lbm_set_solid(mask, L.lbm_bulk_mu(p, L.lbm_maxwell(p)[0]))
+        if overlapped:
+            s.lbm_step(steps)
+        elif moments:
+            s.lbm_step_timed(steps)
+        else:
+            for _ in range(steps):
+                s.lbm_step(1)
+                torch.cuda.synchronize()
+        rho = s.lbm_get_density()
+        assert np.all(np.isfinite(rho))
+        out.append(rho)
+    assert np.array_equal(out[0], out[1])
