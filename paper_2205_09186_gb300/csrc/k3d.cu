@@ -138,16 +138,31 @@ cudaError_t launch_mu(const Launch& c, bool zero_edges = false) {
 }
 
 // Whether a step runs on node-parallel passes (step3d_node.cuh) or on the mu and
-// collision passes. By nodes: rows of whole 16-byte chunks suit the collision pass's
-// tensor copies, so it takes over where one population array (76 bytes a node)
-// outgrows about two thirds of the L2; on other rows it issues four times as many
-// copies and is worth its halo only well beyond the L2. Measured, tau 0.8, us a step
-// on the two passes and here: 96^3 58 and 51, 104^3 83 and 70, 128^3 105 and 126;
-// 97^3 80 and 54, 129^3 143 and 131, 161^3 271 and 251, 193^3 412 and 425. With
-// observables, whose sums cost small blocks more: 125 x 70 x 43 63 and 39, 64^3 61
-// and 36, 96^3 79 and 87.
+// collision passes.  By nodes first: small lattices leave the tiled passes' CTAs too
+// few, large ones outgrow the L2 (76 bytes a node in one population array) from which
+// the node passes read back.  Between the two by how much of its tiles (32 columns x
+// 11 rows) the lattice fills: a node costs the node passes the same everywhere, the
+// tiled ones 1 / fill; less at tau = 1, more on rows that are not whole 16-byte chunks
+// (four times as many copies), so that there they win only well beyond the L2.
+// Measured, us a step on the tiled passes and here: tau 1, 96 x 99 x 120 EFDS2 (fill
+// 1) 53 and 65, 128 x 88 x 96 EFDS6 (1) 55 and 65, 96^3 EFDS6 (0.97) 49 and 52, 104^3
+// (0.77) 83 and 69; 101^3 EFDS6 (0.72) 82 and 63, 113^3 EFDS2 (0.82) 86 and 85, 125^3
+// (0.92) 100 and 116, 153^3 (0.95) 178 and 209, 133^3 EFDS6 (0.77) 156 and 146.
+// tau 0.8, 128 x 55 x 128 EFDS6 (1) 57 and 57, 96 x 99 x 120 (1) 66 and 71, 104^3 83
+// and 70, 128^3 105 and 126; 121^3 (0.95) 122 and 114, 125^3 123 and 127, 137^3 (0.82)
+// 187 and 164, 153^3 218 and 230, 161^3 (0.82) 285 and 266, 193^3 412 and 425.  With
+// observables, whose sums cost small blocks more: 125 x 70 x 43 63 and 39, 64^3 61 and
+// 36, 96^3 79 and 87.
+template <int R, bool TAU1>
 bool node_rule(const KParams& kp, bool vec, bool obs) {
-  return kp.n <= (obs ? 600000 : (vec ? 1200000 : 4200000));
+  if (obs) return kp.n <= 600000;
+  if (kp.n <= (vec ? (TAU1 ? 700000 : 950000) : 1000000)) return true;
+  if (kp.n > (vec ? 1200000 : 4200000)) return false;
+  const double fill = double(kp.nx) * kp.ny / (double(CX) * ColTiles(kp.nx).nt * CY * RowBands(kp.ny, CY).nb);
+  const bool large = kp.n > 1900000;
+  const double most = TAU1 ? (vec ? 0.85 : (large ? 0.695 + 0.045 * R : 0.77 + 0.06 * R))
+                           : (large ? 0.80 + 0.025 * R : 0.95);
+  return fill < most;
 }
 
 // the three node-parallel passes (step3d_node.cuh)
@@ -181,7 +196,7 @@ cudaError_t launch_split(const Launch& c, int* nblocks, bool obs) {
   if (!c.mu) return cudaErrorInvalidValue;
   // 16-byte copies need rows of whole chunks and aligned bases
   const bool vec = c.kp.nx % 4 == 0 && aligned16(c.fin) && aligned16(c.rin) && aligned16(c.mu) && c.tmap;
-  if (!c.tiled && node_rule(c.kp, vec, obs)) return launch_node<S, TAU1, M64>(c, nblocks, obs);
+  if (!c.tiled && node_rule<Sch<S>::R, TAU1>(c.kp, vec, obs)) return launch_node<S, TAU1, M64>(c, nblocks, obs);
   const int zc = c.zc > 0 ? c.zc : split_zchunk_heuristic(c.kp, Sch<S>::R, TYC, CollShape<S, CY, 2, COLL_FD>::MINB);
   const long long ctas = coll3d_ctas(c.kp, zc);
   if (nblocks) {

@@ -339,3 +339,19 @@ def test_overlapped_launches_agree_with_separate_ones(L, lattice, shape, kw, ste
         assert np.all(np.isfinite(rho))
         out.append(rho)
     assert np.array_equal(out[0], out[1])
+
+
+# sizes in the range of the node-parallel passes whose lattice fills its tiles: a step
+# is not to cost more a node than one of the same cross section just beyond the range,
+# which runs on the tiled passes (on the node-parallel ones it cost 15 to 20% more)
+@pytest.mark.parametrize("shape,beyond", [((96, 99, 120), 130), ((128, 88, 96), 110), ((153, 153, 153), 182)])
+@pytest.mark.parametrize("scheme", ["EFDS2", "EFDS4"])
+def test_d3q19_single_steps_across_the_node_range(L, shape, beyond, scheme):
+    kw = dict(lattice=L.LBM_D3Q19, nx=shape[0], ny=shape[1], Tr=0.9, k=0.3, kappa=0.1, scheme=scheme,
+              precision=L.LBM_FP32DEV)
+    ns = []
+    for nz in (shape[2], beyond):
+        s = L.Sim(L.make_params(nz=nz, **kw))
+        s.lbm_init_droplet(25.0)
+        ns.append(best_ms(lambda: s.lbm_step(1), calls=20) / nz)
+    assert ns[0] < 1.09 * ns[1], ns
