@@ -323,20 +323,31 @@ cudaError_t wall_run(const WallLaunch& w, int mode, int* nblocks) {
   const dim3 blk(WX, WY), grid = wall_grid(g, 1 << 20);
   cudaStream_t st = w.c.stream;
   Tr* rin = static_cast<Tr*>(const_cast<void*>(w.c.rin));  // wall layers are refreshed in place
-  // wall densities, in one launch while one CTA's rounds are fewer than the
-  // launches they replace are worth (512^2 with a flat wall: 1024 nodes a layer)
+  // Wall densities in one launch while one CTA's rounds are fewer than the launches
+  // they replace are worth: 1024 nodes a layer, in FP64, whose pipe one SM has little
+  // of, 128.  One launch and three, us a step: FP32 512^2 flat wall (1024 a layer)
+  // 22.7 and 24.1, 256^2 (512) 14.8 and 16.2; 32^3 (2048) 24.4 and 17.8, 1800 x 100
+  // (3600) 32.5 and 24.8; FP64 64^2 (128) 33.7 and 34.7, 128^2 (256) 45 and 38.5, 24^3
+  // (1152) 76 and 56.
   const int *nl = w.nlist, most = std::max({nl[0], nl[1], nl[2]});
+  // FP64 launches overlap except where the pass's CTAs find an SM each and are more
+  // than half as many: dealt early, two share an SM and its FP64 pipe (us a step
+  // overlapped and not: 28^3, 98 CTAs, 82 and 58, 32^3 98 and 60, 192^2, 144 CTAs, 63
+  // and 45; 144^2, 90 CTAs, 40 and 45, 24^3 57 and 69, 34^3 98 and 108)
+  const long long ctas = (long long)grid.x * grid.y;
+  const bool pdl = sizeof(Tr) != 8 || 10 * ctas <= 6 * device_sms() || ctas > device_sms();
   cudaError_t e = cudaSuccess;
-  if (most <= 4096) {
-    if (most > 0) e = launch_pdl(k_wall_fill<LAT, Tr>, dim3(1), 1024, 0, st, g, w.layer, w.list, nl[0], nl[1], nl[2], 0, rin);
+  if (most <= (sizeof(Tr) == 8 ? 128 : 1024)) {
+    if (most > 0)
+      e = launch_if_pdl(pdl, k_wall_fill<LAT, Tr>, dim3(1), 1024, 0, st, g, w.layer, w.list, nl[0], nl[1], nl[2], 0, rin);
   } else {
     for (int L = 1; L <= 3 && e == cudaSuccess; ++L)
       if (nl[L - 1] > 0)
-        e = launch_pdl(k_wall_fill<LAT, Tr>, dim3((nl[L - 1] + 255) / 256), 256, 0, st, g, w.layer, w.list, nl[0], nl[1],
-                       nl[2], L, rin);
+        e = launch_if_pdl(pdl, k_wall_fill<LAT, Tr>, dim3((nl[L - 1] + 255) / 256), 256, 0, st, g, w.layer, w.list, nl[0],
+                          nl[1], nl[2], L, rin);
   }
   if (e != cudaSuccess || mode == MODE_WALL_FILL) return e;
-  e = launch_pdl(k_wall_mu<LAT, S, P>, grid, blk, 0, st, g, w.c.kp, w.layer, rin, w.mu_w, static_cast<Tm*>(w.mu));
+  e = launch_if_pdl(pdl, k_wall_mu<LAT, S, P>, grid, blk, 0, st, g, w.c.kp, w.layer, rin, w.mu_w, static_cast<Tm*>(w.mu));
   if (e != cudaSuccess) return e;
   if (mode == MODE_OBS) {
     const dim3 og = wall_grid(g, 4096);
@@ -347,12 +358,12 @@ cudaError_t wall_run(const WallLaunch& w, int mode, int* nblocks) {
     return cudaGetLastError();
   }
   const int cm = mode == MODE_FIELDS ? 1 : 0;
-  e = launch_pdl(k_wall_coll<LAT, S, P>, grid, blk, 0, st, g, w.c.kp, w.c.mrt, w.layer, static_cast<const Tf*>(w.c.fin),
-                 static_cast<Tf*>(w.c.fout), rin, static_cast<const Tm*>(w.mu), w.c.aux.bad_step, w.c.aux.t, cm, w.c.fo.F,
-                 w.c.fo.mu);
+  e = launch_if_pdl(pdl, k_wall_coll<LAT, S, P>, grid, blk, 0, st, g, w.c.kp, w.c.mrt, w.layer, static_cast<const Tf*>(w.c.fin),
+                    static_cast<Tf*>(w.c.fout), rin, static_cast<const Tm*>(w.mu), w.c.aux.bad_step, w.c.aux.t, cm, w.c.fo.F,
+                    w.c.fo.mu);
   if (e == cudaSuccess && mode == MODE_STEP)
-    e = launch_pdl(k_wall_dens<LAT, P>, grid, blk, 0, st, g, w.c.kp, w.layer, static_cast<const Tf*>(w.c.fout),
-                   static_cast<Tr*>(w.c.rout), w.c.aux.bad_step, w.c.aux.t + 1);
+    e = launch_if_pdl(pdl, k_wall_dens<LAT, P>, grid, blk, 0, st, g, w.c.kp, w.layer, static_cast<const Tf*>(w.c.fout),
+                      static_cast<Tr*>(w.c.rout), w.c.aux.bad_step, w.c.aux.t + 1);
   return e;
 }
 

@@ -210,3 +210,42 @@ def test_wide_walls_d2q9(L, rows, precision, tol):
         (s.lbm_init_droplet if s is g else s.init_droplet)(6.0, center=[700.0, 7.0, 0.0])
         (s.lbm_set_solid if s is g else s.set_solid)(mask2, mu_sat())
     compare(g, o, mask2, tol, 8)
+
+
+# layers of 1000 to 1026 nodes (126 to 130 in FP64) either side of the line up to which
+# one CTA fills all three: a flat wall of either lattice has equal layers on both sides
+@pytest.mark.parametrize("lattice,shape", [(2, (16, 63)), (2, (16, 64)), (2, (16, 65)), (2, (16, 511)), (2, (16, 512)),
+                                           (2, (16, 513)), (3, (16, 8, 8)), (3, (16, 20, 25)), (3, (16, 16, 32)),
+                                           (3, (16, 19, 27))])
+@pytest.mark.parametrize("precision,tol", [(0, 1e-12), (1, 1e-5)])
+def test_wall_layers_across_the_one_launch_line(L, lattice, shape, precision, tol):
+    g, o = pair(L, lattice, shape, "EFDS4", precision)
+    for s in (g, o):
+        s.init_droplet(3.0) if s is o else s.lbm_init_droplet(3.0)
+    mask = flat_wall(shape, 7)
+    for s in (g, o):
+        s.set_solid(mask, mu_sat() - 0.01) if s is o else s.lbm_set_solid(mask, mu_sat() - 0.01)
+    compare(g, o, mask, tol, 6)
+
+
+def test_fp64_wall_steps_of_one_wave(L):
+    # 54 and 128 CTAs on 152 SMs: the larger lattice is one wave as well and takes
+    # little longer, but for one SM that fills all wall layers (2048 nodes each) and
+    # for CTAs of the next launch that share an SM (1.7 times as long)
+    import torch
+    ms = []
+    for n in (24, 32):
+        s = L.Sim(L.make_params(lattice=L.LBM_D3Q19, nx=n, ny=n, nz=n, Tr=0.9, k=0.2, kappa=0.1, scheme="EFDS6"))
+        s.lbm_init_droplet(n / 4.0)
+        s.lbm_set_solid(flat_wall((n, n, n), 4), mu_sat())
+        best = 1e30
+        for _ in range(5):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            s.lbm_step(4)
+            e0.record()
+            s.lbm_step(40)
+            e1.record()
+            torch.cuda.synchronize()
+            best = min(best, e0.elapsed_time(e1))
+        ms.append(best)
+    assert ms[1] < 1.4 * ms[0], ms
