@@ -7,6 +7,7 @@
 // Parameter layout (as in the C ABI): per layer W (out x in, row-major) then b.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <new>
@@ -713,6 +714,7 @@ struct lbm_mlp {
   float *x = nullptr, *t = nullptr, *y = nullptr, *zs = nullptr, *hs = nullptr, *loss = nullptr;
   size_t act_floats = 0;
   float* train = nullptr;  // scratch of k_mlp_train (null: training on the separate passes)
+  int train_max = 0;       // samples up to which training runs in one launch
   int ndata = 0;
   int adam_t = 0;
   std::vector<std::pair<void*, size_t>> blocks;
@@ -723,6 +725,25 @@ static size_t train_smem(const Net& net) { return size_t(3 * train_rows(net) + (
 static size_t train_floats(const Net& net, int Bp) { return size_t(3 * net.nl + 2 + 2 * TC) * MAXW * Bp + TC; }
 
 static void free_cb(void* p, size_t, void*) { cudaFree(p); }
+
+// Samples up to which training runs in one launch (a multiple of 32).  Eight CTAs take
+// blocks of 32 samples in turn, the separate passes a CTA per block: theirs is a fixed
+// time up to thousands of samples, long where layers are wide.  Both as fitted, us an
+// iteration: 12 + per layer 4.5 + 130 in out / 128^2 (60 for the first, which hands
+// nothing back) against, per block, 2.4 a layer + 3.1 in out / 128^2 (4.6).  Measured,
+// separate and one launch: 4-128-128-128-64 with 512 samples 398 and 270, 640 399 and
+// 335, 1024 402 and 532; 128-128 320 77 and 71, 384 77 and 86; 4-64-64-64 256 94 and
+// 78, 384 94 and 113; 4-16-16-2 96 32 and 28, 128 32 and 35; 1-1 160 17 and 10, 384 17
+// and 21.
+static int train_limit(const Net& net) {
+  double passes = 12.0, block = 0.0;
+  for (int l = 0; l < net.nl; ++l) {
+    const double p = double(net.sizes[l]) * net.sizes[l + 1] / (128.0 * 128.0);
+    passes += 4.5 + (l == 0 ? 60.0 : 130.0) * p;
+    block += 2.4 + (l == 0 ? 4.6 : 3.1) * p;
+  }
+  return 32 * int(std::max(1.0, passes / block));
+}
 
 static float* mget(lbm_mlp* m, size_t floats) {
   const size_t b = floats * 4 + 256;
@@ -781,7 +802,8 @@ extern "C" int lbm_mlp_create(const int* sizes, int nlayers, int max_batch, void
     lbm_mlp_destroy(m);
     return LBM_ENOMEM;
   }
-  if (train_smem(m->net) <= size_t(227) * 1024) m->train = mget(m, train_floats(m->net, (max_batch + 31) / 32 * 32));
+  m->train_max = std::min(train_limit(m->net), (max_batch + 31) / 32 * 32);
+  if (train_smem(m->net) <= size_t(227) * 1024) m->train = mget(m, train_floats(m->net, m->train_max));
   cudaMemsetAsync(m->m, 0, size_t(off) * 4, m->stream);
   cudaMemsetAsync(m->v, 0, size_t(off) * 4, m->stream);
   if (cudaStreamSynchronize(m->stream) != cudaSuccess) { lbm_mlp_destroy(m); return LBM_ECUDA; }
@@ -909,7 +931,7 @@ extern "C" int lbm_mlp_train(lbm_mlp* m, int iters, float lr, float* host_loss) 
   // a launch per 2000 iterations (some tens of milliseconds): other work on
   // the GPU's queue is not kept waiting by a long training call
   int done = 0;
-  while (m->train && done < iters) {
+  while (m->train && m->ndata <= m->train_max && done < iters) {
     const int n = iters - done < 2000 ? iters - done : 2000;
     if (!launch_train(m, n, lr)) break;
     done += n;

@@ -99,3 +99,52 @@ def test_cluster_training_follows_oracle(L, sizes, batch):
     assert loss == pytest.approx(lo, rel=1e-4)
     d = np.abs(pg - po)
     assert np.quantile(d, 0.99) < 1e-4 and np.median(d) < 1e-6
+
+
+# training runs in one launch of eight CTAs up to a number of samples that depends on
+# the layers' widths, on the separate passes beyond it: samples either side of the line
+# (96 and 128 for the narrow network, 320 and 352 for the single layer)
+@pytest.mark.parametrize("sizes,batch", [([4, 16, 16, 2], 96), ([4, 16, 16, 2], 97), ([128, 128], 320), ([128, 128], 321),
+                                         ([1, 1], 192), ([1, 1], 193)])
+def test_training_across_the_one_launch_line(L, sizes, batch):
+    # (tolerances as in test_cluster_training_follows_oracle)
+    p0 = init_params(sizes, 6).astype(np.float32).astype(np.float64)
+    rng = np.random.default_rng(batch)
+    x = rng.uniform(-1, 1, (batch, sizes[0])).astype(np.float32).astype(np.float64)
+    t = np.tanh(x @ rng.standard_normal((sizes[0], sizes[-1]))).astype(np.float32).astype(np.float64)
+    m = L.MLP(sizes, batch)
+    m.lbm_mlp_set_params(p0)
+    m.lbm_mlp_set_data(x, t)
+    m.lbm_mlp_train(5, lr=1e-3)
+    loss = m.lbm_mlp_train(7, lr=1e-3)
+    pg = m.lbm_mlp_get_params()
+    po, mo, vo = p0.copy(), np.zeros_like(p0), np.zeros_like(p0)
+    for it in range(1, 13):
+        lo, g = O.mlp_loss_grad(sizes, po, x, t)
+        O.adam_step(po, mo, vo, g, 1e-3, it)
+    assert loss == pytest.approx(lo, rel=1e-4)
+    d = np.abs(pg - po)
+    assert np.quantile(d, 0.99) < 1e-4 and np.median(d) < 1e-6
+
+
+def test_training_time_does_not_grow_with_the_samples(L):
+    # 4096 samples are 128 CTAs of the separate passes, which take as long as a few; a
+    # cluster of eight CTAs takes 30 times as long as for 128
+    import torch
+    ms = []
+    for batch in (64, 4096):
+        sizes = [4, 16, 16, 2]
+        m = L.MLP(sizes, batch)
+        rng = np.random.default_rng(3)
+        m.lbm_mlp_set_params(init_params(sizes, 7))
+        m.lbm_mlp_set_data(rng.uniform(-1, 1, (batch, 4)), rng.uniform(-1, 1, (batch, 2)))
+        best = 1e30
+        for _ in range(5):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            m.lbm_mlp_train(50, 1e-4)
+            e1.record()
+            torch.cuda.synchronize()
+            best = min(best, e0.elapsed_time(e1))
+        ms.append(best)
+    assert ms[1] < 5 * ms[0], ms
