@@ -210,9 +210,12 @@ int lbm_set_solid(lbm_handle* h, const unsigned char* mask, double mu_w);
  * where several thread blocks contribute to one node's next density, their
  * partial sums are combined in an order-independent way (two floating-point
  * additions onto zero, or exact 64-bit fixed-point additions).  Calls of n >= 2
- * steps with tau = 1 may carry only the moments from step to step and form the
- * populations of the last one (FP32DEV explicit schemes): n single steps then
- * agree with them within FP32 rounding. */
+ * steps (n >= 3 or 4 on some D3Q19 lattices) with tau = 1 and LBM_BGK, FP32DEV and
+ * no walls carry only the moments from step to step and form the populations of
+ * the last one: D2Q9 EFDS2/4/6, E4 and E8 with FP32 mu, D3Q19 EFDS2/4/6 with either
+ * mu and D3Q19 compact schemes with FP32 mu and lines of at most 512 nodes (all but
+ * the narrowest lattices; batches as well, two steps at a time).  n single steps
+ * agree with such a call within FP32 rounding, not in every bit. */
 int lbm_step(lbm_handle* h, long long n);
 
 /* As lbm_step (n <= 100000), timing every step on the handle's stream with

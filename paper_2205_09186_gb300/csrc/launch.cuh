@@ -52,11 +52,12 @@ int fast_zchunk_heuristic(const KParams& kp, int R);
 // field dump (MODE_FIELDS); returns the number of CTAs through *nblocks
 using StepFn = cudaError_t (*)(const Launch&, int mode, int* nblocks);
 
-// n >= 2 steps of the D3Q19 FP32DEV line schemes, explicit or compact, at tau = 1 on the
+// Several steps of the D3Q19 FP32DEV line schemes, explicit or compact, at tau = 1 on the
 // moments rho, j (mom3d.cuh): from the populations and density fin, rin back
 // into the same buffers; fout is scratch.  mom3d_ok: whether the case and the
-// scratch (19 N floats) allow it.
+// scratch (19 N floats) allow it; mom3d_least: the steps of a call from which it pays.
 bool mom3d_ok(const KParams& kp, int scheme, int prec);
+int mom3d_least(const KParams& kp, int scheme);
 cudaError_t mom3d_steps(const Launch& c, int scheme, int prec, long long n);
 
 // the same for D2Q9 FP32DEV, explicit and isotropic schemes (mom2d.cuh)

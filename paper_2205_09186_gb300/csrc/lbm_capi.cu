@@ -935,11 +935,12 @@ extern "C" int lbm_autotune(lbm_handle* h, int* zc_out) {
 
 // calls of two or more steps that run on the moments: the state between the
 // steps of one call is never seen, and at tau = 1 the populations are not
-// needed to advance it.  A call costs gather + expand once (0.63 ms at 256^3)
-// and 0.31 ms a step against 0.608 on the populations: break-even at two.
+// needed to advance it.  A call costs gather and expansion once (0.63 ms at 256^3)
+// and 0.31 ms a step against 0.61 on the populations; D2Q9 forms the populations in
+// its last step and pays from two on.
 static bool on_moments(const lbm_handle* h, long long n) {
   if (n < 2 || (!h->mu && !h->compact) || h->layer || (h->compact && h->D == 2)) return false;
-  return h->D == 3 ? mom3d_ok(h->kp, h->p.scheme, h->prec) : mom2d_ok(h->kp, h->p.scheme, h->prec, h->mrt.on != 0);
+  return h->D == 3 ? mom3d_ok(h->kp, h->p.scheme, h->prec) && n >= mom3d_least(h->kp, h->p.scheme) : mom2d_ok(h->kp, h->p.scheme, h->prec, h->mrt.on != 0);
 }
 static cudaError_t moment_steps(lbm_handle* h, const Launch& c, long long n) {
   return h->D == 3 ? mom3d_steps(c, h->p.scheme, h->prec, n) : mom2d_steps(c, h->p.scheme, n);

@@ -128,6 +128,24 @@ bool mom3d_ok(const KParams& kp, int scheme, int prec) {
   return (compact ? 12 : 9) * P <= 19 * kp.n && 19 * kp.n < (1LL << 31);
 }
 
+// A call's gather and expansion cost as much as two of its steps on the moments, so
+// two steps pay only where a step on the populations is dear.  Not where rows are
+// whole 16-byte chunks beyond the node-parallel passes' sizes and the stencil is wide
+// or the populations are partly in the L2, nor where the compact schemes' lines are
+// solved in registers (multiples of 32; CFDS8's mu pass is dearer).  Measured, us a
+// step of single steps, two and three a call: 160^3 EFDS2 143, 158, 134, EFDS6 159,
+// 187, 159; 256^3 EFDS2 566, 524, 430, EFDS4 580, 564, 466, EFDS6 610, 619, 516; 192^3
+// EFDS6 281, 270, 224, 224^3 417, 440, 367; 129^3 EFDS6 134, 111.  CFDS4 128 x 128 x 64
+// 84, 68; 128^3 115, 128, 114; 160^3 202, 236, 210; 224^3 550, 589, 522; 256^3 847, 795;
+// CFDS8 160^3 283, 245.
+int mom3d_least(const KParams& kp, int scheme) {
+  if (scheme == S_EFDS2 || scheme == S_EFDS4 || scheme == S_EFDS6)
+    return kp.nx % 4 == 0 && kp.n > 1200000 && (scheme == S_EFDS6 || kp.n < 6000000) ? 3 : 2;
+  const bool regs = kp.nx % 32 == 0 && kp.ny % 32 == 0 && kp.nz % 32 == 0;
+  if (!regs || scheme == S_CFDS8 || kp.n < 1500000 || kp.n > 14000000) return 2;
+  return scheme == S_CFDS4 && kp.n > 3000000 && kp.n < 6000000 ? 4 : 3;
+}
+
 cudaError_t mom3d_steps(const Launch& c, int scheme, int prec, long long n) {
   switch (scheme) {
     case S_EFDS2:
