@@ -41,9 +41,17 @@ cudaError_t launch_split2d_t(const Launch& c, int* nblocks) {
   // launch's blocks are dealt while those before still run, two then share an SM
   // (E8 at tau 0.9, us a step overlapped and not: 300^2 14.9 and 12.3, 420^2 12.5 and
   // 16.4, 600^2 19.0 and 20.6; EFDS6 at tau 0.8: 300^2 8.6 to 11.7 and 12.3, 512^2
-  // 14.1 and 17.8, 1024^2 32.8 and 36.2)
+  // 14.1 and 17.8, 1024^2 32.8 and 36.2).  Nor where the SMs hold more than one and a
+  // half to two tiles each and the second of them waits for longer than a launch: the
+  // widest stencil behind its vector mu pass, and it and the isotropic ones on
+  // lattices of two tile rows (EFDS6 at tau 1: 3600 x 40 14.8 and 12.4, 900 x 240 14.8
+  // and 14.4; 900 x 210 12.1 and 14.4, 700 x 390 13.1 and 16.4; E8 4000 x 40 15.3 and
+  // 14.4; EFDS4 12.2 and 12.3)
   const dim3 gc((c.kp.nx + T2X - 1) / T2X, (c.kp.ny + T2Y - 1) / T2Y);
-  const bool pdl = !Sch<S>::ISO || (long long)gc.x * gc.y > device_sms();
+  const long long tiles = (long long)gc.x * gc.y, sms = device_sms();
+  const bool wide = Sch<S>::R == 3, two = 2 * tiles > 3 * sms && tiles <= 2 * sms;
+  const bool late = two && ((wide && c.kp.nx % 4 == 0 && !c.mrt.on) || (gc.y <= 2 && (wide || Sch<S>::ISO)));
+  const bool pdl = !late && (!Sch<S>::ISO || tiles > sms);
   cudaError_t e = cudaSuccess;
   if constexpr (!Sch<S>::ISO) {
     if (c.kp.nx % 4 == 0 && (reinterpret_cast<uintptr_t>(c.rin) & 15) == 0 && (reinterpret_cast<uintptr_t>(c.mu) & 15) == 0) {
