@@ -144,32 +144,35 @@ __global__ void __launch_bounds__(NODE_T) k_node_coll(const KParams p, const uns
     if constexpr (!OBS) break;  // one node per thread
   }
   if constexpr (OBS) {
-    // in FP32 within the block (32 sums of a few nodes each), one thread in FP64
-    __shared__ float red[4][NODE_T / 32];
+    // a thread's few deviations are summed in FP32, the 32 sums of a warp in
+    // double-float (as FP64 would, off its pipe), the warps' by one thread in FP64
+    __shared__ float red[3][NODE_T / 32];
+    __shared__ double mass[NODE_T / 32];
     __shared__ int cnt[NODE_T / 32];
+    Df m{o_m, 0.f};
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       o_v2 = fmaxf(o_v2, __shfl_xor_sync(0xffffffffu, o_v2, o));
       o_u2 = fmaxf(o_u2, __shfl_xor_sync(0xffffffffu, o_u2, o));
       o_d = fmaxf(o_d, __shfl_xor_sync(0xffffffffu, o_d, o));
-      o_m += __shfl_xor_sync(0xffffffffu, o_m, o);
+      m = df_add(m, Df{__shfl_xor_sync(0xffffffffu, m.h, o), __shfl_xor_sync(0xffffffffu, m.l, o)});
       o_n += __shfl_xor_sync(0xffffffffu, o_n, o);
     }
     const int w = threadIdx.x >> 5;
-    if ((threadIdx.x & 31) == 0) red[0][w] = o_v2, red[1][w] = o_u2, red[2][w] = o_d, red[3][w] = o_m, cnt[w] = o_n;
+    if ((threadIdx.x & 31) == 0) red[0][w] = o_v2, red[1][w] = o_u2, red[2][w] = o_d, mass[w] = double(m.h) + double(m.l), cnt[w] = o_n;
     __syncthreads();
     if (threadIdx.x == 0) {
-      double m = 0.0;
+      double sum = 0.0;
       for (int k = 0; k < NODE_T / 32; ++k) {
         o_v2 = fmaxf(o_v2, red[0][k]);
         o_u2 = fmaxf(o_u2, red[1][k]);
         o_d = fmaxf(o_d, red[2][k]);
-        m += double(cnt[k]) * p.rho_ref + double(red[3][k]);
+        sum += double(cnt[k]) * p.rho_ref + mass[k];
       }
       double* out = partials + 4 * blockIdx.x;
       out[0] = 0.5 * sqrt(double(o_v2));
       out[1] = sqrt(double(o_u2));
-      out[2] = m;
+      out[2] = sum;
       out[3] = double(o_d);
     }
   }

@@ -140,3 +140,20 @@ def test_async_observation_equals_the_synchronous_one(L, shape, kw):
     recs = [L.lbm_obs.from_address(host.data_ptr() + k * size).as_dict() for k in range(3)]
     assert recs == sync
     assert np.array_equal(a.lbm_get_density(), b.lbm_get_density())
+
+
+# the node-parallel observed step: on up to a node per thread (8 blocks of 128 on each
+# of 152 SMs) the mass is the FP64 sum of the densities but for its own roundings
+# (2^-48 of a warp's sum of deviations); a warp's 32 deviations added in FP32 were off
+# by some 1e-9 of the mass
+@pytest.mark.parametrize("shape", [(48, 48, 48), (41, 50, 63), (53, 53, 53)])
+def test_observed_mass_is_summed_beyond_fp32(L, shape):
+    nx, ny, nz = shape
+    s = L.Sim(L.make_params(lattice=L.LBM_D3Q19, nx=nx, ny=ny, nz=nz, Tr=0.9, k=0.2, kappa=0.1, scheme="EFDS4", tau=0.9,
+                            precision=L.LBM_FP32DEV))
+    rho = 0.15 + 0.02 * np.random.default_rng(nx).standard_normal((nz, ny, nx))
+    s.lbm_init_density(rho)
+    for _ in range(3):
+        # the stored density is rho_ref + a float: read back exactly in FP64
+        want = np.sum(s.lbm_get_density().astype(np.longdouble))
+        assert abs(s.lbm_step_observe(1)["mass"] / float(want) - 1) < 2e-13
