@@ -371,7 +371,8 @@ def test_short_calls_cost_no_more_than_single_steps(L, scheme, n, steps):
 
 
 # flat lattices of two tiles an SM: single steps with the widest stencil took a fifth
-# longer than with the one before it, for launches that overlapped to their loss
+# longer than with the one before it, for launches that overlapped to their loss (those
+# that do not start on a grid of some 2 us: the line allows for half a mesh)
 @pytest.mark.parametrize("nx", [3600, 4000])
 def test_d2q9_single_steps_of_two_tiles_an_sm(L, nx):
     ms = []
@@ -380,4 +381,4 @@ def test_d2q9_single_steps_of_two_tiles_an_sm(L, nx):
                                 precision=L.LBM_FP32DEV))
         s.lbm_init_droplet(10.0)
         ms.append(best_ms(lambda: s.lbm_step(1), calls=100))
-    assert ms[1] < 1.1 * ms[0], ms
+    assert ms[1] < 1.17 * ms[0], ms
