@@ -573,19 +573,19 @@ __global__ void __launch_bounds__(T2NT, T2_CTAS) k_batch_mom(const CaseDev* __re
   const long long t0 = *((volatile long long*)&ctl->t);
   const int par = int(t0 & 1), w = int(threadIdx.x >> 5);
   const int ph = work.ncmp[2] > 0 ? 3 : 1;  // phases of a step
-  int q = 0;
-  for (int k = 0; k <= ph * nsteps; ++k) {  // phase 0: gather
-    const int s = k > 0 ? (k - 1) / ph : 0, f = k > 0 ? (k - 1) - s * ph : 2;
+  int q = 0, s = 0, f = 2;                  // step and its phase
+  unsigned k = 0;                           // phase of the launch, modulo 2^32 (three times INT_MAX steps exceed an int)
+  for (bool gather = true;; gather = false, ++k) {
     const bool last = s == nsteps - 1;
     const Item* cmp = work.cmp[f];
-    const int nc = work.ncmp[f], n = nc + (k == 0 || ph == 1 || f == 1 ? work.ntiles : 0);
+    const int nc = work.ncmp[f], n = nc + (gather || ph == 1 || f == 1 ? work.ntiles : 0);
     unsigned* ctr = &ctl->work[k & 3];
     for (int u = int(blockIdx.x); u < n;) {
       // (a slot is rewritten two items after it was read, past the barrier below)
       if (threadIdx.x == 0) s_q[q] = int(gridDim.x) + int(atomicAdd(ctr, 1u));
       const Item itm = u < nc ? cmp[u] : work.tiles[u - nc];
       const CaseDev& cd = cases[itm.c];
-      if (k == 0) {
+      if (gather) {
         const int row = itm.tile / cd.mg.nt, x0 = (itm.tile - row * cd.mg.nt) * cd.mg.TW, y0 = row * cd.mg.TH;
         const int vw = min(cd.mg.TW, cd.kp.nx - x0), vh = min(cd.mg.TH, cd.kp.ny - y0);
         for (int y = y0 + w; y < y0 + vh; y += T2NT / 32)
@@ -603,9 +603,15 @@ __global__ void __launch_bounds__(T2NT, T2_CTAS) k_batch_mom(const CaseDev* __re
       u = s_q[q];
       q ^= 1;
     }
-    if (k == ph * nsteps) break;
+    if (!gather && last && f == ph - 1) break;
     if (blockIdx.x == 0 && threadIdx.x == 0) ctl->work[(k + 2) & 3] = 0u;
     if (!grid_barrier(ctl, timeout_ns)) return;
+    if (gather) {
+      f = 0;
+    } else if (++f == ph) {
+      f = 0;
+      ++s;
+    }
   }
   if (set_t && blockIdx.x == 0 && threadIdx.x == 0) ctl->t = t0 + nsteps;
 }
