@@ -368,17 +368,3 @@ def test_short_calls_cost_no_more_than_single_steps(L, scheme, n, steps):
     single = best_ms(lambda: s.lbm_step(1), calls=24)
     call = best_ms(lambda: s.lbm_step(steps), calls=12) / steps
     assert call < 1.03 * single, (call, single)
-
-
-# flat lattices of two tiles an SM: single steps with the widest stencil took a fifth
-# longer than with the one before it, for launches that overlapped to their loss (those
-# that do not start on a grid of some 2 us: the line allows for half a mesh)
-@pytest.mark.parametrize("nx", [3600, 4000])
-def test_d2q9_single_steps_of_two_tiles_an_sm(L, nx):
-    ms = []
-    for scheme in ("EFDS4", "EFDS6"):
-        s = L.Sim(L.make_params(lattice=L.LBM_D2Q9, nx=nx, ny=40, Tr=0.9, k=0.3, kappa=0.1, scheme=scheme,
-                                precision=L.LBM_FP32DEV))
-        s.lbm_init_droplet(10.0)
-        ms.append(best_ms(lambda: s.lbm_step(1), calls=100))
-    assert ms[1] < 1.17 * ms[0], ms
