@@ -68,8 +68,10 @@ Mom2Geo mom2_geo(const KParams& kp, int sms) {
   g.TW = ((kp.nx + nt - 1) / nt + 3) / 4 * 4;
   g.nt = (kp.nx + g.TW - 1) / g.TW;
   double best = 1e300;
-  for (int nr = (kp.ny + T2H - 1) / T2H; nr <= kp.ny; ++nr) {
-    const int th = (kp.ny + nr - 1) / nr, rows = (kp.ny + th - 1) / th;
+  // (each height once, the tallest first: a call of two steps on a long lattice is not
+  // to wait for the search)
+  for (int most = std::min(T2H, kp.ny); most > 0; --most) {
+    const int nr = (kp.ny + most - 1) / most, th = (kp.ny + nr - 1) / nr, rows = (kp.ny + th - 1) / th;
     if (th < 8 && best < 1e300) break;
     const long long tiles = (long long)g.nt * rows;
     const long long k = (tiles + sms - 1) / sms;

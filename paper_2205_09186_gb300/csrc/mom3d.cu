@@ -35,16 +35,17 @@ MomGeo mom_geo(const KParams& kp) {
 void mom_cut(const KParams& kp, MomGeo* g, int* zc) {
   const long long slots = device_sms();
   double best = 1e300;
-  for (int nb = (kp.ny + MW3 - 4) / (MW3 - 3); nb <= kp.ny; ++nb) {
-    const int rb = (kp.ny + nb - 1) / nb, bands = (kp.ny + rb - 1) / rb;
+  // (each height of a band and each chunk once, the largest first)
+  for (int most = std::min(MW3 - 3, kp.ny); most > 0; --most) {
+    const int nb = (kp.ny + most - 1) / most, rb = (kp.ny + nb - 1) / nb, bands = (kp.ny + rb - 1) / rb;
     if (2 * rb < MW3 - 3 && best < 1e300) break;
-    for (int n = 1; n <= kp.nz; ++n) {
-      const int c = (kp.nz + n - 1) / n;
+    for (int n = 1, c; n <= kp.nz; n = (kp.nz + c - 2) / (c - 1)) {
+      c = (kp.nz + n - 1) / n;
       if (c < 2 && n > 1) break;
       const long long ctas = (long long)g->nt * bands * ((kp.nz + c - 1) / c);
       const double cost = double((ctas + slots - 1) / slots) * (c + 4) * (rb + 7);
       if (cost < best - 1e-9) { best = cost; *zc = c; g->RB = rb; g->nb = bands; }
-      if (ctas > 8 * slots) break;
+      if (ctas > 8 * slots || c < 2) break;
     }
   }
 }

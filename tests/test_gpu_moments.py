@@ -368,3 +368,25 @@ def test_short_calls_cost_no_more_than_single_steps(L, scheme, n, steps):
     single = best_ms(lambda: s.lbm_step(1), calls=24)
     call = best_ms(lambda: s.lbm_step(steps), calls=12) / steps
     assert call < 1.03 * single, (call, single)
+
+
+# the cut of a lattice is searched in every call: on long lattices that took tens of
+# thousands of trips, half a millisecond of the caller's time
+@pytest.mark.parametrize("lattice,shape", [("D2", (40, 500000, 1)), ("D3", (16, 400000, 16))])
+def test_calls_on_long_lattices_return_at_once(L, lattice, shape):
+    import time
+    import torch
+    us = []
+    for s3 in ((40, 64, 1) if lattice == "D2" else (16, 64, 16), shape):
+        s = L.Sim(L.make_params(lattice=L.LBM_D3Q19 if lattice == "D3" else L.LBM_D2Q9, nx=s3[0], ny=s3[1], nz=s3[2],
+                                Tr=0.9, k=0.3, kappa=0.1, scheme="EFDS2", precision=L.LBM_FP32DEV))
+        s.lbm_init_droplet(4.0)
+        best = 1e9
+        for _ in range(30):
+            torch.cuda.synchronize()
+            t = time.perf_counter()
+            s.lbm_step(2)
+            best = min(best, time.perf_counter() - t)
+        us.append(1e6 * best)
+        s.close()
+    assert us[1] < 3 * us[0] + 20, us
