@@ -73,7 +73,11 @@ extern "C" {
 
 /* storage precision */
 #define LBM_FP64 0    /* populations, density and all arithmetic in FP64 */
-#define LBM_FP32DEV 1 /* populations stored in FP32 as f_i - w_i rho_ref, density as rho - rho_ref */
+/* populations stored in FP32 as f_i - w_i rho_ref, density as rho - rho_ref.  Sums
+ * over a node's populations, and over the neighbours of a wall node (Eq. A.1), are
+ * FP32 ones, with walls compensated ones, which round as sums in FP64; sums over the
+ * lattice (the mass) are FP64 beyond one thread's few nodes */
+#define LBM_FP32DEV 1
 
 /*
  * Simulation parameters.
@@ -90,12 +94,16 @@ extern "C" {
  *  tau       BGK relaxation time (> 0.5)
  *  scheme    LBM_EFDS2 .. LBM_E8
  *  precision LBM_FP64 or LBM_FP32DEV
- *  mu_fp64   FP32DEV only: evaluate the EOS chemical potential in FP64
+ *  mu_fp64   FP32DEV only: evaluate the EOS chemical potential beyond FP32
  *            (slower on GB300, whose FP64 rate is a small fraction of FP32).
- *            D3Q19 with LBM_EFDS2/4/6: k^2 psi'(rho) in FP64 from rho_ref +
- *            the float deviation, the mu field then rounded to float for the
- *            stencils (3.5x the step time at 256^3); elsewhere mu and its
- *            gradient stay in FP64 in the kernels
+ *            D3Q19 with LBM_EFDS2/4/6: mu from rho_ref + the float deviation,
+ *            rounded once to the float mu field that the stencils read.
+ *            Carnahan-Starling evaluates it as sums of two floats (about
+ *            2^-45 of its terms): the float that FP64 gives but for about one
+ *            node in 10^5 or fewer, where the value lies next to the middle
+ *            of two floats (1.3x the step time at 256^3); the other equations
+ *            of state, and densities outside (1e-30, 1e30), in FP64.
+ *            Elsewhere mu and its gradient stay in FP64 in the kernels
  *  rho_ref   FP32DEV only: reference density of the stored deviations;
  *            <= 0 selects the Maxwell gas density at Tr
  *  collision LBM_BGK, or LBM_MRT (D2Q9; LBM_ENOTSUP on D3Q19)
