@@ -77,8 +77,8 @@ constexpr int MUX = 32, MUY = 8, MUZ = 8, MUT = MUX * MUY;
 // M64: the EOS chemical potential k^2 psi'(rho) from rho = rho_ref + deviation
 // beyond FP32, the Laplacian (FP32 as with M64 off) subtracted, the sum rounded
 // once to the float mu field: Carnahan-Starling in double-float, which rounds
-// to the float FP64 gives but for about one node in a million, on the FP32 pipe
-// (256^3, k_mom_mu: 1.74 -> 0.129 ms); the other equations of state, and densities outside
+// to the float FP64 gives but for fewer than one node in 10^5, on the FP32 pipe
+// (256^3, k_mom_mu: 1.74 -> 0.131 ms); the other equations of state, and densities outside
 // the double-float's range, in FP64.
 template <bool M64>
 struct MuConst {
